@@ -36,21 +36,35 @@ __device__ __forceinline__ uint64_t smem_desc_strided(uint32_t addr, uint32_t lb
          ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | (1ull << 46);
 }
 
-// The same layout for 4-byte elements (TF32): a core-matrix row holds 4 of them.
-__host__ __device__ __forceinline__ uint32_t cm_offset4(int row, int k, int kc) {
-  return (uint32_t)(((row >> 3) * kc + (k >> 2)) * 128 + (row & 7) * 16 + (k & 3) * 4);
-}
-
-// Instruction descriptor of kind::tf32 (A and B read as TF32 from FP32, both
-// K-major) with an FP32 accumulator: formats 2 at bits 7 and 10.
-__host__ __device__ constexpr uint32_t idesc_tf32(int m, int n) {
-  return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
-}
-
 // Instruction descriptor of kind::f16 with BF16 A and B (both K-major) and an
 // FP32 accumulator: N/8 at bit 17, M/16 at bit 24.
 __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
+}
+
+// The same with both operands MN-major (bits 15 and 16): for rows of an operand
+// (its M or N index) contiguous in shared memory.  Without swizzle element (mn, k)
+// then sits at (mn / 8) * SBO + (k / 8) * LBO + (k % 8) * 16 + (mn % 8) * 2 bytes.
+__host__ __device__ constexpr uint32_t idesc_bf16_mn(int m, int n) { return idesc_bf16(m, n) | (1u << 15) | (1u << 16); }
+
+// An FP32 value as two BF16 values (hi, lo) that add up to it after its lowest 13
+// mantissa bits are cut -- what kind::tf32 reads of it -- and as three that add up
+// to all of it.  Infinities and NaN go to hi alone.
+__device__ __forceinline__ void split_tf32(float g, uint16_t& hi, uint16_t& lo) {
+  const uint32_t t = __float_as_uint(g) & 0xffffe000u, h = t & 0xffff0000u;
+  const float r = __uint_as_float(t) - __uint_as_float(h);
+  hi = (uint16_t)(h >> 16);
+  lo = (t & 0x7f800000u) == 0x7f800000u ? (uint16_t)0 : (uint16_t)(__float_as_uint(r) >> 16);
+}
+__device__ __forceinline__ void split_fp32(float g, uint16_t& hi, uint16_t& mid, uint16_t& lo) {
+  const uint32_t t = __float_as_uint(g), h = t & 0xffff0000u;
+  const bool finite = (t & 0x7f800000u) != 0x7f800000u;
+  const float r1 = finite ? g - __uint_as_float(h) : 0.f;
+  const uint32_t m = __float_as_uint(r1) & 0xffff0000u;
+  const float r2 = r1 - __uint_as_float(m);
+  hi = (uint16_t)((h | (finite || !(t & 0xffffu) ? 0u : 0x10000u)) >> 16);  // a NaN stays one
+  mid = (uint16_t)(m >> 16);
+  lo = (uint16_t)(__float_as_uint(r2) >> 16);
 }
 
 // One warp: allocate ncols (power of two >= 32) TMEM columns; base written to *slot.
@@ -73,15 +87,6 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint6
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
-}
-
-// D[tmem] (+)= A * B^T, M x N x 8 with TF32 operands, one thread.
-__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                         uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
       "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
 }
 

@@ -65,12 +65,11 @@ constexpr int kW3 = kB2 + kCh, kB3 = kW3 + kCh * kCh * 9, kWf1 = kB3 + kCh, kBf1
 constexpr int kWf2 = kBf1 + kHid, kBf2 = kWf2 + kHid, kNParams = kBf2 + 1;
 static_assert(kNParams == 187137, "parameter layout");
 
-constexpr int kBackBlocks = 256;      // blocks (and partial sums) of the conv backward kernels
+constexpr int kBackBlocks = 304;      // blocks (and partial sums) of the conv backward kernels: two per SM
 constexpr int kPartialStride = kCh * kCh * 9 + kCh;  // >= parts * weights + biases of any layer
 constexpr uint32_t kFc1Slices = 8;                   // stamp slices of the fc1 weight gradient
 static_assert((size_t)kFc1Slices * (kHid * kF + kHid) <= (size_t)kBackBlocks * kPartialStride,
               "fc1 slices fit the partial buffer");
-static_assert(kPartialStride >= 3 * kCh * kQ * 9 + kCh, "partial stride");
 
 __device__ __forceinline__ float bf(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 __device__ __forceinline__ float ld(const __nv_bfloat16* p) { return __bfloat162float(*p); }
@@ -560,240 +559,383 @@ __global__ void __launch_bounds__(256) k_fc1_dx(const float* __restrict__ g4,
   }
 }
 
-// ---- conv1 weight gradient (CUDA cores) -----------------------------------------
-
-constexpr int kBackThreads = 256;
-
-// The first layer (C = 9 input channels of HI x HI, output 32 x HO x HO): gin
-// is the masked delta of its output [n][32][HO*HO], its input the stamps (no
-// input delta is needed).  Block partial (at partial + blockIdx.x *
-// kPartialStride): [parts][32][C][9] weight sums, then [32] bias sums.
-template <int C, int HI>
-__global__ void __launch_bounds__(kBackThreads) k_conv1_dw(const float* __restrict__ gin,
-                                                           const uint16_t* __restrict__ stamps,
-                                                           const uint32_t* __restrict__ idx, uint32_t n,
-                                                           float* __restrict__ partial) {
-  constexpr int HO = HI - 2, P = HO * HO, Q = HI * HI;
-  constexpr int PARTS = kBackThreads / (8 * C);  // 3 for C = 9
-  static_assert(PARTS >= 1, "too many channels");
-  extern __shared__ __align__(16) float sm[];
-  float* g_s = sm;             // [32][P]
-  float* a_s = g_s + kCh * P;  // [C][Q]
-  const int t = threadIdx.x;
-  // weight-gradient ownership: (4 output channels, 1 input channel, 1 pixel part)
-  const int c_own = t % C, oq = (t / C) % 8, part = t / (8 * C);
-  const bool owner = part < PARTS;
-  float acc[4][9];
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-#pragma unroll
-    for (int tap = 0; tap < 9; ++tap) acc[j][tap] = 0.f;
-  float accb = 0.f;
-  for (uint32_t b = blockIdx.x; b < n; b += gridDim.x) {
-    __syncthreads();
-    for (int i = t; i < kCh * P; i += blockDim.x) g_s[i] = gin[(size_t)b * kCh * P + i];
-    for (int i = t; i < C * Q; i += blockDim.x)
-      a_s[i] = bf((float)stamps[(size_t)(idx ? idx[b] : b) * C * Q + i] * 0.0625f);
-    __syncthreads();
-    if (owner) {
-      for (int p = part; p < P; p += PARTS) {
-        const int y = p / HO, x = p - y * HO;
-        float g[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) g[j] = g_s[(oq * 4 + j) * P + p];
-        const float* ap = a_s + c_own * Q + y * HI + x;
-#pragma unroll
-        for (int tap = 0; tap < 9; ++tap) {
-          const float a = ap[(tap / 3) * HI + tap % 3];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[j][tap] = fmaf(g[j], a, acc[j][tap]);
-        }
-      }
-    }
-    if (t < kCh) {
-      for (int p = 0; p < P; ++p) accb += g_s[t * P + p];
-    }
-  }
-  float* out = partial + (size_t)blockIdx.x * kPartialStride;
-  if (owner) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int tap = 0; tap < 9; ++tap)
-        out[(size_t)part * kCh * C * 9 + ((oq * 4 + j) * C + c_own) * 9 + tap] = acc[j][tap];
-  }
-  if (t < kCh) out[PARTS * kCh * C * 9 + t] = accb;
-}
-
-// ---- conv backward on the tensor cores (TF32) for the 32-channel layers ------
+// ---- conv backward on the tensor cores -------------------------------------------
 //
-// Per block (a fixed set of stamps, so gradients stay bit-reproducible):
-//   dW[k = (c, tap)][o] += sum_p im2col(a)[k][p] * g[o][p]: M = 288 rows of k
-//     (three 128-row tiles, the last padded), N = 32, K = output pixels in
-//     chunks of 32; accumulated in TMEM across the block's stamps.
-//   dX[q][c] = sum_(o, tap) g[o][q - tap] * w[o][c][tap]: M = input pixels in
-//     128-row tiles, N = 32, K = 288 in chunks of 32; masked by the ReLU of the
-//     layer's input and written per stamp.
-// Operands are FP32 read as TF32 (activations and weights are BF16 values, so
-// exact; deltas round to TF32) in the no-swizzle K-major layout with 4-byte
-// elements; one thread issues the MMAs, completion through an mbarrier with a
-// bounded wait.  Bias gradients stay on the CUDA cores.
-constexpr int kBtThreads = 256;
-constexpr int kBtKCX = 9 * kCh / 4;                 // dX K (o, tap) = 288: 72 core matrices
-constexpr int kBtSmWb = 0;                           // [32 c][288] dX B operand (resident)
-constexpr int kBtSmA = kBtSmWb + kCh * 9 * kCh * 4;  // A chunk: 384 x 32 (dW) or up to 256 x 32 (dX)
-constexpr int kBtSmB = kBtSmA + 384 * 32 * 4;        // dW B chunk: 32 x 32
-constexpr int kBtSmG = kBtSmB + kCh * 32 * 4;        // g [32][P], then a [32][Q], then barrier
-
-// Position i of a 4-byte-element operand with 32 K per row (8 core matrices
-// per row group) in the no-swizzle K-major layout: its row and k, so that
-// cm_offset4(cm_row(i), cm_k(i), 8) == 4 i.
-__device__ __forceinline__ int cm_row(int i) { return (i >> 8) * 8 + ((i >> 2) & 7); }
-__device__ __forceinline__ int cm_k(int i) { return ((i >> 5) & 7) * 4 + (i & 3); }
-
-template <int HI>
-constexpr size_t back_tc_smem() {
-  return (size_t)kBtSmG + (size_t)kCh * (HI - 2) * (HI - 2) * 4 + (size_t)kCh * HI * HI * 4 + 16;
-}
+// Per block (a fixed set of stamps, so gradients stay bit-reproducible), for a
+// 32-channel layer with HI x HI inputs and HO x HO outputs:
+//   dX[q][c] = sum_(tap, o) g[o][q - tap] * w[o][c][tap]
+//   dW[o][c][tap] = sum_p g[o][p] * a[c][p + tap]
+// Both are implicit GEMMs over buffers laid out as in the forward: [8-channel
+// chunk][pixel row][8 channels], rows 16 bytes apart, pixel rows of HI columns.
+//   g sits at row (y + 2) HI + x + 2 with zeros around it, so dX is the forward's
+//   shifted-descriptor convolution with the taps reversed (K-major, M = 128 input
+//   pixels a tile, N = 32 channels c, K = 16 channels o per MMA).
+//   For dW the same buffers are read MN-major (channels contiguous): M = channels o,
+//   N = 32 channels c, K = 16 pixels per MMA; a tap is again a shifted start of a.
+// The deltas enter as two BF16 parts, hi + lo = the value cut to TF32's 11 bits
+// (split_tf32), and weights and activations are BF16 values: products are exact
+// and add up in FP32, as with kind::tf32, but operands need no im2col, whose
+// building on the CUDA cores took nearly all of the time: with it 4096 stamps took
+// 1.205 ms (HI = 13) and 0.804 ms (HI = 11), now 0.135 and 0.101.  hi and lo are 4 chunks each; a copy of both
+// shifted by one pixel follows, so the 128 rows of one dW MMA are (hi, lo) at two
+// neighbouring taps.  TMEM: dW 6 x 32 columns (per dy: taps 0 and 1, then tap 2 whose
+// upper half is not used), dX 32 per tile; 256 in all, two CTAs per SM, so that one
+// CTA's loads and epilogue overlap the other's MMAs.  The next stamp's values are
+// fetched into registers while the MMAs run.  The masked dX goes to gout, bias
+// gradients are FP32 sums of the uncut deltas.
+constexpr int kBcThreads = 512;  // 16 warps: 4 TMEM lane quadrants x 4 eight-channel slices
 
 template <int HI>
-__global__ void __launch_bounds__(kBtThreads, 1) k_conv_back_tc(
+struct ConvBack {
+  static constexpr int C = kCh, HO = HI - 2, P = HO * HO, Q = HI * HI, W = HI;
+  static constexpr int MT = (Q + 127) / 128;               // dX tiles
+  static constexpr int KD = (HO * W + 15) / 16 * 16;       // dW's K: g's pixels in rows of W
+  static constexpr int OFF = 2 * W + 2;                    // row of g's first pixel
+  static constexpr int RG = (MT * 128 + OFF + 7) / 8 * 8;  // rows of g: the last tile's last tap ends here
+  static constexpr int RA = (KD + OFF + 7) / 8 * 8;        // rows of a
+  static constexpr int kSmA = 16 * RG * 16;
+  static constexpr int kSmW = kSmA + 4 * RA * 16;
+  static constexpr int kSmBar = kSmW + 9 * C * C * 2;
+  static constexpr int kSmem = kSmBar + 32;
+  static constexpr int GI = (4 * P + kBcThreads - 1) / kBcThreads;  // (chunk, pixel) items per thread
+  static constexpr int AI = (4 * Q + kBcThreads - 1) / kBcThreads;
+  static_assert(OFF + KD + 1 <= RG && RA >= Q, "dW windows stay inside the buffers");
+  static_assert(32 * 32 * 9 * 4 <= kSmA && 8 * kBcThreads * 4 <= kSmA, "the last sums fit g's buffer");
+  static_assert(2 * kSmem <= 225 * 1024 && kSmA % 128 == 0 && kSmW % 128 == 0, "two CTAs per SM, operand alignment");
+  static_assert(GI == 1, "a thread keeps one (chunk, pixel) of g: its bias sums");
+};
+
+template <int HI>
+__global__ void __launch_bounds__(kBcThreads, 2) k_conv_back_tc(
     const float* __restrict__ gin, const __nv_bfloat16* __restrict__ ain, uint32_t n,
     const __nv_bfloat16* __restrict__ w, float* __restrict__ gout, float* __restrict__ partial,
     uint32_t* __restrict__ status) {
-  constexpr int C = kCh, HO = HI - 2, P = HO * HO, Q = HI * HI;
-  constexpr int NCW = (P + 31) / 32, MQ = (Q + 127) / 128, KC = 8;
-  static_assert(MQ * 128 <= 384, "dX tile fits the A buffer");
+  using L = ConvBack<HI>;
+  constexpr int C = L::C, HO = L::HO, P = L::P, Q = L::Q, W = L::W, RG = L::RG, RA = L::RA;
   extern __shared__ __align__(1024) unsigned char smb[];
-  unsigned char* Wb = smb + kBtSmWb;
-  unsigned char* Ab = smb + kBtSmA;
-  unsigned char* Bb = smb + kBtSmB;
-  float* g_s = reinterpret_cast<float*>(smb + kBtSmG);
-  float* a_s = g_s + C * P;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(a_s + C * Q);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 1);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (warp == 0) tc::tmem_alloc(tslot, 256);  // dW: columns [0, 96), dX: [128, 128 + 32 MQ)
-  if (tid == 0) tc::mbar_init(bar, 1);
-  for (int i = tid; i < C * 9 * C; i += kBtThreads) {  // Wb[c][(o, tap)] = w[o][c][tap]
-    const int c = i / (9 * C), K = i - c * 9 * C, o = K / 9, tap = K - o * 9;
-    *reinterpret_cast<float*>(Wb + tc::cm_offset4(c, K, kBtKCX)) = ld(w + (o * C + c) * 9 + tap);
+  unsigned char* Ab = smb + L::kSmA;
+  unsigned char* Wb = smb + L::kSmW;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smb + L::kSmBar);  // dX done, dW done
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 2);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q4 = warp & 3, h = warp >> 2;
+  if (warp == 0) tc::tmem_alloc(tslot, 256);
+  if (tid == 0) {
+    tc::mbar_init(bar, 1);
+    tc::mbar_init(bar + 1, 1);
   }
-  tc::fence_smem_to_async();
+  for (int i = tid; i < L::kSmW / 16; i += kBcThreads) reinterpret_cast<uint4*>(smb)[i] = make_uint4(0, 0, 0, 0);
+  for (int i = tid; i < 9 * C * C; i += kBcThreads) {  // dX's B operand per tap: B_t[c][o] = w[o][c][t]
+    const int t = i / (C * C), c = (i / C) % C, o = i % C;
+    *reinterpret_cast<__nv_bfloat16*>(Wb + t * C * C * 2 + tc::cm_offset(c, o, 4)) = w[(o * C + c) * 9 + t];
+  }
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = *tslot;
-  const uint32_t a0 = tc::smem_u32(Ab), b0 = tc::smem_u32(Bb), wb0 = tc::smem_u32(Wb);
-  constexpr uint32_t idesc = tc::idesc_tf32(128, 32);
-  uint32_t phase = 0;
-  float accb = 0.f;
-  bool any = false, ok = true;
-  // one chunk of MMAs issued by thread 0, then everyone waits for them
-  auto run = [&](auto issue) -> bool {
+  const uint32_t g0 = tc::smem_u32(smb), a0 = tc::smem_u32(Ab), w0 = tc::smem_u32(Wb);
+  const int g_chunk = tid / P, g_p = tid - g_chunk * P;
+  const bool g_item = tid < 4 * P;
+  const int g_row = L::OFF + (g_p / HO) * W + g_p % HO;
+  float gv[8], accb[8];
+  uint32_t av[L::AI][4];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) gv[j] = accb[j] = 0.f;
+  auto fetch = [&](uint32_t b) {
+    if (b >= n) return;
+    const float* g = gin + (size_t)b * C * P + g_chunk * 8 * P + g_p;
+    if (g_item) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) gv[j] = g[j * P];
+    }
+    const uint16_t* a = reinterpret_cast<const uint16_t*>(ain) + (size_t)b * C * Q;
+#pragma unroll
+    for (int i = 0; i < L::AI; ++i) {
+      const int it = tid + i * kBcThreads, chunk = it / Q, q = it - chunk * Q;
+      if (it < 4 * Q) {
+#pragma unroll
+        for (int j = 0; j < 8; j += 2)
+          av[i][j / 2] = (uint32_t)a[(chunk * 8 + j) * Q + q] | ((uint32_t)a[(chunk * 8 + j + 1) * Q + q] << 16);
+      }
+    }
+  };
+  fetch(blockIdx.x);
+  uint32_t phase = 0, any = 0;
+  bool ok = true;
+  for (uint32_t b = blockIdx.x; b < n; b += gridDim.x) {
+    if (g_item) {
+      uint32_t hi[4], lo[4];
+#pragma unroll
+      for (int j = 0; j < 8; j += 2) {
+        uint16_t h0, l0, h1, l1;
+        tc::split_tf32(gv[j], h0, l0);
+        tc::split_tf32(gv[j + 1], h1, l1);
+        hi[j / 2] = (uint32_t)h0 | ((uint32_t)h1 << 16);
+        lo[j / 2] = (uint32_t)l0 | ((uint32_t)l1 << 16);
+        accb[j] += gv[j];
+        accb[j + 1] += gv[j + 1];
+      }
+      const uint4 vh = make_uint4(hi[0], hi[1], hi[2], hi[3]), vl = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+      uint4* at = reinterpret_cast<uint4*>(smb) + g_chunk * RG + g_row;
+      at[0] = vh;
+      at[4 * RG] = vl;
+      at[8 * RG + 1] = vh;   // the copy one pixel on
+      at[12 * RG + 1] = vl;
+    }
+#pragma unroll
+    for (int i = 0; i < L::AI; ++i) {
+      const int it = tid + i * kBcThreads, chunk = it / Q, q = it - chunk * Q;
+      if (it < 4 * Q)
+        reinterpret_cast<uint4*>(Ab)[chunk * RA + q] = make_uint4(av[i][0], av[i][1], av[i][2], av[i][3]);
+    }
     tc::fence_smem_to_async();
     tc::fence_before_sync();
     __syncthreads();
     if (tid == 0) {
       tc::fence_after_sync();
-      issue();
-      tc::commit(bar);
-    }
-    const bool done = tc::mbar_wait(bar, phase, 1u << 22);
-    phase ^= 1u;
-    return !__syncthreads_or(!done);
-  };
-  for (uint32_t b = blockIdx.x; b < n && ok; b += gridDim.x) {
-    for (int i = tid; i < C * P; i += kBtThreads) g_s[i] = gin[(size_t)b * C * P + i];
-    for (int i = tid; i < C * Q; i += kBtThreads) a_s[i] = ld(ain + (size_t)b * C * Q + i);
-    __syncthreads();
-    if (tid < C)
-      for (int p = 0; p < P; ++p) accb += g_s[tid * P + p];
-    // dW: im2col(a)^T x g over chunks of 32 output pixels
-    for (int ch = 0; ch < NCW && ok; ++ch) {
-      const int p0 = ch * 32;
-      // buffers are filled in memory order (a warp writes one 128-byte core
-      // matrix): element i is (row, k) = cm_row(i), cm_k(i)
-      for (int i = tid; i < 384 * 32; i += kBtThreads) {
-        const int k = cm_row(i), kk = cm_k(i), p = p0 + kk;
-        float v = 0.f;
-        if (k < 9 * C && p < P) {
-          const int c = k / 9, tap = k - c * 9, y = p / HO, x = p - y * HO;
-          v = a_s[c * Q + (y + tap / 3) * HI + x + tap % 3];
-        }
-        reinterpret_cast<float*>(Ab)[i] = v;
-      }
-      for (int i = tid; i < C * 32; i += kBtThreads) {
-        const int o = cm_row(i), p = p0 + cm_k(i);
-        reinterpret_cast<float*>(Bb)[i] = p < P ? g_s[o * P + p] : 0.f;
-      }
-      const uint32_t acc0 = (any || ch > 0) ? 1u : 0u;
-      ok = run([&] {
-        for (int mt = 0; mt < 3; ++mt)
-          for (int ks = 0; ks < 4; ++ks)
-            tc::mma_tf32(tmem + (uint32_t)(mt * 32), tc::smem_desc(a0 + (uint32_t)(mt * 16 * KC * 128 + ks * 256), KC),
-                         tc::smem_desc(b0 + (uint32_t)(ks * 256), KC), idesc, (acc0 | (uint32_t)ks) ? 1u : 0u);
-      });
-    }
-    any = true;
-    // dX: im2col(g) x w over chunks of 32 of (o, tap)
-    for (int ch = 0; ch < 9 && ok; ++ch) {
-      for (int i = tid; i < MQ * 128 * 32; i += kBtThreads) {
-        const int q = cm_row(i), K = ch * 32 + cm_k(i), o = K / 9, tap = K - o * 9;
-        float v = 0.f;
-        if (q < Q) {
-          const int yi = q / HI, xi = q - yi * HI, yo = yi - tap / 3, xo = xi - tap % 3;
-          if (yo >= 0 && yo < HO && xo >= 0 && xo < HO) v = g_s[o * P + yo * HO + xo];
-        }
-        reinterpret_cast<float*>(Ab)[i] = v;
-      }
-      ok = run([&] {
-        for (int mt = 0; mt < MQ; ++mt)
-          for (int ks = 0; ks < 4; ++ks)
-            tc::mma_tf32(tmem + (uint32_t)(128 + mt * 32),
-                         tc::smem_desc(a0 + (uint32_t)(mt * 16 * KC * 128 + ks * 256), KC),
-                         tc::smem_desc(wb0 + (uint32_t)(ch * 8 * 128 + ks * 256), kBtKCX), idesc,
-                         (ch > 0 || ks > 0) ? 1u : 0u);
-      });
-    }
-    if (!ok) break;
-    tc::fence_after_sync();
-    {  // dX epilogue: warp w reads lane quadrant w % 4, columns 16 (w / 4) .. + 15
-      const int q4 = warp & 3, h = warp >> 2;
-      float* go = gout + (size_t)b * C * Q;
-      for (int mt = 0; mt < MQ; ++mt) {
-        float v[16];
-        tc::ld16(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(128 + mt * 32 + h * 16), v);
-        const int q = mt * 128 + q4 * 32 + lane;
-        if (q < Q) {
+      constexpr uint32_t id_x = tc::idesc_bf16(128, 32), id_w = tc::idesc_bf16_mn(128, 32);
+      for (int t = 0; t < L::MT; ++t)
+        for (int tap = 0; tap < 9; ++tap) {
+          const uint32_t shift = (uint32_t)((2 - tap / 3) * W + 2 - tap % 3) + (uint32_t)(t * 128);
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int c = h * 16 + j;
-            go[c * Q + q] = a_s[c * Q + q] > 0.f ? v[j] : 0.f;
+          for (int k = 0; k < 4; ++k)  // hi, channels 0-15 and 16-31, then lo
+            tc::mma_bf16(tmem + 192u + (uint32_t)(t * 32),
+                         tc::smem_desc_strided(g0 + ((uint32_t)(2 * k * RG) + shift) * 16u, (uint32_t)(RG * 16), 128u),
+                         tc::smem_desc(w0 + (uint32_t)(tap * C * C * 2 + 2 * (k & 1) * 128), 4), id_x, (tap | k) != 0);
+        }
+      tc::commit(bar);
+      for (int blk = 0; blk < 6; ++blk) {  // taps (dy, 0) and (dy, 1) for blk = dy; (dy, 2) for blk = 3 + dy
+        const uint32_t shift = (uint32_t)((blk % 3) * W + (blk < 3 ? 0 : 2));
+        for (int k = 0; k < L::KD / 16; ++k)
+          tc::mma_bf16(tmem + (uint32_t)(blk * 32),
+                       tc::smem_desc_strided(g0 + (uint32_t)(L::OFF + 16 * k) * 16u, 128u, (uint32_t)(RG * 16)),
+                       tc::smem_desc_strided(a0 + (shift + (uint32_t)(16 * k)) * 16u, 128u, (uint32_t)(RA * 16)), id_w,
+                       any | (uint32_t)k);
+      }
+      tc::commit(bar + 1);
+    }
+    any = 1;
+    fetch(b + gridDim.x);
+    ok = tc::mbar_wait(bar, phase, 1u << 22);
+    if (__syncthreads_or(!ok)) {
+      ok = false;
+      break;
+    }
+    tc::fence_after_sync();
+    float* go = gout + (size_t)b * C * Q;
+#pragma unroll
+    for (int t = 0; t < L::MT; ++t) {
+      float v[8];
+      tc::ld8(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(192 + t * 32 + h * 8), v);
+      const int q = t * 128 + q4 * 32 + lane;
+      if (q < Q) {  // mask by the input's ReLU
+        const uint4 a = reinterpret_cast<const uint4*>(Ab)[h * RA + q];
+        const uint32_t aw[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const uint32_t bits = (aw[j / 2] >> (16 * (j & 1))) & 0xffffu;
+          go[(h * 8 + j) * Q + q] = bits != 0u && bits < 0x8000u ? v[j] : 0.f;
+        }
+      }
+    }
+    ok = tc::mbar_wait(bar + 1, phase, 1u << 22);
+    phase ^= 1u;
+    tc::fence_before_sync();
+    if (__syncthreads_or(!ok)) {  // the buffers and dX's columns are free for the next stamp
+      ok = false;
+      break;
+    }
+    tc::fence_after_sync();
+  }
+  if (!ok && tid == 0) atomicOr(status, 1u);
+  float* out = partial + (size_t)blockIdx.x * kPartialStride;  // [32 o][C][9], then [32] biases
+  if (ok) {
+    // dW: lanes 0-31 and 32-63 are hi and lo of output channel o at the block's first
+    // tap, 64-95 and 96-127 at its second; both parts are added in shared memory
+    tc::fence_after_sync();
+    float* sum = reinterpret_cast<float*>(smb);
+    for (int part = 0; part < 2; ++part) {
+      if ((q4 & 1) == part) {
+        for (int blk = 0; blk < (q4 < 2 ? 6 : 3); ++blk) {
+          float v[8];
+          tc::ld8(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(blk * 32 + h * 8), v);
+          const int tap = (blk % 3) * 3 + (blk < 3 ? q4 / 2 : 2);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            float* s = sum + (lane * C + h * 8 + j) * 9 + tap;
+            *s = (part ? *s : 0.f) + v[j];
           }
         }
       }
+      __syncthreads();
     }
-    tc::fence_before_sync();
-    __syncthreads();  // g_s, a_s and the dX columns are free for the next stamp
-  }
-  if (!ok && tid == 0) atomicOr(status, 1u);
-  tc::fence_after_sync();
-  float* out = partial + (size_t)blockIdx.x * kPartialStride;  // [32 o][C][9], then [32] biases
-  if (ok) {
-    const int q4 = warp & 3, h = warp >> 2;
-    for (int mt = 0; mt < 3; ++mt) {
-      float v[16];
-      tc::ld16(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(mt * 32 + h * 16), v);
-      const int k = mt * 128 + q4 * 32 + lane;
-      if (k < 9 * C) {
-        const int c = k / 9, tap = k - c * 9;
+    for (int i = tid; i < C * C * 9; i += kBcThreads) out[i] = any ? sum[i] : 0.f;
+    __syncthreads();
+    // biases: 16 threads per channel add its pixels' sums
 #pragma unroll
-        for (int j = 0; j < 16; ++j) out[((h * 16 + j) * C + c) * 9 + tap] = any ? v[j] : 0.f;
+    for (int j = 0; j < 8; ++j) sum[j * kBcThreads + tid] = accb[j];
+    __syncthreads();
+    const int o = tid >> 4;
+    float s = 0.f;
+    for (int p = tid & 15; p < P; p += 16) s += sum[(o & 7) * kBcThreads + (o >> 3) * P + p];
+#pragma unroll
+    for (int x = 8; x > 0; x >>= 1) s += __shfl_xor_sync(0xffffffffu, s, x);
+    if ((tid & 15) == 0) out[C * C * 9 + o] = s;
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == 0) tc::tmem_free(tmem, 256);
+}
+
+// ---- conv1 weight gradient ---------------------------------------------------------
+//
+// dW[o][c][tap] = sum_p g1[o][p] x[c][p + tap] over 9 input channels of 15 x 15
+// counts, per block as above.  The deltas enter in full, as three BF16 parts (hi,
+// mid, lo: split_fp32), the inputs are BF16 values, so every product is exact and
+// adds up in FP32 as on the CUDA cores before (4096 stamps: 0.203 ms, now 0.098).  Both
+// operands MN-major: M = (3 parts x 32 channels o, 32 rows unused), N = 16 (9 channels
+// c), K = 16 pixels of rows of 15 columns; a tap is a shifted start of x.
+constexpr int kC1K = 208;                    // 13 rows of 15 columns, padded to 16
+constexpr int kC1RG = kC1K, kC1RX = 240;     // rows: x to 207 + 2 * 15 + 2
+constexpr int kC1SmX = 16 * kC1RG * 16;      // chunks 12..15 of g's buffer are never written
+constexpr int kC1SmBar = kC1SmX + 2 * kC1RX * 16;
+constexpr int kC1Smem = kC1SmBar + 16;
+constexpr int kC1Items = (4 * kH1 * kH1 + kBcThreads - 1) / kBcThreads;  // (chunk, pixel) items per thread
+static_assert(kC1RX >= kC1K + 2 * kS + 2 && kC1RX >= kS * kS && 2 * kC1Smem <= 225 * 1024, "conv1 windows");
+static_assert(kCh * kQ * 9 * 4 <= kC1SmX && 2 * 8 * kBcThreads * 4 <= kC1SmX, "the last sums fit g's buffer");
+
+__global__ void __launch_bounds__(kBcThreads, 2) k_conv1_dw_tc(const float* __restrict__ gin,
+                                                               const uint16_t* __restrict__ stamps,
+                                                               const uint32_t* __restrict__ idx, uint32_t n,
+                                                               float* __restrict__ partial,
+                                                               uint32_t* __restrict__ status) {
+  constexpr int C = kCh, P = kH1 * kH1, Q = kS * kS;
+  extern __shared__ __align__(1024) unsigned char smb[];
+  uint16_t* xs = reinterpret_cast<uint16_t*>(smb + kC1SmX);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smb + kC1SmBar);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q4 = warp & 3, h = warp >> 2;
+  if (warp == 0) tc::tmem_alloc(tslot, 256);  // 9 taps x 16 columns
+  if (tid == 0) tc::mbar_init(bar, 1);
+  for (int i = tid; i < kC1SmBar / 16; i += kBcThreads) reinterpret_cast<uint4*>(smb)[i] = make_uint4(0, 0, 0, 0);
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tmem = *tslot, g0 = tc::smem_u32(smb), x0 = tc::smem_u32(smb + kC1SmX);
+  constexpr int kPer = (kQ * Q + kBcThreads - 1) / kBcThreads;
+  float gv[kC1Items][8], accb[kC1Items][8];
+  uint16_t xv[kPer];
+#pragma unroll
+  for (int i = 0; i < kC1Items; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) gv[i][j] = accb[i][j] = 0.f;
+  auto fetch = [&](uint32_t b) {
+    if (b >= n) return;
+#pragma unroll
+    for (int i = 0; i < kC1Items; ++i) {
+      const int it = tid + i * kBcThreads, chunk = it / P, p = it - chunk * P;
+      if (it < 4 * P) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) gv[i][j] = gin[(size_t)b * C * P + (chunk * 8 + j) * P + p];
       }
     }
+    const uint16_t* st = stamps + (size_t)(idx ? idx[b] : b) * kQ * Q;
+#pragma unroll
+    for (int r = 0; r < kPer; ++r) {
+      const int i = tid + r * kBcThreads;
+      xv[r] = i < kQ * Q ? st[i] : (uint16_t)0;
+    }
+  };
+  fetch(blockIdx.x);
+  uint32_t phase = 0, any = 0;
+  bool ok = true;
+  for (uint32_t b = blockIdx.x; b < n; b += gridDim.x) {
+#pragma unroll
+    for (int i = 0; i < kC1Items; ++i) {
+      const int it = tid + i * kBcThreads, chunk = it / P, p = it - chunk * P;
+      if (it < 4 * P) {
+        uint32_t part[3][4];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          uint16_t v[3];
+          tc::split_fp32(gv[i][j], v[0], v[1], v[2]);
+#pragma unroll
+          for (int k = 0; k < 3; ++k)
+            part[k][j / 2] = (j & 1) ? part[k][j / 2] | ((uint32_t)v[k] << 16) : (uint32_t)v[k];
+          accb[i][j] += gv[i][j];
+        }
+        uint4* at = reinterpret_cast<uint4*>(smb) + chunk * kC1RG + (p / kH1) * kS + p % kH1;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) at[4 * k * kC1RG] = make_uint4(part[k][0], part[k][1], part[k][2], part[k][3]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < kPer; ++r) {
+      const int i = tid + r * kBcThreads;
+      if (i < kQ * Q) {
+        const int c = i / Q, p = i - c * Q;
+        xs[((c >> 3) * kC1RX + p) * 8 + (c & 7)] = __bfloat16_as_ushort(__float2bfloat16_rn((float)xv[r] * 0.0625f));
+      }
+    }
+    tc::fence_smem_to_async();
+    tc::fence_before_sync();
+    __syncthreads();
+    if (tid == 0) {
+      tc::fence_after_sync();
+      constexpr uint32_t id = tc::idesc_bf16_mn(128, 16);
+      for (int tap = 0; tap < 9; ++tap)
+        for (int k = 0; k < kC1K / 16; ++k)
+          tc::mma_bf16(tmem + (uint32_t)(tap * 16),
+                       tc::smem_desc_strided(g0 + (uint32_t)(16 * k) * 16u, 128u, (uint32_t)(kC1RG * 16)),
+                       tc::smem_desc_strided(x0 + (uint32_t)((tap / 3) * kS + tap % 3 + 16 * k) * 16u, 128u,
+                                             (uint32_t)(kC1RX * 16)),
+                       id, any | (uint32_t)k);
+      tc::commit(bar);
+    }
+    any = 1;
+    fetch(b + gridDim.x);
+    ok = tc::mbar_wait(bar, phase, 1u << 22);
+    phase ^= 1u;
+    if (__syncthreads_or(!ok)) {
+      ok = false;
+      break;
+    }
   }
-  if (tid < C) out[C * C * 9 + tid] = accb;
+  if (!ok && tid == 0) atomicOr(status, 1u);
+  float* out = partial + (size_t)blockIdx.x * kPartialStride;  // [32 o][9 c][9], then [32] biases
+  if (ok) {
+    tc::fence_after_sync();
+    float* sum = reinterpret_cast<float*>(smb);
+    for (int part = 0; part < 3; ++part) {  // lanes 32 part + o
+      if (q4 == part && h < 2) {
+        for (int tap = 0; tap < 9; ++tap) {
+          float v[8];
+          tc::ld8(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(tap * 16 + h * 8), v);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const int c = h * 8 + j;
+            if (c < kQ) {
+              float* s = sum + (lane * kQ + c) * 9 + tap;
+              *s = (part ? *s : 0.f) + v[j];
+            }
+          }
+        }
+      }
+      __syncthreads();
+    }
+    for (int i = tid; i < C * kQ * 9; i += kBcThreads) out[i] = sum[i];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kC1Items; ++i)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) sum[j * (kC1Items * kBcThreads) + tid + i * kBcThreads] = accb[i][j];
+    __syncthreads();
+    const int o = tid >> 4;
+    float s = 0.f;
+    for (int p = tid & 15; p < P; p += 16) s += sum[(o & 7) * (kC1Items * kBcThreads) + (o >> 3) * P + p];
+#pragma unroll
+    for (int x = 8; x > 0; x >>= 1) s += __shfl_xor_sync(0xffffffffu, s, x);
+    if ((tid & 15) == 0) out[C * kQ * 9 + o] = s;
+  }
   tc::fence_before_sync();
   __syncthreads();
   if (warp == 0) tc::tmem_free(tmem, 256);
@@ -847,11 +989,6 @@ __global__ void k_adam(float* __restrict__ master, float* __restrict__ m, float*
 
 // ---- host side -----------------------------------------------------------------
 
-template <int C, int HI>
-constexpr size_t conv1_dw_smem() {
-  return sizeof(float) * ((size_t)kCh * (HI - 2) * (HI - 2) + (size_t)C * HI * HI);
-}
-
 cudaError_t set_attrs() {
   static bool done = false;
   if (done) return cudaSuccess;
@@ -860,13 +997,12 @@ cudaError_t set_attrs() {
     e = cudaFuncSetAttribute(k_fc_fwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kFcTcSmem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_conv_back_tc<kH2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)back_tc_smem<kH2>());
+                             ConvBack<kH2>::kSmem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_conv_back_tc<kH1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)back_tc_smem<kH1>());
+                             ConvBack<kH1>::kSmem);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_conv1_dw<kQ, kS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)conv1_dw_smem<kQ, kS>());
+    e = cudaFuncSetAttribute(k_conv1_dw_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kC1Smem);
   if (e == cudaSuccess) done = true;
   return e;
 }
@@ -913,17 +1049,17 @@ cudaError_t gradients(sas_vet* vt, const uint16_t* stamps, const float* labels, 
   }
   k_fc1_dx<<<dim3((kF + 63) / 64, (n + 31) / 32), 256, 0, s>>>(vt->g4, vt->wb, vt->a3, n, vt->g3);
   const int nb = (int)std::min<uint32_t>(n, kBackBlocks);
-  k_conv_back_tc<kH2><<<nb, kBtThreads, back_tc_smem<kH2>(), s>>>(vt->g3, vt->a2, n, vt->wb + kW3, vt->g2,
+  k_conv_back_tc<kH2><<<nb, kBcThreads, ConvBack<kH2>::kSmem, s>>>(vt->g3, vt->a2, n, vt->wb + kW3, vt->g2,
                                                                    vt->partial, vt->status);
   k_reduce_partials<<<(kCh * kCh * 9 + kCh + 7) / 8, 256, 0, s>>>(vt->partial, nb, 1, kCh * kCh * 9,
                                                                       grad, kW3, kB3);
-  k_conv_back_tc<kH1><<<nb, kBtThreads, back_tc_smem<kH1>(), s>>>(vt->g2, vt->a1, n, vt->wb + kW2, vt->g1,
+  k_conv_back_tc<kH1><<<nb, kBcThreads, ConvBack<kH1>::kSmem, s>>>(vt->g2, vt->a1, n, vt->wb + kW2, vt->g1,
                                                                    vt->partial, vt->status);
   k_reduce_partials<<<(kCh * kCh * 9 + kCh + 7) / 8, 256, 0, s>>>(vt->partial, nb, 1, kCh * kCh * 9,
                                                                       grad, kW2, kB2);
-  k_conv1_dw<kQ, kS><<<nb, kBackThreads, conv1_dw_smem<kQ, kS>(), s>>>(vt->g1, stamps, idx, n, vt->partial);
+  k_conv1_dw_tc<<<nb, kBcThreads, kC1Smem, s>>>(vt->g1, stamps, idx, n, vt->partial, vt->status);
   k_reduce_partials<<<(kCh * kQ * 9 + kCh + 7) / 8, 256, 0, s>>>(
-      vt->partial, nb, kBackThreads / (8 * kQ), kCh * kQ * 9, grad, kW1, kB1);
+      vt->partial, nb, 1, kCh * kQ * 9, grad, kW1, kB1);
   note_launch(10);
   return cudaGetLastError();
 }

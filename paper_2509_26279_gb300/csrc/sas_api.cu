@@ -173,8 +173,10 @@ namespace {
 // The search (Sec. 2.1 steps 1-3); with weights (one uint8 per detection, in
 // host or device memory like the catalog) cells are scored by the sum over
 // epochs of their largest weight and n_min is the score threshold.
+// windows: the window search (sas_hier.cu) may be used; it is run again without
+// when a field turns out not to fit it.
 int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weights, uint32_t n_min,
-               const sas_opts* opts, void* stream, sas_result** out) {
+               const sas_opts* opts, void* stream, sas_result** out, bool windows = true) {
   if (!grid || !cat || !out) return fail(SAS_ERR_ARG, "null argument");
   const Tracer tr;
   const sas_grid_desc& d = grid->d;
@@ -230,31 +232,52 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
   }
 
   res->weighted = weights != nullptr;
+  // The largest weight sizes the super-bins and the mean one the windows.
+  double mean_weight = 0;
+  int sb_auto = 0;
   if (weights && o.superbin == 0) {
-    // the super-bin heuristic models unit increments: give it the distinct-epoch
-    // count that a score of n_min needs at the largest weight
-    uint32_t wmax = 0;
+    unsigned long long st[2] = {0, 0};
     if (cat->on_device) {
-      std::vector<uint8_t> hw(n);
-      ce = cudaMemcpy(hw.data(), weights, n, cudaMemcpyDeviceToHost);
+      unsigned long long* d_st = nullptr;
+      ce = cudaMallocAsync((void**)&d_st, 16, s);
+      if (ce == cudaSuccess) {
+        ce = launch_weight_stats(weights, n, d_st, s);
+        if (ce == cudaSuccess) ce = cudaMemcpyAsync(st, d_st, 16, cudaMemcpyDeviceToHost, s);
+        if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
+        cudaFreeAsync(d_st, s);
+      }
       if (ce != cudaSuccess) {
         delete res;
-        return cuda_fail(ce, "copy weights");
+        return cuda_fail(ce, "weights");
       }
-      for (uint8_t v : hw) wmax = std::max<uint32_t>(wmax, v);
     } else {
-      for (uint64_t i = 0; i < n; ++i) wmax = std::max<uint32_t>(wmax, weights[i]);
+      for (uint64_t i = 0; i < n; ++i) {
+        st[0] = std::max<unsigned long long>(st[0], weights[i]);
+        st[1] += weights[i];
+      }
     }
-    o.superbin = (uint32_t)choose_superbin(d, n, (n_min + std::max(wmax, 1u) - 1) / std::max(wmax, 1u), v_end - v_begin);
+    const uint32_t wmax = std::max((uint32_t)st[0], 1u);
+    mean_weight = std::max((double)st[1] / (double)n, 0.01);
+    // the super-bin heuristic models unit increments: give it the distinct-epoch
+    // count that a score of n_min needs at the largest weight
+    sb_auto = choose_superbin(d, n, (n_min + wmax - 1) / wmax, v_end - v_begin);
   }
+  sas_opts op = o;  // with the super-bin side that the weights ask for
+  if (sb_auto) op.superbin = (uint32_t)sb_auto;
 
   FieldPlan plan;
-  if (int rc = plan_field(d, n, E, cat->t, tph, n_min, v_begin, v_end, o, di, &plan)) {
+  if (int rc = plan_field(d, n, E, cat->t, tph, n_min, v_begin, v_end, op, di, &plan)) {
     delete res;
     return rc;
   }
-  const CoarseGeom& cg = plan.cg;
-  const uint64_t nb = plan.nb;
+  // A caller that sets tile sizes gets the one-level kernel with those tiles.
+  WindowPlan wplan;
+  const bool use_win = windows && n_low == n_min && !o.peaks_only && !o.tile_kx && !o.tile_ky && !o.tile_bx &&
+                       !o.tile_by && !o.counter_bits && !o.coarse_bins && !o.superbin && !o.velocity_block &&
+                       plan_windows(d, n, n_min, mean_weight, v_begin, v_end, di, plan, &wplan);
+  bool without = false;  // the window search gave up: run again without it
+  const CoarseGeom& cg = use_win ? wplan.cg : plan.cg;
+  const uint64_t nb = use_win ? wplan.nb : plan.nb;
   const SearchGeom& g = plan.g;
   tr.mark("planned");
 
@@ -291,7 +314,7 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
     Det* d_dets = nullptr;
     int32_t *d_sxt = nullptr, *d_syt = nullptr;
     uint32_t* d_small = nullptr;  // [0] flags [1] n_emit [2] n_valid
-    unsigned long long* d_small64 = nullptr;  // [0] pairs [1] tile counter [2] raw total
+    unsigned long long* d_small64 = nullptr;  // [0] pairs [1] tile counter [2] raw total [3] balance [4] level-1 pairs
     Emit* d_emits = nullptr;
     Key* d_keys = nullptr;
     uint32_t* d_raw = nullptr;
@@ -306,6 +329,8 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
     uint32_t n_out = 0;
     unsigned long long n_ids = 0;
     StackArgs sa{};
+    WindowArgs wa{};
+    uint64_t n_keys = 0;
 
     if (!cat->on_device) {
       CK(sc.alloc(&hx, n), "alloc x");
@@ -348,11 +373,11 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
     res->g = g;
     res->cg = cg;
     CK(sc.alloc(&d_small, 4), "alloc counters");
-    CK(sc.alloc(&d_small64, 4), "alloc counters64");
+    CK(sc.alloc(&d_small64, 5), "alloc counters64");
     CK(cudaMemsetAsync(d_ecount, 0, E * 4, s), "memset");
     CK(cudaMemsetAsync(d_bcount, 0, (nb + 1) * 4, s), "memset");
     CK(cudaMemsetAsync(d_small, 0, 16, s), "memset");
-    CK(cudaMemsetAsync(d_small64, 0, 32, s), "memset");
+    CK(cudaMemsetAsync(d_small64, 0, 40, s), "memset");
     tr.mark("allocated");
 
     // a1-a3: ingest and validate, bucket, reference epoch, shift tables
@@ -364,9 +389,96 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
     CK(launch_shift_tables(g, d_dt, d_ecount, d_sxt, d_syt, &d_small[0], s), "shift tables");
     tr.mark("prep launched");
 
+    if (use_win) {  // a4-a7 in two levels: windows of groups of velocities, then their bins
+      const TileCfg& tc = wplan.tc;
+      const SearchGeom& c = wplan.g;
+      const uint32_t list_cap = std::max(wplan.list_cap, hint + hint / 4);
+      uint32_t key_cap = 1u << 17;
+      CK(sc.alloc(&d_emits, list_cap), "alloc windows");
+      CK(sc.alloc(&d_keys, key_cap), "alloc keys");
+      wa.gx = wplan.gx;
+      wa.gy = wplan.gy;
+      wa.win = wplan.win;
+      wa.unit = wplan.unit;
+      wa.g = g;
+      wa.cgm = c;
+      wa.cg = cg;
+      wa.dets = d_dets;
+      wa.boff = d_boff;
+      wa.ecount = d_ecount;
+      wa.dt = d_dt;
+      wa.sxt = d_sxt;
+      wa.syt = d_syt;
+      CK(sc.alloc(&wa.sXt, (size_t)c.nvx * E), "alloc group shifts");
+      CK(sc.alloc(&wa.sYt, (size_t)c.nvy * E), "alloc group shifts");
+      CK(sc.alloc(&wa.mx, d.nvx), "alloc shift bounds");
+      CK(sc.alloc(&wa.my, d.nvy), "alloc shift bounds");
+      if (wplan.masked) {
+        CK(sc.alloc(&wa.vact, (size_t)c.nvx * c.nvy), "alloc active groups");
+        CK(sc.alloc(&wa.vsum, ((size_t)d.nvx + 1) * ((size_t)d.nvy + 1)), "alloc point counts");
+      }
+      wa.wts = d_w;
+      wa.windows = d_emits;
+      wa.n_windows = &d_small[1];
+      wa.list_cap = list_cap;
+      wa.n_min = n_min;
+      wa.n_valid = &d_small[2];
+      wa.raw_total = &d_small64[2];
+      wa.n_pairs = &d_small64[0];
+      wa.flags = &d_small[0];
+      CK(stack_set_smem_attr_windows(tc.kx, tc.ky, tc.cb, tc.smem), "smem attribute");
+      fill_window_args(wplan, n_min, (uint32_t)(v_begin / d.nvx), (uint32_t)((v_end - 1) / d.nvx), &sa);
+      sa.vact = wa.vact;
+      sa.w = d_w;
+      sa.dets = d_dets;
+      sa.boff = d_boff;
+      sa.ecount = d_ecount;
+      sa.sxt = wa.sXt;
+      sa.syt = wa.sYt;
+      sa.emits = d_emits;
+      sa.emit_cap = list_cap;
+      sa.n_emit = &d_small[1];
+      sa.n_pairs = &d_small64[4];
+      sa.balance = &d_small64[3];
+      sa.flags = &d_small[0];
+      sa.tile_counter = &d_small64[1];
+      cudaEventRecord(evs0, s);
+      CK(launch_window_tables(wa, s), "group tables");
+      CK(launch_window_pairs(wa, dx, dy, dep, n, s), "pair count");
+      CK(launch_stack_windows(sa, (int)std::min<uint64_t>((uint64_t)di.sms, std::max<uint64_t>(sa.n_tiles, 1)), s),
+         "window kernel");
+      for (;;) {
+        wa.keys = d_keys;
+        wa.key_cap = key_cap;
+        CK(launch_window_cells(wa, di.sms, s), "window cells");
+        cudaEventRecord(evs1, s);
+        CK(cudaMemcpyAsync(h_small, d_small, 12, cudaMemcpyDeviceToHost, s), "read counters");
+        CK(cudaMemcpyAsync(h_small64, d_small64, 32, cudaMemcpyDeviceToHost, s), "read counters");
+        CK(cudaMemcpyAsync(&h_t0, d_t0, 8, cudaMemcpyDeviceToHost, s), "read t0");
+        CK(cudaStreamSynchronize(s), "stack sync");
+        tr.mark("windows done");
+        if (h_small[0] & kFlagEpoch) { rc = fail(SAS_ERR_RANGE, "an epoch index is >= n_epochs"); goto done; }
+        if (h_small[0] & kFlagPos) { rc = fail(SAS_ERR_RANGE, "a detection has |x| or |y| >= 2^29"); goto done; }
+        if (h_small[0] & kFlagShift) { rc = fail(SAS_ERR_RANGE, "a shift |v*(t-t0)/TPH| >= 2^28"); goto done; }
+        if (h_small[0] & kFlagInternal) { rc = fail(SAS_ERR_INTERNAL, "stack kernel invariant"); goto done; }
+        if ((h_small[0] & (kFlagWindow | kFlagEmitCap)) || h_small64[3] != 0 || h_small[1] > list_cap) {
+          without = true;
+          rc = SAS_ERR_INTERNAL;
+          goto done;
+        }
+        if (h_small[2] <= key_cap) break;
+        key_cap = h_small[2];
+        if (key_cap >= (1u << 30)) { rc = fail(SAS_ERR_OOM, "too many candidate bins; raise n_min"); goto done; }
+        CK(sc.alloc(&d_keys, key_cap), "alloc keys");
+        CK(cudaMemsetAsync(&d_small[2], 0, 4, s), "memset");
+        CK(cudaMemsetAsync(&d_small64[2], 0, 8, s), "memset");
+      }
+      n_keys = key_cap;
+    }
+
     // a4-a6: the stack kernel; reruns (exact) with wider counters if one wrapped
     // or with a longer emission list if it overflowed.
-    for (int attempt = 0;; ++attempt) {
+    for (int attempt = 0; !use_win; ++attempt) {
       const TileCfg& tc = plan.tc;
       CK(sc.alloc(&d_emits, emit_cap), "alloc emissions");
       CK(stack_set_smem_attr(tc.kx, tc.ky, tc.cb, tc.smem), "smem attribute");
@@ -405,7 +517,7 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
       if (attempt >= 4) { rc = fail(SAS_ERR_INTERNAL, "stack kernel did not converge"); goto done; }
       if ((h_small[0] & kFlagCounter) || h_small64[3] != 0) {  // a counter wrapped
         CK(cudaMemsetAsync(&d_small[0], 0, 4, s), "memset");
-        if (int r2 = replan_wider(d, n, n_min, o, di, &plan)) { rc = r2; goto done; }
+        if (int r2 = replan_wider(d, n, n_min, op, di, &plan)) { rc = r2; goto done; }
         continue;
       }
       if (h_small[1] > emit_cap || (h_small[0] & kFlagEmitCap)) {
@@ -422,17 +534,19 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
     {
       const uint32_t n_emit = h_small[1];
       const_cast<sas_grid*>(grid)->emit_hint.store(n_emit, std::memory_order_relaxed);
-      const uint64_t n_keys = (uint64_t)n_emit * plan.tc.s * plan.tc.s;
+      cudaEventRecord(evc0, s);
+      if (!use_win) {
+      n_keys = (uint64_t)n_emit * plan.tc.s * plan.tc.s;
       if (n_keys >= (1ull << 31)) { rc = fail(SAS_ERR_OOM, "too many candidate bins; raise n_min"); goto done; }
       CK(sc.alloc(&d_keys, n_keys), "alloc keys");
       // a5/a7: exact distinct and raw counts of every bin of the emitted super-bins
-      cudaEventRecord(evc0, s);
       CK(launch_cell_count(d_emits, n_emit, plan.tc.s, g, cg, d_dets, d_boff, d_ecount, d_sxt,
                            d_syt, n_min, sa.n_low, d_keys, &d_small[2], &d_small64[2], d_w, s), "cell count");
       CK(cudaMemcpyAsync(&h_small[2], &d_small[2], 4, cudaMemcpyDeviceToHost, s), "read n_valid");
       CK(cudaMemcpyAsync(&h_small64[2], &d_small64[2], 8, cudaMemcpyDeviceToHost, s), "read raw");
       CK(cudaStreamSynchronize(s), "count sync");
       tr.mark("counts done");
+      }
       {  // a8: total order of the valid keys
         const uint32_t n_valid = h_small[2];
         uint32_t n_pad = 1;
@@ -500,7 +614,7 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
       if (p) cudaFreeAsync(p, s);
     cudaStreamSynchronize(s);
     delete res;
-    return rc;
+    return without ? stack_impl(grid, cat, weights, n_min, opts, stream, out, false) : rc;
   }
   *out = res;
   return SAS_OK;

@@ -24,6 +24,7 @@ enum : uint32_t {
   kFlagTimeout = 16u,    // a bounded wait gave up
   kFlagInternal = 32u,   // invariant violated
   kFlagEmitCap = 64u,    // emission list capacity exceeded (rerun with more)
+  kFlagWindow = 128u,    // the window search cannot take this field (rerun without it)
 };
 
 constexpr uint32_t kInvalidBucket = 0xFFFFFFFFu;
@@ -99,6 +100,9 @@ struct StackArgs {
   TileCfg tc;
   uint32_t magic;      // umulhi(X, magic) = X / (s*bin) for 0 <= X < tile extent
   int32_t bin_is_one;  // s*bin == 1: the quotient is X itself
+  int32_t win;         // window search: cells per window side (2 or 3)
+  uint32_t rows_m;     // window search: (tid * rows_m) >> 20 = tid / rows for tid < 1024
+  uint64_t cell_m;     // window search: reciprocal of the bucket cell (div_magic)
   int32_t merge;       // the P columns of a counter word span at most two super-bins
   uint32_t n_min;
   uint32_t n_low;            // the counters' top bit means count >= n_low (n_low == n_min: one threshold)
@@ -108,6 +112,7 @@ struct StackArgs {
   int32_t nst_x, nst_y;      // spatial tiles
   uint64_t n_tiles;          // work units = velocity blocks x spatial tiles
   const Det* dets;
+  const uint8_t* vact;       // window search: lattice points with a searched fine point, or null: all
   const uint8_t* w;          // [n] weight per detection id (weighted stacking), or null: all 1
   const uint32_t* boff;      // [E*ncy*ncx + 1]
   const uint32_t* ecount;    // [E] detections per epoch
@@ -156,6 +161,20 @@ int choose_superbin(const sas_grid_desc& d, uint64_t n, uint32_t n_min, uint64_t
 int plan_field(const sas_grid_desc& d, uint64_t n, uint32_t E, const int64_t* t, int64_t tph,
                uint32_t n_min, uint64_t v_begin, uint64_t v_end, const sas_opts& o,
                const DevInfo& di, FieldPlan* fp);
+// Tiles, staging and buckets for a lattice and grid (see sas_plan.cu).
+struct TilePlan {
+  TileCfg tc;
+  CoarseGeom cg;
+};
+int choose_tiles(const sas_grid_desc& d, uint32_t E, uint64_t n, int64_t dT, int64_t tph, int kx, int ky, int cb, int sb,
+                 const sas_opts& o, const DevInfo& di, int n_rows, const CoarseGeom* fixed_cg, TilePlan* p);
+// The bucket grid that covers every detection which can project into the
+// domain for some lattice velocity (cells grow until their number fits).
+void bucket_grid(const sas_grid_desc& d, uint32_t E, int64_t dT, int64_t tph, CoarseGeom* cg);
+// umulhi(X, magic_for(bin)) == X / bin for 0 <= X <= x_max
+bool magic_exact(int32_t bin, int64_t x_max);
+// log P(Poisson(lam) >= k)
+double log_poisson_tail(double lam, int k);
 // Same plan with counters twice as wide (after a counter wrapped).
 int replan_wider(const sas_grid_desc& d, uint64_t n, uint32_t n_min, const sas_opts& o,
                  const DevInfo& di, FieldPlan* fp);
@@ -175,6 +194,8 @@ cudaError_t launch_scatter(const int32_t* x, const int32_t* y, const uint16_t* e
                            const uint32_t* bucket_of, uint32_t* cursor, Det* dets, cudaStream_t s);
 cudaError_t launch_epoch_setup(uint32_t E, const int64_t* t, const uint32_t* ecount, int64_t* dt,
                                int64_t* t0, cudaStream_t s);
+// Largest and summed weight (uint8) of n detections: out[0], out[1].
+cudaError_t launch_weight_stats(const uint8_t* w, uint64_t n, unsigned long long* out, cudaStream_t s);
 cudaError_t launch_shift_tables(const SearchGeom& g, const int64_t* dt, const uint32_t* ecount,
                                 int32_t* sxt, int32_t* syt, uint32_t* flags, cudaStream_t s);
 // exclusive scan, out[i] = sum(in[0..i)), out has n+1 entries
@@ -204,6 +225,70 @@ cudaError_t launch_stack_multi_peaks(int kx, int ky, int cb, const StackArgs* fa
                                      const unsigned long long* unit_base, int n_fields,
                                      unsigned long long* counter, size_t smem, int grid, cudaStream_t s);
 cudaError_t stack_set_smem_attr_peaks(int kx, int ky, int cb, size_t smem);
+
+// sas_stack_windows.cu: the kernel over blocks of cells
+bool windows_config_supported(int kx, int ky, int cb);
+cudaError_t launch_stack_windows(const StackArgs& a, int grid, cudaStream_t s);
+cudaError_t launch_stack_multi_windows(int kx, int ky, int cb, const StackArgs* fargs,
+                                       const unsigned long long* unit_base, int n_fields,
+                                       unsigned long long* counter, size_t smem, int grid, cudaStream_t s);
+cudaError_t stack_set_smem_attr_windows(int kx, int ky, int cb, size_t smem);
+
+// ---- window search (sas_hier.cu) --------------------------------------------
+
+// The coarser lattice and grid of a window search, and its tiles.
+struct WindowPlan {
+  int gx, gy;          // fine lattice points per group side
+  int win;             // cells per window side
+  int unit;            // mpx of the fine square that a window is searched for
+  SearchGeom g;        // coarse lattice and cells (bin = the cell side in mpx)
+  CoarseGeom cg;       // buckets of the search
+  TileCfg tc;
+  uint64_t nb;         // buckets
+  uint32_t list_cap;   // windows the list has room for
+  bool masked;         // some lattice points are not searched
+};
+// Whether the window search is expected to take fewer instructions than the
+// stack kernel over the fine lattice as planned in fp; fills wp if so.
+// mean_weight: of the detections in weighted stacking (n_min is the score threshold), else 0.
+bool plan_windows(const sas_grid_desc& d, uint64_t n, uint32_t n_min, double mean_weight, uint64_t v_begin,
+                  uint64_t v_end, const DevInfo& di, const FieldPlan& fp, WindowPlan* wp);
+// Level 1's arguments (lattice rows ky_lo..ky_hi of the fine lattice).
+void fill_window_args(const WindowPlan& wp, uint32_t n_min, uint32_t ky_lo, uint32_t ky_hi, StackArgs* sa);
+// Device arrays of a window search, besides those of every search.
+struct WindowArgs {
+  int32_t gx, gy, win, unit;
+  SearchGeom g;          // fine
+  SearchGeom cgm;        // coarse
+  CoarseGeom cg;
+  const Det* dets;
+  const uint32_t* boff;
+  const uint32_t* ecount;
+  const int64_t* dt;
+  const int32_t* sxt;    // fine shifts [nvx][E], [nvy][E]
+  const int32_t* syt;
+  int32_t* sXt;          // coarse shifts
+  int32_t* sYt;
+  int32_t* mx;           // [nvx] least fine - coarse shift over the epochs, and [nvy]
+  int32_t* my;
+  uint8_t* vact;         // coarse lattice points with a searched fine one, or null
+  uint32_t* vsum;        // [(nvy + 1)][(nvx + 1)] searched points below and left, or null: all are searched
+  const uint8_t* wts;    // weight per detection id (weighted stacking), or null
+  const Emit* windows;
+  const uint32_t* n_windows;
+  uint32_t list_cap;
+  uint32_t n_min;
+  Key* keys;
+  uint32_t key_cap;
+  uint32_t* n_valid;
+  unsigned long long* raw_total;
+  unsigned long long* n_pairs;
+  uint32_t* flags;
+};
+cudaError_t launch_window_tables(const WindowArgs& a, cudaStream_t s);
+cudaError_t launch_window_pairs(const WindowArgs& a, const int32_t* x, const int32_t* y, const uint16_t* epoch,
+                                uint64_t n, cudaStream_t s);
+cudaError_t launch_window_cells(const WindowArgs& a, int sms, cudaStream_t s);
 
 // sas_post.cu
 // Appends one key per bin of an emitted super-bin that lies in the domain and

@@ -51,12 +51,6 @@ constexpr int kEmitCap = 256;
 constexpr int kPeakCap = 1024;  // one counter per thread and batch
 constexpr int kMaxEpochChunk = 256;     // staged records carry the epoch in 8 bits
 
-struct Plan {
-  TileCfg tc;
-  CoarseGeom cg;
-  int ky_lo, ky_hi;
-};
-
 // Upper bound of |floor(v*dt/TPH) - floor(v'*dt/TPH)| over dt in [0, dT] for
 // |v - v'| <= dv_span.
 int64_t spread_bound(int64_t dv_span, int64_t dT, int64_t tph) {
@@ -101,7 +95,7 @@ int choose_superbin(const sas_grid_desc& d, uint64_t n, uint32_t n_min, uint64_t
 
 int choose_tiles(const sas_grid_desc& d, uint32_t E, uint64_t n, int64_t dT, int64_t tph, int kx,
                  int ky, int cb, int sb, const sas_opts& o, const DevInfo& di, int n_rows,
-                 const CoarseGeom* fixed_cg, Plan* p) {
+                 const CoarseGeom* fixed_cg, TilePlan* p) {
   if (!stack_config_supported(kx, ky, cb))
     return set_errorf(SAS_ERR_ARG, "unsupported tile (kx=%d, ky=%d, counter_bits=%d)", kx, ky, cb);
   TileCfg tc{};
@@ -226,6 +220,27 @@ int choose_tiles(const sas_grid_desc& d, uint32_t E, uint64_t n, int64_t dT, int
 
 int64_t ceil_div64(int64_t a, int64_t b) { return -floor_div64(-a, b); }
 
+// Every detection that can project into the domain for some lattice velocity and
+// some dt in [0, dT] lies inside the grid.
+void bucket_grid(const sas_grid_desc& d, uint32_t E, int64_t dT, int64_t tph, CoarseGeom* cg) {
+  const int64_t vxa = d.vx0, vxb = (int64_t)d.vx0 + (int64_t)(d.nvx - 1) * d.dvx;
+  const int64_t vya = d.vy0, vyb = (int64_t)d.vy0 + (int64_t)(d.nvy - 1) * d.dvy;
+  auto clampd = [](int64_t v) { return std::max(-kLimDomain, std::min(kLimDomain, v)); };
+  const int64_t sx_lo = clampd(floor_div64(std::min<int64_t>(std::min(vxa, vxb), 0) * dT, tph));
+  const int64_t sx_hi = clampd(ceil_div64(std::max<int64_t>(std::max(vxa, vxb), 0) * dT, tph));
+  const int64_t sy_lo = clampd(floor_div64(std::min<int64_t>(std::min(vya, vyb), 0) * dT, tph));
+  const int64_t sy_hi = clampd(ceil_div64(std::max<int64_t>(std::max(vya, vyb), 0) * dT, tph));
+  for (;;) {
+    cg->gx0 = (int32_t)(d.x_min + sx_lo);
+    cg->gy0 = (int32_t)(d.y_min + sy_lo);
+    cg->ncx = (int32_t)ceil_div64((int64_t)d.nbx * d.bin + (sx_hi - sx_lo) + 1, cg->cell);
+    cg->ncy = (int32_t)ceil_div64((int64_t)d.nby * d.bin + (sy_hi - sy_lo) + 1, cg->cell);
+    if ((uint64_t)E * cg->ncx * cg->ncy <= ((uint64_t)1 << 27)) break;
+    if (cg->cell >= kLimDomain / 2) break;
+    cg->cell *= 2;  // fewer, larger buckets
+  }
+}
+
 int plan_field(const sas_grid_desc& d, uint64_t n, uint32_t E, const int64_t* t, int64_t tph,
                uint32_t n_min, uint64_t v_begin, uint64_t v_end, const sas_opts& o,
                const DevInfo& di, FieldPlan* fp) {
@@ -247,7 +262,7 @@ int plan_field(const sas_grid_desc& d, uint64_t n, uint32_t E, const int64_t* t,
   if (o.superbin > 4) return set_error(SAS_ERR_ARG, "superbin must be 0..4");
   const int sb = o.superbin ? (int)o.superbin : choose_superbin(d, n, n_min, v_end - v_begin);
   const int n_rows = (int)((v_end - 1) / d.nvx - v_begin / d.nvx + 1);
-  Plan plan;
+  TilePlan plan;
   if (int rc = choose_tiles(d, E, n, dT, tph, kx, ky, cb, sb, o, di, n_rows, nullptr, &plan)) {
     // the default 8 x 8 tile can exceed the staged coordinates' shift spread
     // where 8 x 4 does not: fall back to it unless the caller chose the tile
@@ -255,27 +270,10 @@ int plan_field(const sas_grid_desc& d, uint64_t n, uint32_t E, const int64_t* t,
     ky = 4;
     if (int rc2 = choose_tiles(d, E, n, dT, tph, kx, ky, cb, sb, o, di, n_rows, nullptr, &plan)) return rc2;
   }
-  // Bucket grid: every detection that can project into the domain for some
-  // lattice velocity and some dt in [0, dT] lies inside it.
-  const int64_t vxa = d.vx0, vxb = (int64_t)d.vx0 + (int64_t)(d.nvx - 1) * d.dvx;
-  const int64_t vya = d.vy0, vyb = (int64_t)d.vy0 + (int64_t)(d.nvy - 1) * d.dvy;
-  auto clampd = [](int64_t v) { return std::max(-kLimDomain, std::min(kLimDomain, v)); };
-  const int64_t sx_lo = clampd(floor_div64(std::min<int64_t>(std::min(vxa, vxb), 0) * dT, tph));
-  const int64_t sx_hi = clampd(ceil_div64(std::max<int64_t>(std::max(vxa, vxb), 0) * dT, tph));
-  const int64_t sy_lo = clampd(floor_div64(std::min<int64_t>(std::min(vya, vyb), 0) * dT, tph));
-  const int64_t sy_hi = clampd(ceil_div64(std::max<int64_t>(std::max(vya, vyb), 0) * dT, tph));
   CoarseGeom cg = plan.cg;
-  for (;;) {
-    cg.gx0 = (int32_t)(d.x_min + sx_lo);
-    cg.gy0 = (int32_t)(d.y_min + sy_lo);
-    cg.ncx = (int32_t)ceil_div64((int64_t)d.nbx * d.bin + (sx_hi - sx_lo) + 1, cg.cell);
-    cg.ncy = (int32_t)ceil_div64((int64_t)d.nby * d.bin + (sy_hi - sy_lo) + 1, cg.cell);
-    if ((uint64_t)E * cg.ncx * cg.ncy <= ((uint64_t)1 << 27)) break;
-    if (cg.cell >= kLimDomain / 2) break;
-    cg.cell *= 2;  // fewer, larger buckets
-  }
+  bucket_grid(d, E, dT, tph, &cg);
   {  // the bucket cell may have grown: recompute the per-chunk epoch count
-    Plan p2;
+    TilePlan p2;
     if (int rc = choose_tiles(d, E, n, dT, tph, kx, ky, cb, sb, o, di, n_rows, &cg, &p2)) return rc;
     plan.tc = p2.tc;
   }
@@ -307,7 +305,7 @@ int replan_wider(const sas_grid_desc& d, uint64_t n, uint32_t n_min, const sas_o
   (void)n_min;
   if (fp->cb == 32) return set_error(SAS_ERR_INTERNAL, "32-bit counter wrapped");
   const int wider = fp->cb * 2;
-  Plan p2;
+  TilePlan p2;
   if (int rc = choose_tiles(d, fp->g.E, n, fp->dT, fp->g.tph, fp->kx, fp->ky, wider, fp->sb, o, di,
                             fp->n_rows, &fp->cg, &p2))
     return rc;

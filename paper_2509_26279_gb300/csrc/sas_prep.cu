@@ -1,4 +1,5 @@
 // Ingest, bucketing, reference epoch, shift tables and scans (Sec. 2.1 step 1).
+#include <algorithm>
 #include <climits>
 
 #include "sas_internal.cuh"
@@ -220,6 +221,33 @@ cudaError_t scan_impl(const Tin* in, Tout* out, uint64_t n, Tout* scratch, cudaS
   return cudaGetLastError();
 }
 
+// Largest weight and sum of weights, one atomic pair per block.
+__global__ void k_weight_stats(const uint8_t* __restrict__ w, uint64_t n, unsigned long long* __restrict__ out) {
+  uint32_t top = 0;
+  unsigned long long sum = 0;
+  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
+    top = max(top, (uint32_t)w[i]);
+    sum += w[i];
+  }
+  __shared__ unsigned long long s_sum[kPrepThreads / 32];
+  __shared__ uint32_t s_top[kPrepThreads / 32];
+  top = __reduce_max_sync(0xffffffffu, top);
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0) {
+    s_top[threadIdx.x >> 5] = top;
+    s_sum[threadIdx.x >> 5] = sum;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < kPrepThreads / 32; ++i) {
+      top = max(top, s_top[i]);
+      sum += s_sum[i];
+    }
+    atomicMax(&out[0], (unsigned long long)top);
+    atomicAdd(&out[1], sum);
+  }
+}
+
 unsigned grid_for(uint64_t n, int threads) {
   uint64_t b = (n + threads - 1) / threads;
   if (b < 1) b = 1;
@@ -264,6 +292,14 @@ cudaError_t launch_scatter(const int32_t* x, const int32_t* y, const uint16_t* e
 cudaError_t launch_epoch_setup(uint32_t E, const int64_t* t, const uint32_t* ecount, int64_t* dt,
                                int64_t* t0, cudaStream_t s) {
   k_epoch_setup<<<1, 1024, 0, s>>>(E, t, ecount, dt, t0);
+  note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_weight_stats(const uint8_t* w, uint64_t n, unsigned long long* out, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(out, 0, 16, s);
+  if (e != cudaSuccess) return e;
+  k_weight_stats<<<(unsigned)std::min<uint64_t>((n + 8 * kPrepThreads - 1) / (8 * kPrepThreads), 304), kPrepThreads, 0, s>>>(w, n, out);
   note_launch();
   return cudaGetLastError();
 }

@@ -24,7 +24,7 @@ int stack_threads() { return kNT; }
 cudaError_t launch_stack(const StackArgs& a, int grid, cudaStream_t s) {
   if (a.select != kSelectAll) return launch_stack_peaks(a, grid, s);
 #define SAS_LAUNCH(KX, KY, CB) \
-  if (a.tc.kx == KX && a.tc.ky == KY && a.tc.cb == CB) return launch_t<KX, KY, CB, false>(a, grid, s);
+  if (a.tc.kx == KX && a.tc.ky == KY && a.tc.cb == CB) return launch_t<KX, KY, CB, kModePlain>(a, grid, s);
   SAS_STACK_CONFIGS(SAS_LAUNCH)
 #undef SAS_LAUNCH
   return cudaErrorInvalidValue;
@@ -37,7 +37,7 @@ cudaError_t launch_stack_multi(int kx, int ky, int cb, bool peaks, const StackAr
   StackArgs proto{};
 #define SAS_LAUNCH_M(KX, KY, CB)                                                                   \
   if (kx == KX && ky == KY && cb == CB)                                                            \
-    return launch_multi_t<KX, KY, CB, false>(proto, fargs, unit_base, n_fields, counter, smem, grid, s);
+    return launch_multi_t<KX, KY, CB, kModePlain>(proto, fargs, unit_base, n_fields, counter, smem, grid, s);
   SAS_STACK_CONFIGS(SAS_LAUNCH_M)
 #undef SAS_LAUNCH_M
   return cudaErrorInvalidValue;
@@ -45,7 +45,7 @@ cudaError_t launch_stack_multi(int kx, int ky, int cb, bool peaks, const StackAr
 
 cudaError_t stack_set_smem_attr(int kx, int ky, int cb, size_t smem) {
   cudaError_t e = cudaErrorInvalidValue;
-#define SAS_ATTR(KX, KY, CB) if (kx == KX && ky == KY && cb == CB) e = attr_t<KX, KY, CB, false>(smem);
+#define SAS_ATTR(KX, KY, CB) if (kx == KX && ky == KY && cb == CB) e = attr_t<KX, KY, CB, kModePlain>(smem);
   SAS_STACK_CONFIGS(SAS_ATTR)
 #undef SAS_ATTR
   if (e != cudaSuccess) return e;

@@ -44,19 +44,30 @@
 // the counters at or over N_min that are not peaks are dropped as well.  Only
 // a counter with the top bit set can be larger than a tested one, so a word
 // holding one is reset after every test of the tile (a second pass) and every
-// other word as soon as it is read.  The kernel is instantiated with and
-// without the peak tests (PEAKS), in two translation units.
+// other word as soon as it is read.
+//
+// Window search (kModeWindows): the same kernel over a coarser lattice and grid
+// (sas_hier.cu says how they are chosen and why no bin is missed).  A lattice
+// point stands for a group of fine ones and a counter for one cell; the finish
+// pass adds the counters of every win x win block of cells and emits the block's
+// first cell when the sum reaches N_min.  Tiles overlap by win - 1 cells, so
+// each block of cells lies in one tile.
+//
+// The kernel is instantiated per mode, in three translation units.
 #pragma once
 
 #include <type_traits>
 
-#include "sas_internal.cuh"
+#include "sas_count.cuh"
 
 namespace sas {
 
 namespace {
 
 constexpr int kNT = 1024;
+// What the finish pass emits: super-bins at or over n_min (kModePlain), those and
+// the tile-local peaks (kModePeaks), blocks of cells (kModeWindows).
+enum { kModePlain = 0, kModePeaks = 1, kModeWindows = 2 };
 constexpr int32_t kOutside = -(1 << 30);  // table entry of a lattice column that does not exist
 
 struct SmemLayout {
@@ -290,6 +301,46 @@ __device__ __forceinline__ uint32_t process_rec(uint32_t xr, uint32_t yr,
   else return (uint32_t)__popc(m);
 }
 
+// The window search's record loop: lattice columns are many steps apart, so no
+// two of a word share a reduction; each (detection, lattice point) pair is one.
+// No lattice mask: points past the lattice's last column count too, and the
+// finish pass drops them.  A pair outside the tile adds zero to the tile's last
+// cell on that axis: three instructions a pair (increment, address, reduction),
+// where a select of a conflict-free address would make it five, on a loop whose
+// shared-memory pipe is not the limit.
+template <int KX, int KY, int CB, bool WT>
+__device__ __forceinline__ uint32_t process_rec_windows(int32_t x, int32_t y, const int32_t* __restrict__ ox,
+                                                        const int32_t* __restrict__ oy, uint32_t cells_s,
+                                                        uint32_t tw_x, uint32_t tw_y, uint32_t magic, int tx, int txty,
+                                                        uint32_t w_in) {
+  using C = Counter<CB>;
+  static_assert(KX == 4 && KY == 4, "one 16-byte load per axis");
+  const uint32_t w = WT ? w_in : 1u;
+  const int4 ox4 = *reinterpret_cast<const int4*>(ox), oy4 = *reinterpret_cast<const int4*>(oy);
+  const int32_t oxv[4] = {ox4.x, ox4.y, ox4.z, ox4.w}, oyv[4] = {oy4.x, oy4.y, oy4.z, oy4.w};
+  uint32_t col4[KX], inc[KX], okx = 0;
+#pragma unroll
+  for (int k = 0; k < KX; ++k) {
+    const uint32_t X = (uint32_t)(x - oxv[k]);
+    const bool ok = X < tw_x;
+    okx += ok;
+    inc[k] = ok ? w << (CB * (k % C::P)) : 0u;
+    col4[k] = __umulhi(min(X, tw_x - 1u), magic) * 4u + (uint32_t)((k / C::P) * txty * 4);
+  }
+  uint32_t oky = 0;
+#pragma unroll
+  for (int k = 0; k < KY; ++k) {
+    const uint32_t Y = (uint32_t)(y - oyv[k]);
+    const bool ok = Y < tw_y;
+    oky += ok;
+    const uint32_t row = cells_s + __umulhi(min(Y, tw_y - 1u), magic) * (uint32_t)(4 * tx) +
+                         (uint32_t)(k * (KX / C::P) * txty * 4);
+#pragma unroll
+    for (int q = 0; q < KX; ++q) red_shared(row + col4[q], ok ? inc[q] : 0u);
+  }
+  return okx * oky;
+}
+
 // Sum of the counters packed in one word.
 template <int CB>
 __device__ __forceinline__ uint32_t word_sum(uint32_t w) {
@@ -300,7 +351,7 @@ __device__ __forceinline__ uint32_t word_sum(uint32_t w) {
 
 // Everything one work unit needs lives in shared memory: the counter tile, the
 // staged records, the shift tables, the windows and the bucket segments.
-template <int KX, int KY, int CB, bool PEAKS>
+template <int KX, int KY, int CB, int MODE>
 __device__ __forceinline__ void run_unit(const StackArgs& a, uint64_t unit, unsigned char* smem,
                                          bool init_cells, int64_t& balance, uint64_t& pairs64,
                                          uint32_t& my_flags) {
@@ -754,7 +805,7 @@ __device__ __forceinline__ void run_unit(const StackArgs& a, uint64_t unit, unsi
     };
 
     auto finish = [&](int kx0, int ky0) {
-      if constexpr (PEAKS) finish_peaks(kx0, ky0); else finish_plain(kx0, ky0);
+      if constexpr (MODE == kModePeaks) finish_peaks(kx0, ky0); else finish_plain(kx0, ky0);
     };
 
     const int nvt_bx = min(tc.bvx, (kxb - kxa) / KX + 1);
@@ -798,6 +849,310 @@ __device__ __forceinline__ void run_unit(const StackArgs& a, uint64_t unit, unsi
     }
 }
 
+// One unit of the window search: a spatial tile x one tile of KX x KY lattice
+// points, all epochs at once (the plan sees to it: E <= 255 epochs, one bucket row
+// per thread).  Set-up is what small units pay for, so it is kept short: bucket
+// ranges once per epoch, divisions by multiplication, one scan.
+template <int KX, int KY, int CB>
+__device__ __forceinline__ void run_unit_windows(const StackArgs& a, uint32_t unit, unsigned char* smem, bool init_cells,
+                                                 int64_t& balance, uint64_t& pairs64, uint32_t& my_flags) {
+  using C = Counter<CB>;
+  constexpr int P = C::P;
+  const TileCfg& tc = a.tc;
+  const SmemLayout L = layout(tc);
+  uint32_t* cells = reinterpret_cast<uint32_t*>(smem + L.cells);
+  const uint32_t cells_s = (uint32_t)__cvta_generic_to_shared(cells);
+  int32_t* s_ox = reinterpret_cast<int32_t*>(smem + L.ox);
+  int32_t* s_oy = reinterpret_cast<int32_t*>(smem + L.oy);
+  int4* s_win = reinterpret_cast<int4*>(smem + L.win);  // [E] bucket columns and rows: first, last, first, last
+  uint32_t* s_seg_pos = reinterpret_cast<uint32_t*>(smem + L.seg_pos);
+  uint32_t* s_seg_src = reinterpret_cast<uint32_t*>(smem + L.seg_src);
+  Emit* s_emit = reinterpret_cast<Emit*>(smem + L.emit);
+  uint32_t* s_misc = reinterpret_cast<uint32_t*>(smem + L.misc);
+  // s_misc: [0..32) records and [48..80) segments before each warp, [32], [33] their totals,
+  //         [43] emission count, [44] flush base, [45] noted rows
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const SearchGeom& g = a.g;
+  const CoarseGeom& cg = a.cg;
+  const uint32_t E = g.E;
+  const uint32_t n_words = (uint32_t)KY * (KX / P) * tc.tx * tc.ty;
+  const int txty = tc.tx * tc.ty, halo = a.win - 1;
+  const int oxs = ox_stride(tc), oys = oy_stride(tc);
+  const uint4 start4 = make_uint4(0, 0, 0, 0);
+  if (init_cells) {  // first unit of this block, or of another field
+    for (uint32_t i = tid; i < n_words / 4; i += kNT) reinterpret_cast<uint4*>(cells)[i] = start4;
+    if (tid == 0) s_misc[43] = s_misc[45] = 0;
+    __syncthreads();
+  }
+  const uint32_t n_st = (uint32_t)(a.nst_x * a.nst_y), vb = unit / n_st, st = unit - vb * n_st;
+  const uint32_t vty = vb / (uint32_t)a.nvt_x, sty = st / (uint32_t)a.nst_x;
+  const int kx0 = a.kx_lo + (int)(vb - vty * (uint32_t)a.nvt_x) * KX, ky0 = a.ky_lo + (int)vty * KY;
+  const int kxb = min(kx0 + KX, g.nvx) - 1, kyb = min(ky0 + KY, g.nvy) - 1;
+  if (a.vact) {
+    const int kx = kx0 + lane % KX, ky = ky0 + lane / KX;
+    const bool act = lane < KX * KY && kx <= kxb && ky <= kyb && a.vact[(size_t)ky * g.nvx + kx];
+    if (!__any_sync(0xffffffffu, act)) return;  // the same for every warp
+  }
+  // tiles overlap by the window side less one cell
+  const int bx0 = (int)(st - sty * (uint32_t)a.nst_x) * (tc.tx - halo), by0 = (int)sty * (tc.ty - halo);
+  const uint32_t tw_x = (uint32_t)min(tc.tx, g.nbx - bx0) * (uint32_t)g.bin;
+  const uint32_t tw_y = (uint32_t)min(tc.ty, g.nby - by0) * (uint32_t)g.bin;
+  const int32_t X0 = g.x_min + bx0 * g.bin, Y0 = g.y_min + by0 * g.bin;
+
+  // --- shift tables (tile origin plus shift) and bucket ranges of every epoch ---
+  for (int i = tid; i < (KX + KY) * 256; i += kNT) {
+    const uint32_t e = (uint32_t)i & 255u;
+    const int k = i >> 8;
+    if (e >= E) continue;
+    if (k < KX)  // columns past the lattice's edge repeat the last one; their windows are dropped
+      s_ox[e * oxs + k] = X0 + a.sxt[(size_t)min(kx0 + k, g.nvx - 1) * E + e];
+    else
+      s_oy[e * oys + k - KX] = ky0 + k - KX <= kyb ? Y0 + a.syt[(size_t)(ky0 + k - KX) * E + e] : kOutside;
+  }
+  if (tid < (int)E) {
+    const uint32_t e = tid;
+    int4 r = make_int4(0, -1, 0, -1);
+    if (a.ecount[e] > 0) {
+      const int32_t s0 = a.sxt[(size_t)kx0 * E + e], s1 = a.sxt[(size_t)kxb * E + e];
+      const int32_t t0 = a.syt[(size_t)ky0 * E + e], t1 = a.syt[(size_t)kyb * E + e];
+      bucket_range(X0 + min(s0, s1) - cg.gx0, abs(s1 - s0) + (int32_t)tw_x, a.cell_m, cg.ncx, r.x, r.y);
+      bucket_range(Y0 + min(t0, t1) - cg.gy0, abs(t1 - t0) + (int32_t)tw_y, a.cell_m, cg.ncy, r.z, r.w);
+      if (r.w - r.z >= tc.rows) my_flags |= kFlagInternal;
+    }
+    s_win[e] = r;
+  }
+  __syncthreads();
+  // --- one segment of records per (epoch, bucket row): thread t owns item t; the
+  //     non-empty ones are listed in order with the records before them ---------
+  uint32_t total, n_seg;
+  {
+    const uint32_t el = ((uint32_t)tid * a.rows_m) >> 20;  // tid / rows
+    const int r = tid - (int)el * tc.rows;
+    uint32_t len = 0, src = 0;
+    if (el < E) {
+      const int4 w = s_win[el];
+      if (w.x <= w.y && w.z + r <= w.w) {
+        const size_t b0 = ((size_t)el * cg.ncy + (w.z + r)) * cg.ncx;
+        src = a.boff[b0 + w.x];
+        len = a.boff[b0 + w.y + 1] - src;
+      }
+    }
+    uint32_t inc = len;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += v;
+    }
+    const uint32_t some = __ballot_sync(0xffffffffu, len != 0);
+    if (lane == 31) {
+      s_misc[warp] = inc;
+      s_misc[48 + warp] = (uint32_t)__popc(some);
+    }
+    __syncthreads();
+    if (warp == 0) {
+      const uint32_t x = s_misc[lane], y = s_misc[48 + lane];
+      uint32_t sx = x, sy = y;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t u = __shfl_up_sync(0xffffffffu, sx, o), v = __shfl_up_sync(0xffffffffu, sy, o);
+        if (lane >= o) {
+          sx += u;
+          sy += v;
+        }
+      }
+      s_misc[lane] = sx - x;
+      s_misc[48 + lane] = sy - y;
+      if (lane == 31) {
+        s_misc[32] = sx;
+        s_misc[33] = sy;
+      }
+    }
+    __syncthreads();
+    total = s_misc[32];
+    n_seg = s_misc[33];
+    if (len) {
+      const uint32_t q = s_misc[48 + warp] + (uint32_t)__popc(some & ((1u << lane) - 1u));
+      s_seg_pos[q] = s_misc[warp] + inc - len;
+      s_seg_src[q] = src;
+    }
+    __syncthreads();
+  }
+
+  // --- the records, straight from the buckets: a staged copy would be read once.
+  //     A warp takes a contiguous share, 32 at a time; no segment is empty, so the
+  //     32 lie in the 32 segments from the first one's on ------------------------
+  {
+    uint32_t pairs = 0, added = 0;  // pairs, and the weight they added
+    auto records = [&](auto weighted) {
+                constexpr bool WT = decltype(weighted)::value;
+                                const uint32_t share = ((total + kNT - 1) / kNT) * 32u;
+                const uint32_t j_lo = (uint32_t)warp * share, j_hi = min(j_lo + share, total);
+                uint32_t lo = 0;
+                for (uint32_t hi = n_seg; hi - lo > 1 && j_lo < j_hi;) {  // segment of the share's first record
+                  const uint32_t mid = (lo + hi) >> 1;
+                  if (s_seg_pos[mid] <= j_lo) lo = mid; else hi = mid;
+                }
+                for (uint32_t j0 = j_lo; j0 < j_hi; j0 += 32) {
+                  const uint32_t j = min(j0 + lane, j_hi - 1);
+                  const uint32_t at = lo + (uint32_t)lane;
+                  const uint32_t start_at = at < n_seg ? s_seg_pos[at] : 0xffffffffu;
+                  const uint32_t src_at = at < n_seg ? s_seg_src[at] : 0u;
+                  uint32_t k = 0;  // the last of the 32 segments that starts at or before j
+      #pragma unroll
+                  for (int step = 16; step > 0; step >>= 1)
+                    if (__shfl_sync(0xffffffffu, start_at, k + step) <= j) k += step;
+                  const uint32_t d_at = __shfl_sync(0xffffffffu, src_at, k) + (j - __shfl_sync(0xffffffffu, start_at, k));
+                  lo += __shfl_sync(0xffffffffu, k, 31);
+                  if (j0 + lane < j_hi) {
+                    const Det d = a.dets[d_at];
+                    const uint32_t w = WT ? a.w[d.id] : 1u;
+                    const uint32_t p = process_rec_windows<KX, KY, CB, WT>(d.x, d.y, s_ox + d.e * oxs ,
+                                                                           s_oy + d.e * oys , cells_s, tw_x, tw_y,
+                                                                           a.magic, tc.tx, txty, w);
+                    pairs += p;
+                    added += WT ? p * w : p;
+                  }
+                }
+    };
+    if (a.w) records(std::true_type{}); else records(std::false_type{});
+    pairs64 += pairs;
+    balance -= added;
+    __syncthreads();  // the reductions above are asm: order them before any reader
+  }
+
+  // --- windows at or over n_min --------------------------------------------------
+  // A thread walks down a strip of four adjacent columns of one counter plane (row
+  // segments split over the threads), adds each row's win neighbouring words and
+  // keeps the last rows' sums.  The sums stay packed: while every counter is below
+  // a sixteenth of its range (an eighth of that for n_min < 8) a window's sum and the
+  // bias that moves n_min to the top bit fit the counter's field, so a row of four
+  // words takes some 30 instructions.  Rows with a top bit set, or a larger
+  // counter, are noted and added up again afterwards in wider fields (emit_part):
+  // few are, and the loop stays free of that code.  The words are added up (for the
+  // balance) and reset in a second pass, once every neighbour was read.
+  {
+    using Acc = typename std::conditional<CB <= 16, uint32_t, uint64_t>::type;
+    constexpr uint32_t kOnes = CB == 8 ? 0x01010101u : CB == 16 ? 0x00010001u : 1u;
+    constexpr uint32_t kTops = kOnes << (CB - 1);
+    // 9 counters of 15 and a bias of at most 120, or of 7 and 127; of 2047 and 2^15
+    const uint32_t large = CB == 8 ? (a.n_low >= 8 ? 0xf0f0f0f0u : 0xf8f8f8f8u) : CB == 16 ? 0xf800f800u : 0xf8000000u;
+    const uint32_t bias = ((1u << (CB - 1)) - min(a.n_low, 1u << (CB - 1))) * kOnes;
+    const int own_x = tc.tx - halo, own_y = tc.ty - halo;
+    const int quads = tc.tx / 4, planes = KY * (KX / P);
+    const int nseg = max(max(1, kNT / (planes * quads)), (own_y + 29) / 30), rs = (own_y + nseg - 1) / nseg;
+    // the window that begins at (row, col) of the plane's lattice column `q`
+    auto emit = [&](int pl, int row, int col, int q) {
+      const int kx = kx0 + (pl % (KX / P)) * P + q, ky = ky0 + pl / (KX / P);
+      if (col >= own_x || kx > kxb || ky > kyb) return;
+      Emit em;
+      em.v_idx = (uint32_t)ky * (uint32_t)g.nvx + (uint32_t)kx;
+      em.bx = (uint32_t)(bx0 + col);
+      em.by = (uint32_t)(by0 + row);
+      em.flags = kEmitPlain;
+      const uint32_t p = atomicAdd(&s_misc[43], 1u);
+      if (p < (uint32_t)tc.emit_cap) {
+        s_emit[p] = em;
+      } else {
+        const uint32_t gp = atomicAdd(a.n_emit, 1u);
+        if (gp < a.emit_cap) a.emits[gp] = em; else my_flags |= kFlagEmitCap;
+      }
+    };
+    // windows j of 8 of a noted row (column 4 q + j / 2, the word's even or odd fields),
+    // added up in fields twice as wide
+    auto emit_part = [&](int pl, int row, int q, int j) {
+      constexpr uint32_t kHalf = CB == 8 ? 0x00ff00ffu : 0xffffu;
+      const int col = 4 * q + (j >> 1), sh = CB * (j & 1);
+      if (col >= own_x) return;
+      uint32_t sum = 0;
+#pragma unroll
+      for (int t = 0; t < 3; ++t)
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+          if (t <= halo && u <= halo)
+            sum += (cells[(uint32_t)(pl * txty + (row + t) * tc.tx + col + u)] >> sh) & kHalf;
+      if constexpr (CB == 8) {
+        if ((sum & 0xffffu) >= a.n_low) emit(pl, row, col, j & 1);
+        if ((sum >> 16) >= a.n_low) emit(pl, row, col, 2 + (j & 1));
+      } else {
+        if (sum >= a.n_low) emit(pl, row, col, j & 1);
+      }
+    };
+    // noted rows of a strip: bit i for row r0 + i
+    auto strip = [&](auto three, const uint32_t* at, int rows, bool edge) -> uint32_t {
+      constexpr bool W3 = decltype(three)::value;
+      uint32_t p1[4], s2[4], big1 = 0, big2 = 0, noted = 0;  // last row's sums, the last two rows' with the bias
+#pragma unroll
+      for (int j = 0; j < 4; ++j) p1[j] = s2[j] = 0;
+#pragma unroll 2
+      for (int i = W3 ? -2 : -1; i < rows; ++i, at += tc.tx) {
+        const uint4 v = *reinterpret_cast<const uint4*>(at);
+        uint2 n = make_uint2(0, 0);
+        if (!edge) n = *reinterpret_cast<const uint2*>(at + 4);
+        const uint32_t wv[6] = {v.x, v.y, v.z, v.w, n.x, n.y};
+        const uint32_t big = (v.x | v.y | v.z | v.w | n.x | n.y) & large;
+        uint32_t top = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const uint32_t h = wv[j] + wv[j + 1] + (W3 ? wv[j + 2] : 0u);
+          if constexpr (W3) {
+            top |= h + s2[j];
+            s2[j] = h + p1[j] + bias;
+          } else {
+            top |= h + p1[j] + bias;
+          }
+          p1[j] = h;
+        }
+        if (((top & kTops) | big | big1 | (W3 ? big2 : 0u)) && i >= 0) noted |= 1u << i;
+        big2 = big1;
+        big1 = big;
+      }
+      return noted;
+    };
+    for (int it = tid; it < planes * quads * nseg; it += kNT) {
+      const int rest = it / quads, q = it - rest * quads, pl = rest / nseg, r0 = (rest - pl * nseg) * rs;
+      const int rows = min(rs, own_y - r0);
+      if (rows <= 0) continue;
+      const uint32_t* at = cells + (uint32_t)(pl * txty + r0 * tc.tx + 4 * q);
+      uint32_t noted = a.win == 3 ? strip(std::true_type{}, at, rows, q + 1 == quads)
+                                  : strip(std::false_type{}, at, rows, q + 1 == quads);
+      // a mover's rows fall to few threads: list them for all (the segment arrays are free)
+      const uint32_t at0 = noted ? atomicAdd(&s_misc[45], (uint32_t)__popc(noted)) : 0u;
+      for (uint32_t p = at0; noted; ++p) {
+        const int row = r0 + __ffs(noted) - 1;
+        noted &= noted - 1;
+        if (p < (uint32_t)tc.seg_cap) {
+          s_seg_pos[p] = (uint32_t)pl << 24 | (uint32_t)row << 12 | (uint32_t)q;
+        } else {
+          for (int j = 0; j < 8; ++j) emit_part(pl, row, q, j);
+        }
+      }
+    }
+    __syncthreads();
+    const uint32_t n_noted = min(s_misc[45], (uint32_t)tc.seg_cap);
+    for (uint32_t i = tid; i < 8 * n_noted; i += kNT) {
+      const uint32_t r = s_seg_pos[i >> 3];
+      emit_part((int)(r >> 24), (int)((r >> 12) & 0xfffu), (int)(r & 0xfffu), (int)(i & 7u));
+    }
+    __syncthreads();
+    Acc acc = 0;
+    for (uint32_t i = tid; i < n_words / 4; i += kNT) {
+      const uint4 v = reinterpret_cast<const uint4*>(cells)[i];
+      reinterpret_cast<uint4*>(cells)[i] = start4;
+      acc += (Acc)word_sum<CB>(v.x) + (Acc)word_sum<CB>(v.y) + (Acc)word_sum<CB>(v.z) + (Acc)word_sum<CB>(v.w);
+    }
+    balance += (int64_t)acc;
+    const uint32_t ne_tile = min(s_misc[43], (uint32_t)tc.emit_cap);
+    if (ne_tile) {
+      if (tid == 0) s_misc[44] = atomicAdd(a.n_emit, ne_tile);
+      __syncthreads();
+      const uint32_t base = s_misc[44];
+      for (uint32_t i = tid; i < ne_tile; i += kNT) {
+        if (base + i < a.emit_cap) a.emits[base + i] = s_emit[i]; else my_flags |= kFlagEmitCap;
+      }
+    }
+    __syncthreads();
+    if (tid == 0) s_misc[43] = s_misc[45] = 0;
+  }
+}
+
 // Single field: StackArgs as the kernel parameter.  Several fields (one
 // persistent launch over all their units): fargs[f] for field f, whose units
 // are [unit_base[f], unit_base[f + 1]) of one global work counter.
@@ -808,20 +1163,43 @@ struct MultiArgs {
   unsigned long long* counter;
 };
 
-template <int KX, int KY, int CB, bool MULTI, bool PEAKS>
+template <int KX, int KY, int CB, bool MULTI, int MODE>
 __global__ void __launch_bounds__(kNT, 1) k_stack(StackArgs a0, MultiArgs m) {
   static_assert(KX % (32 / CB) == 0, "kx must be a multiple of the counters per word");
   static_assert(KX * KY <= 64, "at most 64 velocities per tile");
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ StackArgs s_args;
-  __shared__ unsigned long long s_unit, s_local;
+  __shared__ unsigned long long s_local;
   __shared__ int s_field;
   const int tid = threadIdx.x;
   int cur_field = -1;
+  int64_t balance = 0;  // (counted excess over the start values) - (pairs added)
+  uint64_t pairs64 = 0;
+  uint32_t my_flags = 0;
+  // Statistics of the units run so far: one global atomic each per warp and field.
+  auto report = [&](const StackArgs& a) {
+    for (int o = 16; o > 0; o >>= 1) {
+      pairs64 += __shfl_xor_sync(0xffffffffu, pairs64, o);
+      balance += __shfl_xor_sync(0xffffffffu, balance, o);
+      my_flags |= __shfl_xor_sync(0xffffffffu, my_flags, o);
+    }
+    if ((tid & 31) == 0) {
+      if (pairs64) atomicAdd(a.n_pairs, (unsigned long long)pairs64);
+      if (balance) atomicAdd(a.balance, (unsigned long long)balance);
+      if (my_flags) atomicOr(a.flags, my_flags);
+    }
+    pairs64 = 0;
+    balance = 0;
+    my_flags = 0;
+  };
+  // The next unit is drawn while the current one runs, so that nobody waits for
+  // the counter's round trip (about 1500 cycles a unit) -- but for the peak tests,
+  // whose registers are full.
+  constexpr bool kAhead = MODE != kModePeaks;
+  unsigned long long t_next = kAhead && tid == 0 ? atomicAdd(MULTI ? m.counter : a0.tile_counter, 1ull) : 0ull;
   while (true) {
     if (tid == 0) {
-      const unsigned long long t = atomicAdd(MULTI ? m.counter : a0.tile_counter, 1ull);
-      s_unit = t;
+      const unsigned long long t = kAhead ? t_next : atomicAdd(MULTI ? m.counter : a0.tile_counter, 1ull);
       if (MULTI) {
         const unsigned long long total = m.unit_base[m.n_fields];
         int f = 0;
@@ -845,46 +1223,42 @@ __global__ void __launch_bounds__(kNT, 1) k_stack(StackArgs a0, MultiArgs m) {
     const int field = s_field;
     if (local == ~0ull) break;
     if (MULTI && field != cur_field) {
+      if (MODE != kModePeaks && cur_field >= 0) {
+        report(s_args);
+        __syncthreads();
+      }
       const uint32_t* src = reinterpret_cast<const uint32_t*>(&m.fargs[field]);
       uint32_t* dst = reinterpret_cast<uint32_t*>(&s_args);
       for (int i = tid; i < (int)(sizeof(StackArgs) / 4); i += kNT) dst[i] = src[i];
       __syncthreads();
     }
     const StackArgs& a = MULTI ? s_args : a0;
-    int64_t balance = 0;  // (counted excess over the start values) - (pairs added)
-    uint64_t pairs64 = 0;
-    uint32_t my_flags = 0;
-    run_unit<KX, KY, CB, PEAKS>(a, local, smem, field != cur_field, balance, pairs64, my_flags);
+    if (kAhead && tid == 0) t_next = atomicAdd(MULTI ? m.counter : a0.tile_counter, 1ull);
+    if constexpr (MODE == kModeWindows)
+      run_unit_windows<KX, KY, CB>(a, (uint32_t)local, smem, field != cur_field, balance, pairs64, my_flags);
+    else
+      run_unit<KX, KY, CB, MODE>(a, local, smem, field != cur_field, balance, pairs64, my_flags);
     cur_field = field;
-    // Per-unit statistics of this field: one global atomic each per warp.
-    for (int o = 16; o > 0; o >>= 1) {
-      pairs64 += __shfl_xor_sync(0xffffffffu, pairs64, o);
-      balance += __shfl_xor_sync(0xffffffffu, balance, o);
-      my_flags |= __shfl_xor_sync(0xffffffffu, my_flags, o);
-    }
-    if ((tid & 31) == 0) {
-      if (pairs64) atomicAdd(a.n_pairs, (unsigned long long)pairs64);
-      if (balance) atomicAdd(a.balance, (unsigned long long)balance);
-      if (my_flags) atomicOr(a.flags, my_flags);
-    }
+    if constexpr (MODE == kModePeaks) report(a);  // its registers are short: no sums kept across units
     __syncthreads();
   }
+  if (MODE != kModePeaks && cur_field >= 0) report(MULTI ? s_args : a0);
 }
 
-template <int KX, int KY, int CB, bool PEAKS>
+template <int KX, int KY, int CB, int MODE>
 cudaError_t launch_t(const StackArgs& a, int grid, cudaStream_t s) {
   MultiArgs m{};
-  k_stack<KX, KY, CB, false, PEAKS><<<grid, kNT, a.tc.smem, s>>>(a, m);
+  k_stack<KX, KY, CB, false, MODE><<<grid, kNT, a.tc.smem, s>>>(a, m);
   note_launch();
   return cudaGetLastError();
 }
 
-template <int KX, int KY, int CB, bool PEAKS>
+template <int KX, int KY, int CB, int MODE>
 cudaError_t launch_multi_t(const StackArgs& proto, const StackArgs* fargs,
                            const unsigned long long* unit_base, int n_fields,
                            unsigned long long* counter, size_t smem, int grid, cudaStream_t s) {
   MultiArgs m{fargs, unit_base, n_fields, counter};
-  k_stack<KX, KY, CB, true, PEAKS><<<grid, kNT, smem, s>>>(proto, m);
+  k_stack<KX, KY, CB, true, MODE><<<grid, kNT, smem, s>>>(proto, m);
   note_launch();
   return cudaGetLastError();
 }
@@ -906,11 +1280,11 @@ inline cudaError_t raise_smem_limit(const void* f, size_t smem) {
   return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim);
 }
 
-template <int KX, int KY, int CB, bool PEAKS>
+template <int KX, int KY, int CB, int MODE>
 cudaError_t attr_t(size_t smem) {
-  cudaError_t e = raise_smem_limit((const void*)k_stack<KX, KY, CB, false, PEAKS>, smem);
+  cudaError_t e = raise_smem_limit((const void*)k_stack<KX, KY, CB, false, MODE>, smem);
   if (e != cudaSuccess) return e;
-  return raise_smem_limit((const void*)k_stack<KX, KY, CB, true, PEAKS>, smem);
+  return raise_smem_limit((const void*)k_stack<KX, KY, CB, true, MODE>, smem);
 }
 
 // Supported (KX, KY, CB) instantiations.

@@ -1,0 +1,155 @@
+"""The two-level window search (the default for large searches) against the
+one-level kernel, which a caller's tile sizes select, byte for byte: candidate
+records, ids and pair counts, over lattices, domains, epochs and thresholds at
+the edges of what the two-level search takes.  The oracle judges one of them."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2509_26279_gb300 import workloads as W
+from tests import cases
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA device", allow_module_level=True)
+
+from paper_2509_26279_gb300 import sas  # noqa: E402
+from tests.test_gpu_parity import assert_same  # noqa: E402
+
+
+def _field(seed, width=1021, height=1777, epochs=60, noise=700, movers=40, span=4.0):
+    r = W.FieldRecipe(width, height, epochs, span, noise, movers, (0.5, 15.0), (0.9, 0.4))
+    return W.make_catalog(r, seed)
+
+
+def _grid(width=1021, height=1777, nvx=75, nvy=83, dvx=364, dvy=364, bin_mpx=2000, x_min=0, y_min=0, **kw):
+    return W.GridSpec(vx0=-(nvx // 2) * dvx, vy0=-(nvy // 2) * dvy, dvx=dvx, dvy=dvy, nvx=nvx, nvy=nvy, x_min=x_min,
+                      y_min=y_min, nbx=-(-width * 1000 // bin_mpx), nby=-(-height * 1000 // bin_mpx), bin=bin_mpx, **kw)
+
+
+def _both(cat, grid, n_min, **kw):
+    """(default search, one-level search) as bytes, and their infos."""
+    out = []
+    for tiles in (dict(), dict(tile_kx=8, tile_ky=8)):
+        o = sas.make_opts(**tiles)
+        for k, v in kw.items():
+            setattr(o, k, v)
+        res = sas.stack_catalog(sas.Grid(grid), cat, n_min, opts=o)
+        c, ids = res.candidates()
+        out.append((c.tobytes(), ids.tobytes(), len(c), res.info()))
+    return out
+
+
+def _check(cat, grid, n_min, **kw):
+    two, one = _both(cat, grid, n_min, **kw)
+    assert two[2] == one[2] and two[0] == one[0] and two[1] == one[1]
+    assert two[3]["n_pairs"] == one[3]["n_pairs"] and two[3]["t0"] == one[3]["t0"]
+    return two, one
+
+
+def _shuffled_times(cat):
+    """Epoch times out of order, the earliest in the middle, epochs 0 and 7 without detections."""
+    t = np.roll(cat.t, 23) + 12345
+    keep = (cat.epoch != 0) & (cat.epoch != 7)
+    return cases.catalog(cat.x[keep], cat.y[keep], cat.epoch[keep], t, cat.ticks_per_hour)
+
+
+GRIDS = [
+    dict(),
+    dict(dvx=-364, dvy=200),                       # one axis backwards, unequal steps: unequal groups
+    dict(nvx=73, nvy=1, dvx=364, dvy=0),            # a single lattice row
+    dict(nvx=9, nvy=300, dvx=364, dvy=120),
+    dict(bin_mpx=2501, x_min=-31000, y_min=17001),  # a domain that is not the field
+    dict(speed_min=3000, speed_max=12000),
+]
+
+
+@pytest.mark.parametrize("grid", GRIDS)
+def test_lattices_and_domains(grid):
+    cat = _field(1)
+    two, one = _check(cat, _grid(**grid), 15)
+    assert two[2] > 0
+    if grid.get("nvy", 83) > 1:
+        assert two[3]["n_emitted"] != one[3]["n_emitted"]   # windows, not super-bins: the two-level search ran
+
+
+@pytest.mark.parametrize("a,b", [(0, 17), (5, 3000), (2100, 75 * 83), (75 * 40, 75 * 41), (75 * 83 - 1, 75 * 83)])
+def test_lattice_ranges(a, b):
+    _check(_field(2), _grid(), 14, v_begin=a, v_end=b)
+
+
+@pytest.mark.parametrize("n_min", [5, 7, 8, 9, 16, 40])
+def test_thresholds(n_min):
+    """Both packings of the window sums (n_min under and over 8) and cells with more than 15 detections."""
+    two, _ = _check(_field(3, noise=150, movers=60), _grid(nvx=111, nvy=111), n_min)
+    assert two[2] > 0
+
+
+@pytest.mark.parametrize("epochs,n_min", [(11, 8), (128, 30), (150, 128), (255, 60), (256, 60)])
+def test_epoch_counts(epochs, n_min):
+    """Few epochs, bucket rows shared by many, the last count that the two-level search takes and the first that it does not."""
+    cat = _field(4, epochs=epochs, noise=60000 // epochs, movers=30)
+    _check(cat, _grid(), n_min)
+
+
+def test_times_out_of_order_and_empty_epochs():
+    two, _ = _check(_shuffled_times(_field(5)), _grid(), 14)
+    assert two[2] > 0
+
+
+def test_repeated_detections():
+    """Every detection three times (raw counts three times the distinct ones), and a cell that wraps an 8-bit counter."""
+    cat = _field(6, noise=400)
+    rep = lambda a: np.concatenate([a, a, a])  # noqa: E731
+    _check(cases.catalog(rep(cat.x), rep(cat.y), rep(cat.epoch), cat.t, cat.ticks_per_hour), _grid(), 14)
+    x = np.concatenate([cat.x, np.full(400, 500_000, np.int32)])
+    y = np.concatenate([cat.y, np.full(400, 500_000, np.int32)])
+    e = np.concatenate([cat.epoch, np.zeros(400, np.uint16)])
+    _check(cases.catalog(x, y, e, cat.t, cat.ticks_per_hour), _grid(), 14)
+
+
+def test_top_k_and_device_arrays():
+    cat, grid = _field(7), _grid()
+    full = _check(cat, grid, 14)[0]
+    assert full[2] > 50
+    top = _both(cat, grid, 14, max_candidates=50)[0]
+    assert top[0] == full[0][:50 * 32]
+    dev = [torch.from_numpy(a).cuda() for a in (cat.x, cat.y, cat.epoch.view(np.int16))]
+    s = torch.cuda.Stream()
+    res = sas.sas_stack(sas.Grid(grid), *dev, cat.t, cat.ticks_per_hour, 14, on_device=True, stream=s)
+    assert res.candidates()[0].tobytes() == full[0]
+
+
+@pytest.mark.parametrize("kind", ["ones", "wide", "zeros", "host"])
+def test_weights(kind):
+    """Weighted stacking through the windows: weights all one, over the whole range with repeated epochs in a bin, mostly
+    zero, and from host arrays."""
+    cat, grid = _field(9, movers=60), _grid()
+    rep = np.concatenate
+    x, y, e = rep([cat.x, cat.x]), rep([cat.y, cat.y]), rep([cat.epoch, cat.epoch])
+    rng = np.random.default_rng(3)
+    w = {"ones": np.ones(len(x)), "wide": rng.integers(0, 256, len(x)), "zeros": 200 * (rng.random(len(x)) < 0.1),
+         "host": 20 + rng.integers(0, 60, len(x))}[kind].astype(np.uint8)
+    s_min = {"ones": 16, "wide": 2600, "zeros": 1000, "host": 900}[kind]
+    got = []
+    for tiles in (dict(), dict(tile_kx=8, tile_ky=4)):
+        o = sas.make_opts(**tiles)
+        if kind == "host":
+            res = sas.sas_stack_weighted(sas.Grid(grid), x, y, e, w, cat.t, cat.ticks_per_hour, s_min, opts=o)
+        else:
+            d = [torch.from_numpy(a).cuda() for a in (x, y, e.view(np.int16), w)]
+            res = sas.sas_stack_weighted(sas.Grid(grid), *d, cat.t, cat.ticks_per_hour, s_min, opts=o, on_device=True)
+        c, ids = res.candidates()
+        got.append((c.tobytes(), ids.tobytes(), res.info()["n_pairs"]))
+    assert got[0] == got[1]
+    assert len(got[0][0]) > 0
+
+
+def test_oracle():
+    cat, grid = _field(8, width=700, height=900, noise=300), _grid(width=700, height=900)
+    res = sas.stack_catalog(sas.Grid(grid), cat, 13)
+    ref = oracle.stack(cat, grid, 13, threads=0)
+    assert len(ref.cands) > 0
+    assert_same(res, ref)

@@ -67,6 +67,16 @@ __device__ __forceinline__ void split_fp32(float g, uint16_t& hi, uint16_t& mid,
   lo = (uint16_t)(__float_as_uint(r2) >> 16);
 }
 
+// 16 bytes from global to shared memory without a register stop; zeros when !valid
+// (the source is not read then).  cp_commit closes a group; cp_wait<N> waits until at
+// most N groups of this thread are in flight.
+__device__ __forceinline__ void cp16(void* dst, const void* src, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(valid ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
 // One warp: allocate ncols (power of two >= 32) TMEM columns; base written to *slot.
 __device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(ncols));

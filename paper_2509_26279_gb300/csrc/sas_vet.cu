@@ -43,12 +43,12 @@ struct sas_vet {
   __nv_bfloat16* a4;     // [B][64]
   float* logits;         // [B]
   float* fcpart;         // [kFcSplit][64][B rounded up to 128] fc1 partial sums
-  float* glogit;         // [B]
   float* g4;             // [B][64]
   float* g3;             // [B][2592]
   float* g2;             // [B][32][11][11]
   float* g1;             // [B][32][13][13]
-  float* partial;        // per-block weight-gradient partial sums
+  float* partial;        // per-block weight-gradient partial sums, one part per conv layer
+  float* lpart;          // per-block sums of the loss and the fc2 gradients
   float* loss;           // [1]
   uint32_t* status;      // [1] nonzero: a tensor-core wait gave up (sas_vet_check)
 };
@@ -67,7 +67,7 @@ static_assert(kNParams == 187137, "parameter layout");
 
 constexpr int kBackBlocks = 304;      // blocks (and partial sums) of the conv backward kernels: two per SM
 constexpr int kPartialStride = kCh * kCh * 9 + kCh;  // >= parts * weights + biases of any layer
-constexpr uint32_t kFc1Slices = 8;                   // stamp slices of the fc1 weight gradient
+constexpr uint32_t kFc1Slices = 14;                  // stamp slices of the fc1 weight gradient
 static_assert((size_t)kFc1Slices * (kHid * kF + kHid) <= (size_t)kBackBlocks * kPartialStride,
               "fc1 slices fit the partial buffer");
 
@@ -111,14 +111,13 @@ static_assert(kSmW1 % 128 == 0 && kSmW2 % 128 == 0 && kSmW3 % 128 == 0 && kSmA1 
                   kSmA2 % 16 == 0, "operand alignment");
 static_assert(2 * kTcSmem <= 227 * 1024, "two CTAs per SM");
 
-// Per-tap weights of a layer as the B operand: B_t[o][c] = w[o][c][t] (c < cin),
-// zero for c >= cin; kc 16-byte chunks per row (K = 8 kc).
+// Per-tap weights of a layer as the B operand: B_t[o][c] = w[o][c][t]; kc 16-byte
+// chunks per row (K = 8 kc; columns c >= cin stay as they are).  Read in memory order.
 __device__ void tc_load_w_taps(const __nv_bfloat16* __restrict__ w, int cin, int kc, unsigned char* dst) {
   const int per_tap = kCh * kc * 8;
-  for (int i = threadIdx.x; i < 9 * per_tap; i += blockDim.x) {
-    const int t = i / per_tap, j = i - t * per_tap, o = j / (kc * 8), c = j - o * (kc * 8);
-    const __nv_bfloat16 v = c < cin ? w[(o * cin + c) * 9 + t] : __float2bfloat16_rn(0.f);
-    *reinterpret_cast<__nv_bfloat16*>(dst + t * per_tap * 2 + tc::cm_offset(o, c, kc)) = v;
+  for (int i = threadIdx.x; i < kCh * cin * 9; i += blockDim.x) {
+    const int o = i / (cin * 9), j = i - o * (cin * 9), c = j / 9, t = j - c * 9;
+    *reinterpret_cast<__nv_bfloat16*>(dst + t * per_tap * 2 + tc::cm_offset(o, c, kc)) = w[i];
   }
 }
 
@@ -212,9 +211,10 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_conv_fwd_tc(const uint16_t* _
   const int tid = threadIdx.x;
   if (tid < 32) tc::tmem_alloc(tslot, kTcTmemCols);
   if (tid == 0) tc::mbar_init(bar, 1);
-  // activation buffers: rows that are never written (input padding, channel
-  // padding of x0) stay zero
-  for (int i = tid; i < kSmW1 / 16; i += kTcThreads) reinterpret_cast<uint4*>(smc)[i] = make_uint4(0, 0, 0, 0);
+  // activation buffers and conv1's weights: rows that are never written (input
+  // padding, channel padding) stay zero
+  for (int i = tid; i < kSmW2 / 16; i += kTcThreads) reinterpret_cast<uint4*>(smc)[i] = make_uint4(0, 0, 0, 0);
+  __syncthreads();
   tc_load_w_taps(wb + kW1, kQ, 2, smc + kSmW1);
   tc_load_w_taps(wb + kW2, kCh, 4, smc + kSmW2);
   tc_load_w_taps(wb + kW3, kCh, 4, smc + kSmW3);
@@ -273,9 +273,11 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_conv_fwd_tc(const uint16_t* _
 // D[stamp][j] = sum_k a3[stamp][k] * fc1.w[j][k]: M = 128 stamps per block,
 // N = 64, K = 2592 in 27 blocks of 96, split over kFcSplit blocks along K so
 // that a batch of 4096 stamps keeps 128 SMs busy.  Both operands are
-// K-contiguous in global memory; every thread copies 16-byte rows of core
-// matrices into the no-swizzle K-major layout of one of three stages while the
-// MMAs of the others run (one mbarrier per stage, bounded waits).  Each block
+// K-contiguous in global memory; 16-byte rows of core matrices go to the no-swizzle
+// K-major layout of one of three stages by asynchronous copies, two blocks ahead of
+// the MMAs (one mbarrier per stage, bounded waits); what bounds a block is the
+// latency of its 7 K blocks, which copies through registers took one after another
+// (41 us for 512 as for 4096 stamps).  Each block
 // writes its FP32 partial D column-major; k_fc_epi adds the kFcSplit partials
 // in a fixed order, adds the bias, applies ReLU, rounds to BF16, stores a4 and
 // forms the logit with fc2 in a fixed order.
@@ -308,33 +310,46 @@ __global__ void __launch_bounds__(kFcTcThreads) k_fc_fwd_tc(const __nv_bfloat16*
   const uint4* a3v = reinterpret_cast<const uint4*>(a3g);
   const uint4* w1v = reinterpret_cast<const uint4*>(wb + kWf1);
   constexpr uint32_t idesc = tc::idesc_bf16(kFcTcRows, kHid);
+  const int nkb = kb_hi - kb_lo;
+  auto load = [&](int l) {  // K block l of this block's into its stage; one copy group
+    if (l < nkb) {
+      unsigned char* A = smf + (l % kFcTcStages) * kFcTcStage;
+      unsigned char* B = A + kFcTcA;
+      const int k8 = (kb_lo + l) * kFcTcKC;  // first 16-byte chunk of the block along K
+      for (int i = tid; i < kFcTcRows * kFcTcKC; i += kFcTcThreads) {
+        const int r = i / kFcTcKC, c = i - r * kFcTcKC;
+        const bool in = b0 + r < n;
+        tc::cp16(A + tc::cm_offset(r, c * 8, kFcTcKC), a3v + (in ? (size_t)(b0 + r) * (kF / 8) + k8 + c : 0), in);
+      }
+      for (int i = tid; i < kHid * kFcTcKC; i += kFcTcThreads) {
+        const int r = i / kFcTcKC, c = i - r * kFcTcKC;
+        tc::cp16(B + tc::cm_offset(r, c * 8, kFcTcKC), w1v + (size_t)r * (kF / 8) + k8 + c, true);
+      }
+    }
+    tc::cp_commit();
+  };
   uint32_t ph[kFcTcStages] = {};
   bool ok = true;
-  for (int kb = kb_lo; kb < kb_hi && ok; ++kb) {
-    const int l = kb - kb_lo, st = l % kFcTcStages;
-    unsigned char* A = smf + st * kFcTcStage;
-    unsigned char* B = A + kFcTcA;
-    if (l >= kFcTcStages) {  // the MMAs that read this stage kFcTcStages blocks ago are done
-      ok = tc::mbar_wait(bar + st, ph[st], 1u << 22);
-      ph[st] ^= 1u;
-      if (__syncthreads_or(!ok)) break;
+  load(0);
+  load(1);
+  for (int l = 0; l < nkb && ok; ++l) {
+    const int st = l % kFcTcStages, nx = (l + 2) % kFcTcStages;
+    if (l + 2 >= kFcTcStages && l + 2 < nkb) {  // the MMAs that read stage nx are done
+      ok = tc::mbar_wait(bar + nx, ph[nx], 1u << 22);
+      ph[nx] ^= 1u;
+      if (__syncthreads_or(!ok)) {
+        ok = false;
+        break;
+      }
     }
-    const int k8 = kb * kFcTcKC;  // first 16-byte chunk of the block along K
-    for (int i = tid; i < kFcTcRows * kFcTcKC; i += kFcTcThreads) {
-      const int r = i / kFcTcKC, c = i - r * kFcTcKC;
-      const uint4 v = b0 + r < n ? a3v[(size_t)(b0 + r) * (kF / 8) + k8 + c] : make_uint4(0, 0, 0, 0);
-      *reinterpret_cast<uint4*>(A + tc::cm_offset(r, c * 8, kFcTcKC)) = v;
-    }
-    for (int i = tid; i < kHid * kFcTcKC; i += kFcTcThreads) {
-      const int r = i / kFcTcKC, c = i - r * kFcTcKC;
-      *reinterpret_cast<uint4*>(B + tc::cm_offset(r, c * 8, kFcTcKC)) = w1v[(size_t)r * (kF / 8) + k8 + c];
-    }
+    load(l + 2);
+    tc::cp_wait<2>();  // block l has arrived
     tc::fence_smem_to_async();
     tc::fence_before_sync();
     __syncthreads();
     if (tid == 0) {
       tc::fence_after_sync();
-      const uint32_t a0 = tc::smem_u32(A), w0 = tc::smem_u32(B);
+      const uint32_t a0 = tc::smem_u32(smf + st * kFcTcStage), w0 = a0 + kFcTcA;
 #pragma unroll
       for (int ks = 0; ks < kFcTcKC / 2; ++ks)
         tc::mma_bf16(tmem, tc::smem_desc(a0 + (uint32_t)(2 * ks * 128), kFcTcKC),
@@ -342,8 +357,9 @@ __global__ void __launch_bounds__(kFcTcThreads) k_fc_fwd_tc(const __nv_bfloat16*
       tc::commit(bar + st);
     }
   }
+  tc::cp_wait<0>();
   if (ok) {  // one commit outstanding on every stage that was used
-    const int used = min(kb_hi - kb_lo, kFcTcStages);
+    const int used = min(nkb, kFcTcStages);
     for (int st = 0; st < used && ok; ++st) {
       ok = tc::mbar_wait(bar + st, ph[st], 1u << 22);
       ph[st] ^= 1u;
@@ -370,150 +386,252 @@ __global__ void __launch_bounds__(kFcTcThreads) k_fc_fwd_tc(const __nv_bfloat16*
   if (tid < 32) tc::tmem_free(tmem, kHid);
 }
 
-// One thread per stamp: the partial sums in split order, bias, ReLU, BF16,
-// then fc2 in j order.
+// 32 stamps x 8 groups of 8 hidden units per block: the partial sums in split
+// order, bias, ReLU, BF16, then fc2 -- each group's products in order, the groups
+// in order.  (One thread per stamp walked its 64 units in turn: 29 us, all latency.)
 __global__ void __launch_bounds__(256) k_fc_epi(const float* __restrict__ part, uint32_t ldp, uint32_t n,
                                                 const __nv_bfloat16* __restrict__ wb, __nv_bfloat16* a4g,
                                                 float* __restrict__ logits) {
-  __shared__ float b1[kHid], w2[kHid];
-  if (threadIdx.x < kHid) {
-    b1[threadIdx.x] = ld(wb + kBf1 + threadIdx.x);
-    w2[threadIdx.x] = ld(wb + kWf2 + threadIdx.x);
-  }
-  __syncthreads();
-  const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= n) return;
-  float logit = 0.f;
-  for (int j = 0; j < kHid; ++j) {
-    float acc = part[(size_t)j * ldp + b];
+  __shared__ float dots[8][32];
+  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+  const uint32_t b = blockIdx.x * 32 + lane;
+  float v[8], dot = 0.f;
+  if (b < n) {
 #pragma unroll
-    for (int sp = 1; sp < kFcSplit; ++sp) acc += part[((size_t)sp * kHid + j) * ldp + b];
-    const float a = bf(fmaxf(acc + b1[j], 0.f));
-    if (a4g) a4g[(size_t)b * kHid + j] = __float2bfloat16_rn(a);
-    logit = fmaf(a, w2[j], logit);
+    for (int k = 0; k < 8; ++k) {
+      const int j = grp * 8 + k;
+      float acc = part[(size_t)j * ldp + b];
+#pragma unroll
+      for (int sp = 1; sp < kFcSplit; ++sp) acc += part[((size_t)sp * kHid + j) * ldp + b];
+      v[k] = acc;
+    }
+    uint32_t pk[4];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int j = grp * 8 + k;
+      const __nv_bfloat16 a = __float2bfloat16_rn(fmaxf(v[k] + ld(wb + kBf1 + j), 0.f));
+      pk[k / 2] = (k & 1) ? pk[k / 2] | ((uint32_t)__bfloat16_as_ushort(a) << 16) : (uint32_t)__bfloat16_as_ushort(a);
+      dot = fmaf(__bfloat162float(a), ld(wb + kWf2 + j), dot);
+    }
+    if (a4g) *reinterpret_cast<uint4*>(a4g + (size_t)b * kHid + grp * 8) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
   }
-  logits[b] = logit + ld(wb + kBf2);
+  dots[grp][lane] = dot;
+  __syncthreads();
+  if (grp == 0 && b < n) {
+    float s = dots[0][lane];
+#pragma unroll
+    for (int g = 1; g < 8; ++g) s += dots[g][lane];
+    logits[b] = s + ld(wb + kBf2);
+  }
 }
 
 // ---- loss, fc2 gradients, fc1 output deltas ------------------------------------
 
-// One block: per-stamp loss and d loss / d logit; loss mean; fc2 gradients.
-constexpr int kLossThreads = 1024;
+// Blocks of 128 stamps: per-stamp loss and d loss / d logit, the fc1 output deltas
+// g4[b][j] = glogit[b] * w2[j] * (a4[b][j] > 0), and this block's sums for the fc2
+// gradients and the loss: lpart[block][66] = fc2.w (64), fc2.b, loss.  k_fc1_sum
+// adds the blocks in order.
+constexpr int kLossStamps = 128, kLossOut = kHid + 2;
 
-__global__ void __launch_bounds__(kLossThreads) k_loss(const float* __restrict__ logits,
-                                                       const float* __restrict__ labels,
-                                                       const uint32_t* __restrict__ idx, uint32_t n,
-                                                       const __nv_bfloat16* __restrict__ a4g,
-                                                       float* __restrict__ glogit,
-                                                       float* __restrict__ grad, float* __restrict__ loss) {
-  __shared__ float red[kLossThreads];
+__global__ void __launch_bounds__(256) k_loss(const float* __restrict__ logits, const float* __restrict__ labels,
+                                              const uint32_t* __restrict__ idx, uint32_t n,
+                                              const __nv_bfloat16* __restrict__ a4g,
+                                              const __nv_bfloat16* __restrict__ wb, float* __restrict__ g4,
+                                              float* __restrict__ lpart) {
+  __shared__ float gl[kLossStamps], red[256], redb[kLossStamps / 32], redl[kLossStamps / 32];
   const int t = threadIdx.x;
   const float inv_n = 1.f / (float)n;
-  float l = 0.f;
-  for (uint32_t b = t; b < n; b += blockDim.x) {
-    const float z = logits[b], y = labels[idx ? idx[b] : b];
-    l += fmaxf(z, 0.f) - z * y + log1pf(expf(-fabsf(z)));
-    glogit[b] = (1.f / (1.f + expf(-z)) - y) * inv_n;
+  const uint32_t b0 = blockIdx.x * kLossStamps, nb = min((uint32_t)kLossStamps, n - b0);
+  if (t < kLossStamps) {
+    float l = 0.f, g = 0.f;
+    if ((uint32_t)t < nb) {
+      const uint32_t b = b0 + t;
+      const float z = logits[b], y = labels[idx ? idx[b] : b];
+      l = fmaxf(z, 0.f) - z * y + log1pf(expf(-fabsf(z)));
+      g = (1.f / (1.f + expf(-z)) - y) * inv_n;
+    }
+    gl[t] = g;
+    for (int o = 16; o > 0; o >>= 1) {
+      l += __shfl_xor_sync(0xffffffffu, l, o);
+      g += __shfl_xor_sync(0xffffffffu, g, o);
+    }
+    if ((t & 31) == 0) {
+      redb[t >> 5] = g;
+      redl[t >> 5] = l;
+    }
   }
-  red[t] = l;
   __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (t < s) red[t] += red[t + s];
-    __syncthreads();
-  }
-  if (t == 0) *loss = red[0] * inv_n;
-  __syncthreads();
-  // fc2.w[j] = sum_b glogit[b] * a4[b][j]; fc2.b = sum_b glogit[b]
-  // 16 parts of the batch per hidden unit, combined in a fixed order
   const int j = t & 63, part = t >> 6;
-  float acc = 0.f, accb = 0.f;
-  for (uint32_t b = part; b < n; b += 16) {
-    const float g = glogit[b];
-    acc = fmaf(g, ld(a4g + (size_t)b * kHid + j), acc);
-    accb += g;
+  const float w2 = ld(wb + kWf2 + j);
+  float acc = 0.f;
+#pragma unroll 8
+  for (uint32_t r = part; r < nb; r += 4) {
+    const size_t at = (size_t)(b0 + r) * kHid + j;
+    const float a = ld(a4g + at), g = gl[r];
+    acc = fmaf(g, a, acc);
+    g4[at] = a > 0.f ? g * w2 : 0.f;
   }
   red[t] = acc;
   __syncthreads();
-  if (t < 64) {
-    float s = 0.f;
-    for (int p = 0; p < 16; ++p) s += red[p * 64 + t];
-    grad[kWf2 + t] = s;
-  }
-  __syncthreads();
-  red[t] = (j == 0) ? accb : 0.f;
-  __syncthreads();
-  if (t == 0) {
-    float s = 0.f;
-    for (int p = 0; p < 16; ++p) s += red[p * 64];
-    grad[kBf2] = s;
-  }
+  float* out = lpart + (size_t)blockIdx.x * kLossOut;
+  if (t < kHid) out[t] = ((red[t] + red[64 + t]) + red[128 + t]) + red[192 + t];
+  if (t == 64) out[kHid] = ((redb[0] + redb[1]) + redb[2]) + redb[3];
+  if (t == 65) out[kHid + 1] = ((redl[0] + redl[1]) + redl[2]) + redl[3];
 }
 
-// g4[b][j] = glogit[b] * w2[j] * (a4[b][j] > 0)
-__global__ void k_g4(const float* __restrict__ glogit, const __nv_bfloat16* __restrict__ a4g,
-                     const __nv_bfloat16* __restrict__ wb, uint32_t n, float* __restrict__ g4) {
-  const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  if (i >= (uint64_t)n * kHid) return;
-  const int j = (int)(i % kHid);
-  g4[i] = ld(a4g + i) > 0.f ? glogit[i / kHid] * ld(wb + kWf2 + j) : 0.f;
-}
+// fc1.w[j][k] = sum_b g4[b][j] * a3[b][k];  fc1.b[j] = sum_b g4[b][j]; on the tensor
+// cores: M = 128 columns k (a3), N = 3 x 64 (j at each of the three BF16 parts of g4,
+// split_fp32: exact products, FP32 sums), K = 16 stamps per MMA, both operands
+// MN-major straight from the row-major arrays.  Grid (21 column tiles, S): slice s
+// adds the stamps [s n / S, (s + 1) n / S) in chunks of 64 through two stages and
+// writes part[s][j][k] and its bias sums part[S * 64 * kF + s * 64 + j]; k_fc1_sum adds
+// the slices in order.  (On the CUDA cores: 90 us for 4096 stamps, 65 for 512.)
+constexpr int kDwThreads = 256, kDwChunk = 64, kDwCols = 128;
+constexpr int kDwTiles = (kF + kDwCols - 1) / kDwCols;
+constexpr int kDwA = (kDwCols / 8) * kDwChunk * 16, kDwB = 24 * kDwChunk * 16, kDwStage = kDwA + kDwB;
+constexpr int kDwSmem = 2 * kDwStage + 32;
 
-// fc1.w[j][k] = sum_b g4[b][j] * a3[b][k];  fc1.b[j] = sum_b g4[b][j].
-// Block: 32 columns k, all 64 rows j, whole batch.
-// Grid (columns / 32, slices): slice s adds the stamps [s n / S, (s + 1) n / S)
-// and writes its partial sums to part[s][j][k] (weights) and part[S * 64 * kF +
-// s * 64 + j] (biases); k_fc1_sum adds the slices in a fixed order.
-__global__ void __launch_bounds__(256) k_fc1_dw(const float* __restrict__ g4,
-                                                const __nv_bfloat16* __restrict__ a3g, uint32_t n,
-                                                float* __restrict__ part) {
-  __shared__ __align__(16) float Gs[32][kHid];
-  __shared__ float Fs[32][33];
-  const int t = threadIdx.x, jq = t & 15, kp = t >> 4;
-  const int k0 = blockIdx.x * 32;
+__global__ void __launch_bounds__(kDwThreads, 2) k_fc1_dw(const float* __restrict__ g4,
+                                                          const __nv_bfloat16* __restrict__ a3g, uint32_t n,
+                                                          float* __restrict__ part, uint32_t* __restrict__ status) {
+  extern __shared__ __align__(1024) unsigned char smd[];
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smd + 2 * kDwStage);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 2);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t S = gridDim.y, s = blockIdx.y;
   const uint32_t lo = (uint32_t)((uint64_t)n * s / S), hi = (uint32_t)((uint64_t)n * (s + 1) / S);
-  float* pw = part + (size_t)s * kHid * kF;                 // [j][k] of this slice
-  float* pb = part + (size_t)S * kHid * kF + (size_t)s * kHid;  // [j] of this slice
-  float acc[4][2] = {}, accb[4] = {};
-  for (uint32_t b0 = lo; b0 < hi; b0 += 32) {
-    for (int i = t; i < 32 * kHid; i += 256) {
-      const uint32_t b = b0 + i / kHid;
-      Gs[i / kHid][i % kHid] = b < hi ? g4[(size_t)b * kHid + i % kHid] : 0.f;
-    }
-    for (int i = t; i < 32 * 32; i += 256) {
-      const uint32_t b = b0 + i / 32;
-      const int k = k0 + i % 32;
-      Fs[i / 32][i % 32] = (b < hi && k < kF) ? ld(a3g + (size_t)b * kF + k) : 0.f;
-    }
-    __syncthreads();
-    for (int bb = 0; bb < 32; ++bb) {
-      const float4 g = *reinterpret_cast<const float4*>(&Gs[bb][jq * 4]);
-      const float f0 = Fs[bb][kp * 2], f1 = Fs[bb][kp * 2 + 1];
-      acc[0][0] = fmaf(g.x, f0, acc[0][0]); acc[0][1] = fmaf(g.x, f1, acc[0][1]);
-      acc[1][0] = fmaf(g.y, f0, acc[1][0]); acc[1][1] = fmaf(g.y, f1, acc[1][1]);
-      acc[2][0] = fmaf(g.z, f0, acc[2][0]); acc[2][1] = fmaf(g.z, f1, acc[2][1]);
-      acc[3][0] = fmaf(g.w, f0, acc[3][0]); acc[3][1] = fmaf(g.w, f1, acc[3][1]);
-      accb[0] += g.x; accb[1] += g.y; accb[2] += g.z; accb[3] += g.w;
-    }
-    __syncthreads();
+  const int k0 = blockIdx.x * kDwCols;
+  if (warp == 0) tc::tmem_alloc(tslot, 256);
+  if (tid == 0) {
+    tc::mbar_init(bar, 1);
+    tc::mbar_init(bar + 1, 1);
   }
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tmem = *tslot;
+  const int jc = tid & 7;  // this thread's chunk of 8 hidden units
+  float accb[8];
 #pragma unroll
-  for (int jj = 0; jj < 4; ++jj) {
-    const int j = jq * 4 + jj;
-#pragma unroll
-    for (int kk = 0; kk < 2; ++kk) {
-      const int k = k0 + kp * 2 + kk;
-      if (k < kF) pw[(size_t)j * kF + k] = acc[jj][kk];
+  for (int j = 0; j < 8; ++j) accb[j] = 0.f;
+  uint32_t ph = 0;  // bit st: parity of stage st's next wait
+  bool ok = true;
+  int l = 0;
+  for (uint32_t c0 = lo; c0 < hi; c0 += kDwChunk, ++l) {
+    const int st = l & 1;
+    unsigned char* A = smd + st * kDwStage;
+    unsigned char* B = A + kDwA;
+    if (l >= 2) {
+      ok = tc::mbar_wait(bar + st, (ph >> st) & 1u, 1u << 22);
+      ph ^= 1u << st;
+      if (__syncthreads_or(!ok)) {
+        ok = false;
+        break;
+      }
     }
-    if (blockIdx.x == 0 && kp == 0) pb[j] = accb[jj];
+    for (int i = tid; i < (kDwCols / 8) * kDwChunk; i += kDwThreads) {
+      const int c = i & 15, r = i >> 4;
+      const bool in = c0 + r < hi && k0 + 8 * c < kF;
+      tc::cp16(A + (c * kDwChunk + r) * 16, a3g + (in ? (size_t)(c0 + r) * kF + k0 + 8 * c : 0), in);
+    }
+    tc::cp_commit();
+#pragma unroll
+    for (int i = 0; i < kDwChunk * 8 / kDwThreads; ++i) {
+      const int r = (tid + i * kDwThreads) >> 3;
+      float4 v0 = make_float4(0.f, 0.f, 0.f, 0.f), v1 = v0;
+      if (c0 + r < hi) {
+        const float4* src = reinterpret_cast<const float4*>(g4 + (size_t)(c0 + r) * kHid + jc * 8);
+        v0 = src[0];
+        v1 = src[1];
+      }
+      const float v[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+      uint32_t pk[3][4];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        uint16_t p[3];
+        tc::split_fp32(v[j], p[0], p[1], p[2]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) pk[k][j / 2] = (j & 1) ? pk[k][j / 2] | ((uint32_t)p[k] << 16) : (uint32_t)p[k];
+        accb[j] += v[j];
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+        reinterpret_cast<uint4*>(B)[(k * 8 + jc) * kDwChunk + r] = make_uint4(pk[k][0], pk[k][1], pk[k][2], pk[k][3]);
+    }
+    tc::cp_wait<0>();
+    tc::fence_smem_to_async();
+    tc::fence_before_sync();
+    __syncthreads();
+    if (tid == 0) {
+      tc::fence_after_sync();
+      const uint32_t a0 = tc::smem_u32(A), b0 = tc::smem_u32(B);
+      constexpr uint32_t id = tc::idesc_bf16_mn(128, 192);
+#pragma unroll
+      for (int k = 0; k < kDwChunk / 16; ++k)
+        tc::mma_bf16(tmem, tc::smem_desc_strided(a0 + (uint32_t)(16 * k) * 16u, 128u, kDwChunk * 16u),
+                     tc::smem_desc_strided(b0 + (uint32_t)(16 * k) * 16u, 128u, kDwChunk * 16u), id, (l | k) != 0);
+      tc::commit(bar + st);
+    }
   }
+  for (int st = 0; st < 2 && ok; ++st)
+    if (l > st) ok = tc::mbar_wait(bar + st, (ph >> st) & 1u, 1u << 22);
+  if (__syncthreads_or(!ok)) ok = false;
+  if (!ok) {
+    if (tid == 0) atomicOr(status, 1u);
+  } else {
+    tc::fence_after_sync();
+    const int q = warp & 3, h = warp >> 2;  // lane quadrant, half of the hidden units
+    const int k = k0 + q * 32 + lane;
+    float* pw = part + (size_t)s * kHid * kF;
+#pragma unroll
+    for (int jj = 0; jj < 32; jj += 16) {
+      float v[3][16];
+#pragma unroll
+      for (int p = 0; p < 3; ++p)
+        tc::ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(p * kHid + h * 32 + jj), v[p]);
+      if (k < kF) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          pw[(size_t)(h * 32 + jj + j) * kF + k] = hi > lo ? (v[0][j] + v[1][j]) + v[2][j] : 0.f;
+      }
+    }
+    if (blockIdx.x == 0) {
+      float* red = reinterpret_cast<float*>(smd);  // [8 j][256]: the MMAs are done
+#pragma unroll
+      for (int j = 0; j < 8; ++j) red[j * kDwThreads + tid] = accb[j];
+      __syncthreads();
+      if (tid < kHid) {
+        float v = 0.f;
+        for (int r = 0; r < kDwThreads / 8; ++r) v += red[(tid & 7) * kDwThreads + r * 8 + (tid >> 3)];
+        part[(size_t)S * kHid * kF + (size_t)s * kHid + tid] = v;
+      }
+    }
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == 0) tc::tmem_free(tmem, 256);
 }
 
-// grad[fc1.w] and grad[fc1.b]: the S slices of k_fc1_dw added in slice order.
-__global__ void k_fc1_sum(const float* __restrict__ part, uint32_t S, float* __restrict__ grad) {
+// grad[fc1.w] and grad[fc1.b]: the S slices of k_fc1_dw added in slice order; the
+// last block adds k_loss's blocks: grad[fc2] and the mean loss.
+__global__ void k_fc1_sum(const float* __restrict__ part, uint32_t S, const float* __restrict__ lpart, uint32_t n_loss,
+                          uint32_t n, float* __restrict__ grad, float* __restrict__ loss) {
+  if (blockIdx.x == gridDim.x - 1) {
+    const uint32_t t = threadIdx.x;
+    if (t >= kLossOut) return;
+    float v = 0.f;
+#pragma unroll 8
+    for (uint32_t b = 0; b < n_loss; ++b) v += lpart[(size_t)b * kLossOut + t];
+    if (t < kHid + 1)
+      grad[(t < kHid ? kWf2 + t : kBf2)] = v;
+    else
+      *loss = v * (1.f / (float)n);
+    return;
+  }
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < (uint32_t)(kHid * kF)) {
     float v = 0.f;
+#pragma unroll 4
     for (uint32_t s = 0; s < S; ++s) v += part[(size_t)s * kHid * kF + i];
     grad[kWf1 + i] = v;
   } else if (i < (uint32_t)(kHid * kF + kHid)) {
@@ -625,8 +743,8 @@ __global__ void __launch_bounds__(kBcThreads, 2) k_conv_back_tc(
   }
   for (int i = tid; i < L::kSmW / 16; i += kBcThreads) reinterpret_cast<uint4*>(smb)[i] = make_uint4(0, 0, 0, 0);
   for (int i = tid; i < 9 * C * C; i += kBcThreads) {  // dX's B operand per tap: B_t[c][o] = w[o][c][t]
-    const int t = i / (C * C), c = (i / C) % C, o = i % C;
-    *reinterpret_cast<__nv_bfloat16*>(Wb + t * C * C * 2 + tc::cm_offset(c, o, 4)) = w[(o * C + c) * 9 + t];
+    const int o = i / (9 * C), c = (i / 9) % C, t = i % 9;
+    *reinterpret_cast<__nv_bfloat16*>(Wb + t * C * C * 2 + tc::cm_offset(c, o, 4)) = w[i];
   }
   tc::fence_before_sync();
   __syncthreads();
@@ -941,26 +1059,31 @@ __global__ void __launch_bounds__(kBcThreads, 2) k_conv1_dw_tc(const float* __re
   if (warp == 0) tc::tmem_free(tmem, 256);
 }
 
-// grad[w_off + i] = sum over blocks and parts of the partial weight sums;
-// grad[b_off + o] likewise for the biases.  Fixed summation order.
-// One warp per element: lane l adds blocks l, l + 32, ... in order, then the
-// lanes combine in a fixed xor pattern.
-__global__ void k_reduce_partials(const float* __restrict__ partial, int n_blocks, int parts, int nw,
-                                  float* __restrict__ grad, int w_off, int b_off) {
-  const int i = (int)((blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (i >= nw + kCh) return;  // whole warps leave together
+// The conv layers' gradients from their blocks' partial sums (weights, then
+// biases: rows of kPartialStride per block, layer l at l * kBackBlocks rows).  Blocks
+// of 32 elements x 8 groups of rows: a row's 32 elements are read together, each
+// group adds its rows in order, the groups are added in order.  (A warp per element,
+// its lanes over the rows, read a sector for every value: 19 us a layer.)
+__global__ void __launch_bounds__(256) k_reduce_partials(const float* __restrict__ partial, int n_blocks,
+                                                         float* __restrict__ grad) {
+  __shared__ float red[8][32];
+  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5, l = blockIdx.y;  // l: conv1, conv2, conv3
+  const int nw = l == 0 ? kCh * kQ * 9 : kCh * kCh * 9, i = blockIdx.x * 32 + lane;
+  const float* p = partial + (size_t)l * kBackBlocks * kPartialStride + i;
   float s = 0.f;
-  for (int blk = lane; blk < n_blocks; blk += 32) {
-    const float* p = partial + (size_t)blk * kPartialStride;
-    if (i < nw) {
-      for (int q = 0; q < parts; ++q) s += p[(size_t)q * nw + i];
-    } else {
-      s += p[(size_t)parts * nw + (i - nw)];
-    }
+  if (i < nw + kCh) {
+    const int r0 = n_blocks * grp / 8, r1 = n_blocks * (grp + 1) / 8;
+#pragma unroll 8
+    for (int r = r0; r < r1; ++r) s += p[(size_t)r * kPartialStride];
   }
+  red[grp][lane] = s;
+  __syncthreads();
+  if (grp == 0 && i < nw + kCh) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) grad[i < nw ? w_off + i : b_off + (i - nw)] = s;
+    for (int g = 1; g < 8; ++g) s += red[g][lane];
+    const int w_off = l == 0 ? kW1 : l == 1 ? kW2 : kW3, b_off = l == 0 ? kB1 : l == 1 ? kB2 : kB3;
+    grad[i < nw ? w_off + i : b_off + (i - nw)] = s;
+  }
 }
 
 // ---- parameters --------------------------------------------------------------
@@ -1002,6 +1125,8 @@ cudaError_t set_attrs() {
     e = cudaFuncSetAttribute(k_conv_back_tc<kH1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              ConvBack<kH1>::kSmem);
   if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_fc1_dw, cudaFuncAttributeMaxDynamicSharedMemorySize, kDwSmem);
+  if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_conv1_dw_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kC1Smem);
   if (e == cudaSuccess) done = true;
   return e;
@@ -1028,7 +1153,7 @@ cudaError_t forward(sas_vet* vt, const uint16_t* stamps, const uint32_t* idx, ui
   const uint32_t tiles = (n + kFcTcRows - 1) / kFcTcRows, ldp = tiles * kFcTcRows;
   k_fc_fwd_tc<<<dim3(tiles, kFcSplit), kFcTcThreads, kFcTcSmem, s>>>(vt->a3, n, vt->wb, vt->fcpart, ldp,
                                                                      vt->status);
-  k_fc_epi<<<(n + 255) / 256, 256, 0, s>>>(vt->fcpart, ldp, n, vt->wb, keep ? vt->a4 : nullptr, logits);
+  k_fc_epi<<<(n + 31) / 32, 256, 0, s>>>(vt->fcpart, ldp, n, vt->wb, keep ? vt->a4 : nullptr, logits);
   note_launch();
   note_launch(2);
   return cudaGetLastError();
@@ -1038,29 +1163,22 @@ cudaError_t gradients(sas_vet* vt, const uint16_t* stamps, const float* labels, 
                       uint32_t n, float* grad, cudaStream_t s) {
   cudaError_t e = forward(vt, stamps, idx, n, true, vt->logits, s);
   if (e != cudaSuccess) return e;
-  k_loss<<<1, kLossThreads, 0, s>>>(vt->logits, labels, idx, n, vt->a4, vt->glogit, grad, vt->loss);
-  k_g4<<<(unsigned)(((uint64_t)n * kHid + 255) / 256), 256, 0, s>>>(vt->glogit, vt->a4, vt->wb, n, vt->g4);
-  {
-    // stamp slices of about 512 (at most the partial buffer's room), summed in order
-    const uint32_t S = std::max<uint32_t>(1, std::min<uint32_t>(kFc1Slices, n / 512));
-    k_fc1_dw<<<dim3((kF + 31) / 32, S), 256, 0, s>>>(vt->g4, vt->a3, n, vt->partial);
-    k_fc1_sum<<<(kHid * kF + kHid + 255) / 256, 256, 0, s>>>(vt->partial, S, grad);
-    note_launch();
-  }
+  const uint32_t n_loss = (n + kLossStamps - 1) / kLossStamps;
+  k_loss<<<n_loss, 256, 0, s>>>(vt->logits, labels, idx, n, vt->a4, vt->wb, vt->g4, vt->lpart);
+  // stamp slices: enough blocks for two per SM, at least one chunk each
+  const uint32_t S = std::max<uint32_t>(1, std::min<uint32_t>(kFc1Slices, n / kDwChunk));
+  k_fc1_dw<<<dim3(kDwTiles, S), kDwThreads, kDwSmem, s>>>(vt->g4, vt->a3, n, vt->partial, vt->status);
+  k_fc1_sum<<<(kHid * kF + kHid + 255) / 256 + 1, 256, 0, s>>>(vt->partial, S, vt->lpart, n_loss, n, grad, vt->loss);
   k_fc1_dx<<<dim3((kF + 63) / 64, (n + 31) / 32), 256, 0, s>>>(vt->g4, vt->wb, vt->a3, n, vt->g3);
   const int nb = (int)std::min<uint32_t>(n, kBackBlocks);
+  const size_t per = (size_t)kBackBlocks * kPartialStride;
   k_conv_back_tc<kH2><<<nb, kBcThreads, ConvBack<kH2>::kSmem, s>>>(vt->g3, vt->a2, n, vt->wb + kW3, vt->g2,
-                                                                   vt->partial, vt->status);
-  k_reduce_partials<<<(kCh * kCh * 9 + kCh + 7) / 8, 256, 0, s>>>(vt->partial, nb, 1, kCh * kCh * 9,
-                                                                      grad, kW3, kB3);
+                                                                 vt->partial + 2 * per, vt->status);
   k_conv_back_tc<kH1><<<nb, kBcThreads, ConvBack<kH1>::kSmem, s>>>(vt->g2, vt->a1, n, vt->wb + kW2, vt->g1,
-                                                                   vt->partial, vt->status);
-  k_reduce_partials<<<(kCh * kCh * 9 + kCh + 7) / 8, 256, 0, s>>>(vt->partial, nb, 1, kCh * kCh * 9,
-                                                                      grad, kW2, kB2);
+                                                                 vt->partial + per, vt->status);
   k_conv1_dw_tc<<<nb, kBcThreads, kC1Smem, s>>>(vt->g1, stamps, idx, n, vt->partial, vt->status);
-  k_reduce_partials<<<(kCh * kQ * 9 + kCh + 7) / 8, 256, 0, s>>>(
-      vt->partial, nb, 1, kCh * kQ * 9, grad, kW1, kB1);
-  note_launch(10);
+  k_reduce_partials<<<dim3((kCh * kCh * 9 + kCh + 31) / 32, 3), 256, 0, s>>>(vt->partial, nb, grad);
+  note_launch(8);
   return cudaGetLastError();
 }
 
@@ -1112,7 +1230,7 @@ int cuda_fail(cudaError_t e, const char* what) {
 
 void free_vet(sas_vet* vt) {
   void* ptrs[] = {vt->master, vt->m, vt->v, vt->grad, vt->wb, vt->a1, vt->a2, vt->a3,
-                  vt->a4, vt->logits, vt->glogit, vt->g4, vt->g3, vt->g2, vt->g1, vt->partial, vt->loss,
+                  vt->a4, vt->logits, vt->lpart, vt->g4, vt->g3, vt->g2, vt->g1, vt->partial, vt->loss,
                   vt->status, vt->fcpart};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -1148,9 +1266,9 @@ int sas_vet_create(int device, uint32_t max_batch, sas_vet** out) {
       {(void**)&vt->grad, N * 4}, {(void**)&vt->wb, N * 2},
       {(void**)&vt->a1, B * vet::kCh * vet::kH1 * vet::kH1 * 2}, {(void**)&vt->a2, B * vet::kCh * vet::kH2 * vet::kH2 * 2},
       {(void**)&vt->a3, B * vet::kF * 2}, {(void**)&vt->a4, B * vet::kHid * 2}, {(void**)&vt->logits, B * 4},
-      {(void**)&vt->glogit, B * 4}, {(void**)&vt->g4, B * vet::kHid * 4}, {(void**)&vt->g3, B * vet::kF * 4},
+      {(void**)&vt->lpart, (B + vet::kLossStamps - 1) / vet::kLossStamps * vet::kLossOut * 4}, {(void**)&vt->g4, B * vet::kHid * 4}, {(void**)&vt->g3, B * vet::kF * 4},
       {(void**)&vt->g2, B * vet::kCh * vet::kH2 * vet::kH2 * 4}, {(void**)&vt->g1, B * vet::kCh * vet::kH1 * vet::kH1 * 4},
-      {(void**)&vt->partial, (size_t)vet::kBackBlocks * vet::kPartialStride * 4}, {(void**)&vt->loss, 4},
+      {(void**)&vt->partial, (size_t)3 * vet::kBackBlocks * vet::kPartialStride * 4}, {(void**)&vt->loss, 4},
       {(void**)&vt->status, 4},
       {(void**)&vt->fcpart, (size_t)vet::kFcSplit * vet::kHid * ((B + 127) / 128 * 128) * 4},
   };

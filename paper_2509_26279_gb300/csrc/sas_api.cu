@@ -6,6 +6,7 @@
 #include <cstdlib>
 #include <cmath>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -25,6 +26,8 @@ struct sas_grid {
 
 struct sas_result {
   int device;
+  void* d_mem;        // one allocation: the bucketed catalog and tables below
+  void* d_out;        // one allocation: candidates and ids (null in a cluster list)
   sas_candidate* d_cands;
   uint32_t* d_ids;
   sas_result_info info;
@@ -92,6 +95,31 @@ struct Scratch {
     *p = static_cast<T*>(q);
     return cudaSuccess;
   }
+};
+
+// Several arrays in one allocation: add() them, allocate `size` bytes, place() them.
+struct Arena {
+  size_t size = 0;
+  struct Part {
+    void** p;
+    size_t at;
+  };
+  std::vector<Part> parts;
+  template <typename T>
+  void add(T** p, size_t count) {
+    parts.push_back({(void**)p, size});
+    size += (std::max<size_t>(count, 1) * sizeof(T) + 255) & ~size_t(255);
+  }
+  void place(char* base) {
+    for (const Part& q : parts) *q.p = base + q.at;
+  }
+};
+
+// What the kernels of a search report, in one block so that one copy reads it.
+struct Counters {
+  uint32_t flags, n_emit, n_valid, pad;
+  unsigned long long pairs, tile, raw, balance, pairs1, n_ids;  // pairs1: of the window search's first level
+  long long t0;
 };
 
 bool fits_i32(int64_t v) { return v >= INT32_MIN && v <= INT32_MAX; }
@@ -304,144 +332,157 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
     const int32_t* dx = cat->x;
     const int32_t* dy = cat->y;
     const uint16_t* dep = cat->epoch;
-    int32_t *hx = nullptr, *hy = nullptr;
-    uint16_t* hep = nullptr;
-    int64_t *d_t = nullptr, *d_dt = nullptr, *d_t0 = nullptr;  // d_dt is kept by the result
-    const uint8_t* d_w = nullptr;
-    uint8_t* hw_dev = nullptr;
-    uint32_t *d_ecount = nullptr, *d_bcount = nullptr, *d_boff = nullptr, *d_cursor = nullptr,
-             *d_bof = nullptr, *d_scan = nullptr;
-    Det* d_dets = nullptr;
-    int32_t *d_sxt = nullptr, *d_syt = nullptr;
-    uint32_t* d_small = nullptr;  // [0] flags [1] n_emit [2] n_valid
-    unsigned long long* d_small64 = nullptr;  // [0] pairs [1] tile counter [2] raw total [3] balance [4] level-1 pairs
-    Emit* d_emits = nullptr;
-    Key* d_keys = nullptr;
-    uint32_t* d_raw = nullptr;
-    unsigned long long *d_idoff = nullptr, *d_scan64 = nullptr;
-    uint32_t* d_ids_tmp = nullptr;
+    const uint8_t* d_w = weights;
+    const bool host = !cat->on_device;
     const uint32_t hint = grid->emit_hint.load(std::memory_order_relaxed);
     uint32_t emit_cap = (uint32_t)std::min<uint64_t>(
         std::max<uint64_t>({(uint64_t)1 << 16, 2 * n, (uint64_t)hint + hint / 4 + 1024}), (uint64_t)1 << 26);
-    uint32_t h_small[3] = {0, 0, 0};
-    unsigned long long h_small64[4] = {0, 0, 0, 0};
-    int64_t h_t0 = 0;
+    if (use_win) emit_cap = std::max(wplan.list_cap, hint + hint / 4);
+    uint32_t key_cap = use_win ? 1u << 17 : 0;
+    const size_t npts = use_win && wplan.masked ? ((size_t)d.nvx + 1) * ((size_t)d.nvy + 1) : 0;
+    const size_t nK = use_win ? (size_t)wplan.g.nvx * wplan.g.nvy : 0;
+    Counters h{};
     uint32_t n_out = 0;
-    unsigned long long n_ids = 0;
     StackArgs sa{};
     WindowArgs wa{};
-    uint64_t n_keys = 0;
+    Key* sorted = nullptr;
+    unsigned long long *d_idoff = nullptr, *d_scan64 = nullptr;
+    uint32_t* d_ids_tmp = nullptr;
 
-    if (!cat->on_device) {
-      CK(sc.alloc(&hx, n), "alloc x");
-      CK(sc.alloc(&hy, n), "alloc y");
-      CK(sc.alloc(&hep, n), "alloc epoch");
+    // Two allocations up to the stack kernel: scratch, and what the result keeps.
+    Counters* d_cnt = nullptr;
+    int32_t *hx = nullptr, *hy = nullptr;
+    uint16_t* hep = nullptr;
+    uint8_t* hw = nullptr;
+    int64_t* d_t = nullptr;
+    uint32_t *d_bcount = nullptr, *d_cursor = nullptr, *d_bof = nullptr, *d_scan = nullptr;
+    uint32_t *d_ecount = nullptr, *d_boff = nullptr;  // kept by the result, as are the next three
+    Det* d_dets = nullptr;
+    int32_t *d_sxt = nullptr, *d_syt = nullptr;
+    Emit* d_emits = nullptr;
+    Key* d_keys = nullptr;
+    // Reads the counters back after the stack stage; the input errors of a search.
+    auto read_counters = [&]() -> cudaError_t {
+      cudaError_t e = cudaMemcpyAsync(&h, d_cnt, sizeof(h), cudaMemcpyDeviceToHost, s);
+      return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+    };
+    auto input_error = [&]() -> int {
+      if (h.flags & kFlagEpoch) return fail(SAS_ERR_RANGE, "an epoch index is >= n_epochs");
+      if (h.flags & kFlagPos) return fail(SAS_ERR_RANGE, "a detection has |x| or |y| >= 2^29");
+      if (h.flags & kFlagShift) return fail(SAS_ERR_RANGE, "a shift |v*(t-t0)/TPH| >= 2^28");
+      if (h.flags & kFlagInternal) return fail(SAS_ERR_INTERNAL, "stack kernel invariant");
+      return SAS_OK;
+    };
+    Arena scratch, keep;
+    scratch.add(&d_cnt, 1);  // the counters and the bucket counts start at zero: one memset
+    // nb grid buckets plus one overflow bucket (detections outside the grid)
+    scratch.add(&d_bcount, nb + 1);
+    const size_t zeroed = scratch.size;
+    scratch.add(&d_t, E);
+    scratch.add(&d_cursor, nb + 1);
+    scratch.add(&d_scan, scan_scratch_elems(nb + 1));
+    scratch.add(&d_bof, n);
+    if (host) {
+      scratch.add(&hx, n);
+      scratch.add(&hy, n);
+      scratch.add(&hep, n);
+      if (weights) scratch.add(&hw, n);
+    }
+    scratch.add(&d_emits, emit_cap);
+    if (use_win) {
+      scratch.add(&d_keys, key_cap);
+      scratch.add(&wa.sXt, (size_t)wplan.g.nvx * E);
+      scratch.add(&wa.sYt, (size_t)wplan.g.nvy * E);
+      scratch.add(&wa.mx, d.nvx);
+      scratch.add(&wa.my, d.nvy);
+      if (wplan.masked) {
+        scratch.add(&wa.vact, nK);
+        scratch.add(&wa.vsum, npts);
+      }
+    }
+    keep.add(&res->d_ecount, E);
+    keep.add(&res->d_dets, n);
+    keep.add(&res->d_boff, nb + 2);
+    keep.add(&res->d_sxt, (size_t)d.nvx * E);
+    keep.add(&res->d_syt, (size_t)d.nvy * E);
+    keep.add(&res->d_dt, E);
+    {
+      char* base = nullptr;
+      CK(sc.alloc(&base, scratch.size), "alloc scratch");
+      scratch.place(base);
+      CK(cudaMallocAsync(&res->d_mem, keep.size, s), "alloc result");
+      keep.place((char*)res->d_mem);
+      CK(cudaMemsetAsync(base, 0, zeroed, s), "memset");
+    }
+    d_ecount = res->d_ecount;
+    d_boff = res->d_boff;
+    d_dets = res->d_dets;
+    d_sxt = res->d_sxt;
+    d_syt = res->d_syt;
+    res->g = g;
+    res->cg = cg;
+    CK(cudaMemsetAsync(d_ecount, 0, E * 4, s), "memset");
+    if (host) {
       CK(cudaMemcpyAsync(hx, cat->x, n * 4, cudaMemcpyHostToDevice, s), "copy x");
       CK(cudaMemcpyAsync(hy, cat->y, n * 4, cudaMemcpyHostToDevice, s), "copy y");
       CK(cudaMemcpyAsync(hep, cat->epoch, n * 2, cudaMemcpyHostToDevice, s), "copy epoch");
       dx = hx; dy = hy; dep = hep;
-    }
-    if (weights) {
-      if (cat->on_device) {
-        d_w = weights;
-      } else {
-        CK(sc.alloc(&hw_dev, n), "alloc weights");
-        CK(cudaMemcpyAsync(hw_dev, weights, n, cudaMemcpyHostToDevice, s), "copy weights");
-        d_w = hw_dev;
+      if (weights) {
+        CK(cudaMemcpyAsync(hw, weights, n, cudaMemcpyHostToDevice, s), "copy weights");
+        d_w = hw;
       }
     }
-    CK(sc.alloc(&d_t, E), "alloc t");
-    CK(cudaMallocAsync((void**)&d_dt, (size_t)E * 8, s), "alloc dt");
-    res->d_dt = d_dt;
-    CK(sc.alloc(&d_t0, 1), "alloc t0");
     CK(cudaMemcpyAsync(d_t, cat->t, E * 8, cudaMemcpyHostToDevice, s), "copy t");
-    CK(cudaMallocAsync((void**)&d_ecount, (size_t)E * 4, s), "alloc ecount");
-    res->d_ecount = d_ecount;
-    // nb grid buckets plus one overflow bucket (detections outside the grid)
-    CK(sc.alloc(&d_bcount, nb + 1), "alloc bucket counts");
-    CK(cudaMallocAsync((void**)&d_boff, (nb + 2) * 4, s), "alloc bucket offsets");
-    res->d_boff = d_boff;
-    CK(sc.alloc(&d_cursor, nb + 1), "alloc cursor");
-    CK(sc.alloc(&d_scan, scan_scratch_elems(nb + 1)), "alloc scan scratch");
-    CK(sc.alloc(&d_bof, n), "alloc bucket_of");
-    CK(cudaMallocAsync((void**)&d_dets, n * sizeof(Det), s), "alloc dets");
-    res->d_dets = d_dets;
-    CK(cudaMallocAsync((void**)&d_sxt, (size_t)d.nvx * E * 4, s), "alloc sx table");
-    res->d_sxt = d_sxt;
-    CK(cudaMallocAsync((void**)&d_syt, (size_t)d.nvy * E * 4, s), "alloc sy table");
-    res->d_syt = d_syt;
-    res->g = g;
-    res->cg = cg;
-    CK(sc.alloc(&d_small, 4), "alloc counters");
-    CK(sc.alloc(&d_small64, 5), "alloc counters64");
-    CK(cudaMemsetAsync(d_ecount, 0, E * 4, s), "memset");
-    CK(cudaMemsetAsync(d_bcount, 0, (nb + 1) * 4, s), "memset");
-    CK(cudaMemsetAsync(d_small, 0, 16, s), "memset");
-    CK(cudaMemsetAsync(d_small64, 0, 40, s), "memset");
     tr.mark("allocated");
 
     // a1-a3: ingest and validate, bucket, reference epoch, shift tables
-    CK(launch_ingest(dx, dy, dep, n, E, cg, d_bcount, d_ecount, d_bof, &d_small[0], s), "ingest");
-    CK(launch_scan_u32(d_bcount, d_boff, nb + 1, d_scan, s), "bucket scan");
-    CK(cudaMemcpyAsync(d_cursor, d_boff, (nb + 1) * 4, cudaMemcpyDeviceToDevice, s), "cursor");
+    CK(launch_ingest(dx, dy, dep, n, E, cg, d_bcount, d_ecount, d_bof, &d_cnt->flags, s), "ingest");
+    CK(launch_scan_u32(d_bcount, d_boff, nb + 1, d_scan, s, d_cursor), "bucket scan");
     CK(launch_scatter(dx, dy, dep, n, d_bof, d_cursor, d_dets, s), "scatter");
-    CK(launch_epoch_setup(E, d_t, d_ecount, d_dt, d_t0, s), "epoch setup");
-    CK(launch_shift_tables(g, d_dt, d_ecount, d_sxt, d_syt, &d_small[0], s), "shift tables");
+    CK(launch_shift_tables(g, d_t, d_ecount, res->d_dt, (int64_t*)&d_cnt->t0, d_sxt, d_syt, &d_cnt->flags, s), "shift tables");
     tr.mark("prep launched");
+
+    sa.w = d_w;
+    sa.dets = d_dets;
+    sa.boff = d_boff;
+    sa.ecount = d_ecount;
+    sa.n_emit = &d_cnt->n_emit;
+    sa.balance = &d_cnt->balance;
+    sa.flags = &d_cnt->flags;
+    sa.tile_counter = &d_cnt->tile;
 
     if (use_win) {  // a4-a7 in two levels: windows of groups of velocities, then their bins
       const TileCfg& tc = wplan.tc;
-      const SearchGeom& c = wplan.g;
-      const uint32_t list_cap = std::max(wplan.list_cap, hint + hint / 4);
-      uint32_t key_cap = 1u << 17;
-      CK(sc.alloc(&d_emits, list_cap), "alloc windows");
-      CK(sc.alloc(&d_keys, key_cap), "alloc keys");
       wa.gx = wplan.gx;
       wa.gy = wplan.gy;
       wa.win = wplan.win;
       wa.unit = wplan.unit;
       wa.g = g;
-      wa.cgm = c;
+      wa.cgm = wplan.g;
       wa.cg = cg;
       wa.dets = d_dets;
       wa.boff = d_boff;
       wa.ecount = d_ecount;
-      wa.dt = d_dt;
+      wa.dt = res->d_dt;
       wa.sxt = d_sxt;
       wa.syt = d_syt;
-      CK(sc.alloc(&wa.sXt, (size_t)c.nvx * E), "alloc group shifts");
-      CK(sc.alloc(&wa.sYt, (size_t)c.nvy * E), "alloc group shifts");
-      CK(sc.alloc(&wa.mx, d.nvx), "alloc shift bounds");
-      CK(sc.alloc(&wa.my, d.nvy), "alloc shift bounds");
-      if (wplan.masked) {
-        CK(sc.alloc(&wa.vact, (size_t)c.nvx * c.nvy), "alloc active groups");
-        CK(sc.alloc(&wa.vsum, ((size_t)d.nvx + 1) * ((size_t)d.nvy + 1)), "alloc point counts");
-      }
       wa.wts = d_w;
       wa.windows = d_emits;
-      wa.n_windows = &d_small[1];
-      wa.list_cap = list_cap;
+      wa.n_windows = &d_cnt->n_emit;
+      wa.list_cap = emit_cap;
       wa.n_min = n_min;
-      wa.n_valid = &d_small[2];
-      wa.raw_total = &d_small64[2];
-      wa.n_pairs = &d_small64[0];
-      wa.flags = &d_small[0];
+      wa.n_valid = &d_cnt->n_valid;
+      wa.raw_total = &d_cnt->raw;
+      wa.n_pairs = &d_cnt->pairs;
+      wa.flags = &d_cnt->flags;
       CK(stack_set_smem_attr_windows(tc.kx, tc.ky, tc.cb, tc.smem), "smem attribute");
       fill_window_args(wplan, n_min, (uint32_t)(v_begin / d.nvx), (uint32_t)((v_end - 1) / d.nvx), &sa);
       sa.vact = wa.vact;
-      sa.w = d_w;
-      sa.dets = d_dets;
-      sa.boff = d_boff;
-      sa.ecount = d_ecount;
       sa.sxt = wa.sXt;
       sa.syt = wa.sYt;
       sa.emits = d_emits;
-      sa.emit_cap = list_cap;
-      sa.n_emit = &d_small[1];
-      sa.n_pairs = &d_small64[4];
-      sa.balance = &d_small64[3];
-      sa.flags = &d_small[0];
-      sa.tile_counter = &d_small64[1];
+      sa.emit_cap = emit_cap;
+      sa.n_pairs = &d_cnt->pairs1;
       cudaEventRecord(evs0, s);
       CK(launch_window_tables(wa, s), "group tables");
       CK(launch_window_pairs(wa, dx, dy, dep, n, s), "pair count");
@@ -452,142 +493,112 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
         wa.key_cap = key_cap;
         CK(launch_window_cells(wa, di.sms, s), "window cells");
         cudaEventRecord(evs1, s);
-        CK(cudaMemcpyAsync(h_small, d_small, 12, cudaMemcpyDeviceToHost, s), "read counters");
-        CK(cudaMemcpyAsync(h_small64, d_small64, 32, cudaMemcpyDeviceToHost, s), "read counters");
-        CK(cudaMemcpyAsync(&h_t0, d_t0, 8, cudaMemcpyDeviceToHost, s), "read t0");
-        CK(cudaStreamSynchronize(s), "stack sync");
+        CK(read_counters(), "stack sync");
         tr.mark("windows done");
-        if (h_small[0] & kFlagEpoch) { rc = fail(SAS_ERR_RANGE, "an epoch index is >= n_epochs"); goto done; }
-        if (h_small[0] & kFlagPos) { rc = fail(SAS_ERR_RANGE, "a detection has |x| or |y| >= 2^29"); goto done; }
-        if (h_small[0] & kFlagShift) { rc = fail(SAS_ERR_RANGE, "a shift |v*(t-t0)/TPH| >= 2^28"); goto done; }
-        if (h_small[0] & kFlagInternal) { rc = fail(SAS_ERR_INTERNAL, "stack kernel invariant"); goto done; }
-        if ((h_small[0] & (kFlagWindow | kFlagEmitCap)) || h_small64[3] != 0 || h_small[1] > list_cap) {
+        if ((rc = input_error())) goto done;
+        if ((h.flags & (kFlagWindow | kFlagEmitCap)) || h.balance != 0 || h.n_emit > emit_cap) {
           without = true;
           rc = SAS_ERR_INTERNAL;
           goto done;
         }
-        if (h_small[2] <= key_cap) break;
-        key_cap = h_small[2];
+        if (h.n_valid <= key_cap) break;
+        key_cap = h.n_valid;
         if (key_cap >= (1u << 30)) { rc = fail(SAS_ERR_OOM, "too many candidate bins; raise n_min"); goto done; }
         CK(sc.alloc(&d_keys, key_cap), "alloc keys");
-        CK(cudaMemsetAsync(&d_small[2], 0, 4, s), "memset");
-        CK(cudaMemsetAsync(&d_small64[2], 0, 8, s), "memset");
+        CK(cudaMemsetAsync(&d_cnt->n_valid, 0, 4, s), "memset");
+        CK(cudaMemsetAsync(&d_cnt->raw, 0, 8, s), "memset");
       }
-      n_keys = key_cap;
+      cudaEventRecord(evc0, s);
     }
 
     // a4-a6: the stack kernel; reruns (exact) with wider counters if one wrapped
     // or with a longer emission list if it overflowed.
     for (int attempt = 0; !use_win; ++attempt) {
       const TileCfg& tc = plan.tc;
-      CK(sc.alloc(&d_emits, emit_cap), "alloc emissions");
-      CK(stack_set_smem_attr(tc.kx, tc.ky, tc.cb, tc.smem), "smem attribute");
       fill_stack_args(plan, n_min, n_low, o.peaks_only, &sa);
-      sa.w = d_w;
-      sa.dets = d_dets;
-      sa.boff = d_boff;
-      sa.ecount = d_ecount;
+      CK(stack_set_smem_attr(tc.kx, tc.ky, tc.cb, tc.smem, sa.select != kSelectAll), "smem attribute");
       sa.sxt = d_sxt;
       sa.syt = d_syt;
       sa.emits = d_emits;
       sa.emit_cap = emit_cap;
-      sa.n_emit = &d_small[1];
-      sa.n_pairs = &d_small64[0];
-      sa.balance = &d_small64[3];
-      sa.flags = &d_small[0];
-      sa.tile_counter = &d_small64[1];
-      CK(cudaMemsetAsync(&d_small[1], 0, 4, s), "memset");
-      CK(cudaMemsetAsync(d_small64, 0, 16, s), "memset");
-      CK(cudaMemsetAsync(&d_small64[3], 0, 8, s), "memset");
+      sa.n_pairs = &d_cnt->pairs;
+      if (attempt > 0) {  // all but t0 starts again
+        CK(cudaMemsetAsync(d_cnt, 0, offsetof(Counters, t0), s), "memset");
+      }
       const int grid_sz = (int)std::min<uint64_t>((uint64_t)di.sms, std::max<uint64_t>(sa.n_tiles, 1));
       cudaEventRecord(evs0, s);
       tr.mark("stack configured");
       CK(launch_stack(sa, grid_sz, s), "stack kernel");
       cudaEventRecord(evs1, s);
       tr.mark("stack launched");
-      CK(cudaMemcpyAsync(h_small, d_small, 12, cudaMemcpyDeviceToHost, s), "read counters");
-      CK(cudaMemcpyAsync(h_small64, d_small64, 32, cudaMemcpyDeviceToHost, s), "read counters");
-      CK(cudaMemcpyAsync(&h_t0, d_t0, 8, cudaMemcpyDeviceToHost, s), "read t0");
-      CK(cudaStreamSynchronize(s), "stack sync");
+      CK(read_counters(), "stack sync");
       tr.mark("stack done");
-      if (h_small[0] & kFlagEpoch) { rc = fail(SAS_ERR_RANGE, "an epoch index is >= n_epochs"); goto done; }
-      if (h_small[0] & kFlagPos) { rc = fail(SAS_ERR_RANGE, "a detection has |x| or |y| >= 2^29"); goto done; }
-      if (h_small[0] & kFlagShift) { rc = fail(SAS_ERR_RANGE, "a shift |v*(t-t0)/TPH| >= 2^28"); goto done; }
-      if (h_small[0] & kFlagInternal) { rc = fail(SAS_ERR_INTERNAL, "stack kernel invariant"); goto done; }
+      if ((rc = input_error())) goto done;
       if (attempt >= 4) { rc = fail(SAS_ERR_INTERNAL, "stack kernel did not converge"); goto done; }
-      if ((h_small[0] & kFlagCounter) || h_small64[3] != 0) {  // a counter wrapped
-        CK(cudaMemsetAsync(&d_small[0], 0, 4, s), "memset");
+      if ((h.flags & kFlagCounter) || h.balance != 0) {  // a counter wrapped
         if (int r2 = replan_wider(d, n, n_min, op, di, &plan)) { rc = r2; goto done; }
         continue;
       }
-      if (h_small[1] > emit_cap || (h_small[0] & kFlagEmitCap)) {
-        if (h_small[1] >= (1u << 28)) {
+      if (h.n_emit > emit_cap || (h.flags & kFlagEmitCap)) {
+        if (h.n_emit >= (1u << 28)) {
           rc = fail(SAS_ERR_OOM, "more than 2^28 cells reach the threshold; raise n_min");
           goto done;
         }
-        CK(cudaMemsetAsync(&d_small[0], 0, 4, s), "memset");
-        emit_cap = h_small[1] + h_small[1] / 4 + 1024;
+        emit_cap = h.n_emit + h.n_emit / 4 + 1024;
+        CK(sc.alloc(&d_emits, emit_cap), "alloc emissions");
         continue;
       }
+      // a5/a7: exact distinct and raw counts of every bin of the emitted super-bins
+      const uint64_t n_keys = (uint64_t)h.n_emit * plan.tc.s * plan.tc.s;
+      if (n_keys >= (1ull << 31)) { rc = fail(SAS_ERR_OOM, "too many candidate bins; raise n_min"); goto done; }
+      CK(sc.alloc(&d_keys, n_keys), "alloc keys");
+      cudaEventRecord(evc0, s);
+      CK(launch_cell_count(d_emits, h.n_emit, plan.tc.s, g, cg, d_dets, d_boff, d_ecount, d_sxt,
+                           d_syt, n_min, sa.n_low, d_keys, &d_cnt->n_valid, &d_cnt->raw, d_w, s), "cell count");
+      if (h.n_emit) CK(read_counters(), "count sync");
+      tr.mark("counts done");
       break;
     }
     {
-      const uint32_t n_emit = h_small[1];
-      const_cast<sas_grid*>(grid)->emit_hint.store(n_emit, std::memory_order_relaxed);
-      cudaEventRecord(evc0, s);
-      if (!use_win) {
-      n_keys = (uint64_t)n_emit * plan.tc.s * plan.tc.s;
-      if (n_keys >= (1ull << 31)) { rc = fail(SAS_ERR_OOM, "too many candidate bins; raise n_min"); goto done; }
-      CK(sc.alloc(&d_keys, n_keys), "alloc keys");
-      // a5/a7: exact distinct and raw counts of every bin of the emitted super-bins
-      CK(launch_cell_count(d_emits, n_emit, plan.tc.s, g, cg, d_dets, d_boff, d_ecount, d_sxt,
-                           d_syt, n_min, sa.n_low, d_keys, &d_small[2], &d_small64[2], d_w, s), "cell count");
-      CK(cudaMemcpyAsync(&h_small[2], &d_small[2], 4, cudaMemcpyDeviceToHost, s), "read n_valid");
-      CK(cudaMemcpyAsync(&h_small64[2], &d_small64[2], 8, cudaMemcpyDeviceToHost, s), "read raw");
-      CK(cudaStreamSynchronize(s), "count sync");
-      tr.mark("counts done");
-      }
-      {  // a8: total order of the valid keys
-        const uint32_t n_valid = h_small[2];
-        uint32_t n_pad = 1;
-        while (n_pad < n_valid) n_pad <<= 1;
-        Key* sort_buf = d_keys;
-        if (n_pad > n_keys) {
-          CK(sc.alloc(&sort_buf, n_pad), "alloc sort buffer");
-          CK(cudaMemcpyAsync(sort_buf, d_keys, (size_t)n_valid * sizeof(Key), cudaMemcpyDeviceToDevice, s), "copy keys");
-        }
-        CK(launch_sort_keys(sort_buf, n_valid, n_pad, s), "sort");
-        d_keys = sort_buf;
-      }
-      cudaEventRecord(evc1, s);
-      n_out = h_small[2];
+      const_cast<sas_grid*>(grid)->emit_hint.store(h.n_emit, std::memory_order_relaxed);
+      // a8: total order of the valid keys; a7: candidates, contributing ids
+      const uint32_t n_emit = h.n_emit, n_valid = h.n_valid;
+      n_out = n_valid;
       if (o.max_candidates > 0 && n_out > o.max_candidates) n_out = (uint32_t)o.max_candidates;
-      const uint64_t id_cap = std::max<uint64_t>(h_small64[2], 1);
-      CK(sc.alloc(&d_raw, n_out), "alloc raw");
-      CK(sc.alloc(&d_idoff, (size_t)n_out + 1), "alloc id offsets");
-      CK(sc.alloc(&d_scan64, scan_scratch_elems(n_out)), "alloc scan scratch");
-      CK(sc.alloc(&d_ids_tmp, id_cap), "alloc ids");
-      CK(cudaMallocAsync((void**)&res->d_ids, id_cap * 4, s), "alloc result ids");
-      CK(cudaMallocAsync((void**)&res->d_cands, std::max<size_t>(n_out, 1) * sizeof(sas_candidate), s),
-         "alloc result candidates");
-      // a7: contributing ids, ascending per candidate
-      CK(launch_key_raw(d_keys, n_out, d_raw, s), "raw");
-      CK(launch_scan_u32_to_u64(d_raw, d_idoff, n_out, d_scan64, s), "id offsets");
-      CK(launch_gather_ids(d_keys, n_out, d_idoff, g, cg, d_dets, d_boff, d_ecount, d_sxt, d_syt,
-                           d_ids_tmp, res->d_ids, &d_small[0], s), "gather ids");
-      CK(launch_write_candidates(d_keys, n_out, d_idoff, res->d_cands, s), "write candidates");
-      CK(cudaMemcpyAsync(&n_ids, &d_idoff[n_out], 8, cudaMemcpyDeviceToHost, s), "read n_ids");
-      CK(cudaMemcpyAsync(&h_small[0], &d_small[0], 4, cudaMemcpyDeviceToHost, s), "read flags");
+      const uint64_t id_cap = std::max<uint64_t>(h.raw, 1);
+      uint32_t n_pad = 1;
+      while (n_pad < n_valid) n_pad <<= 1;
+      Arena post, mine;
+      if (!sort_in_place(n_valid)) post.add(&sorted, n_valid > kSortMerge ? n_pad : n_valid);
+      post.add(&d_idoff, (size_t)n_out + 1);
+      post.add(&d_scan64, candidates_scratch_elems(n_out));
+      post.add(&d_ids_tmp, id_cap);
+      mine.add(&res->d_cands, n_out);
+      mine.add(&res->d_ids, id_cap);
+      {
+        char* base = nullptr;
+        CK(sc.alloc(&base, post.size), "alloc ordering");
+        post.place(base);
+        CK(cudaMallocAsync(&res->d_out, mine.size, s), "alloc result candidates");
+        mine.place((char*)res->d_out);
+      }
+      if (!sorted) sorted = d_keys;
+      CK(launch_sort(d_keys, n_valid, sorted, s), "sort");
+      cudaEventRecord(evc1, s);
+      CK(launch_candidates(sorted, n_out, d_idoff, d_scan64, res->d_cands, &d_cnt->n_ids, s), "candidates");
+      CK(launch_gather_ids(sorted, n_out, d_idoff, g, cg, d_dets, d_boff, d_ecount, d_sxt, d_syt,
+                           d_ids_tmp, res->d_ids, &d_cnt->flags, s), "gather ids");
       cudaEventRecord(ev1, s);
-      CK(cudaStreamSynchronize(s), "final sync");
+      CK(read_counters(), "final sync");
       tr.mark("ids done");
-      if (h_small[0] & kFlagInternal) { rc = fail(SAS_ERR_INTERNAL, "id gather invariant"); goto done; }
+      if (h.flags & kFlagInternal) { rc = fail(SAS_ERR_INTERNAL, "id gather invariant"); goto done; }
+      const unsigned long long n_ids = h.n_ids;
       res->info.n_candidates = n_out;
-      res->complete = n_out == h_small[2];
+      res->complete = n_out == n_valid;
       res->info.n_ids = n_ids;
-      res->info.n_pairs = h_small64[0];
+      res->info.n_pairs = h.pairs;
       res->info.n_emitted = n_emit;
-      res->info.t0 = h_t0;
+      res->info.t0 = h.t0;
       res->info.counter_bits = (uint32_t)plan.tc.cb;
       res->info.tile_kx = (uint32_t)plan.tc.kx;
       res->info.tile_ky = (uint32_t)plan.tc.ky;
@@ -607,10 +618,7 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
 #undef CK
   }
   if (rc != SAS_OK) {
-    if (res->d_ids) cudaFreeAsync(res->d_ids, s);
-    if (res->d_cands) cudaFreeAsync(res->d_cands, s);
-    for (void* p : {(void*)res->d_dets, (void*)res->d_boff, (void*)res->d_ecount, (void*)res->d_sxt,
-                    (void*)res->d_syt, (void*)res->d_dt})
+    for (void* p : {res->d_mem, res->d_out})
       if (p) cudaFreeAsync(p, s);
     cudaStreamSynchronize(s);
     delete res;
@@ -821,9 +829,13 @@ int sas_peaks(const sas_result* r, uint32_t* idx, uint64_t* n_peaks, void* strea
 
 void sas_result_free(sas_result* r) {
   if (!r) return;
-  for (void* p : {(void*)r->d_cands, (void*)r->d_ids, (void*)r->d_dets, (void*)r->d_boff,
-                  (void*)r->d_ecount, (void*)r->d_sxt, (void*)r->d_syt, (void*)r->d_dt})
-    if (p) cudaFree(p);
+  if (r->d_mem) cudaFree(r->d_mem);
+  if (r->d_out) {
+    cudaFree(r->d_out);
+  } else {  // a cluster list: two arrays of its own
+    if (r->d_cands) cudaFree(r->d_cands);
+    if (r->d_ids) cudaFree(r->d_ids);
+  }
   delete r;
 }
 

@@ -284,7 +284,7 @@ int build_pass(sas_batch* b, const DevInfo& di, cudaStream_t s) {
   if (ce == cudaSuccess) ce = cudaMemcpyAsync(B.cand_off, cand_off.data(), (n_fields + 1) * 8, cudaMemcpyHostToDevice, s);
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
   for (const sas_batch::Group& g : b->groups)
-    if (ce == cudaSuccess) ce = stack_set_smem_attr(g.kx, g.ky, g.cb, g.smem);
+    if (ce == cudaSuccess) ce = stack_set_smem_attr(g.kx, g.ky, g.cb, g.smem, g.peaks);
   if (ce == cudaSuccess) ce = batch_set_attrs();
   // One launch of each group's stack kernel before the capture, with its work
   // counter far past the end (0x7F7F...: every CTA leaves at once, and the

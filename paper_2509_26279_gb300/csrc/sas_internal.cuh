@@ -192,17 +192,18 @@ cudaError_t launch_ingest(const int32_t* x, const int32_t* y, const uint16_t* ep
                           uint32_t* bucket_of, uint32_t* flags, cudaStream_t s);
 cudaError_t launch_scatter(const int32_t* x, const int32_t* y, const uint16_t* epoch, uint64_t n,
                            const uint32_t* bucket_of, uint32_t* cursor, Det* dets, cudaStream_t s);
-cudaError_t launch_epoch_setup(uint32_t E, const int64_t* t, const uint32_t* ecount, int64_t* dt,
-                               int64_t* t0, cudaStream_t s);
 // Largest and summed weight (uint8) of n detections: out[0], out[1].
 cudaError_t launch_weight_stats(const uint8_t* w, uint64_t n, unsigned long long* out, cudaStream_t s);
-cudaError_t launch_shift_tables(const SearchGeom& g, const int64_t* dt, const uint32_t* ecount,
+// Reference epoch t0, dt[e] = t[e] - t0 (0 for epochs without detections) and the shift tables of both axes.
+cudaError_t launch_shift_tables(const SearchGeom& g, const int64_t* t, const uint32_t* ecount, int64_t* dt, int64_t* t0,
                                 int32_t* sxt, int32_t* syt, uint32_t* flags, cudaStream_t s);
-// exclusive scan, out[i] = sum(in[0..i)), out has n+1 entries
-cudaError_t launch_scan_u32(const uint32_t* in, uint32_t* out, uint64_t n, uint32_t* scratch,
-                            cudaStream_t s);
-cudaError_t launch_scan_u32_to_u64(const uint32_t* in, unsigned long long* out, uint64_t n,
-                                   unsigned long long* scratch, cudaStream_t s);
+// exclusive scan, out[i] = sum(in[0..i)), out has n+1 entries; out2 (n entries): a copy of out, or null
+cudaError_t launch_scan_u32(const uint32_t* in, uint32_t* out, uint64_t n, uint32_t* scratch, cudaStream_t s,
+                            uint32_t* out2 = nullptr);
+// Id offsets (n) and candidate records of n sorted keys; *n_ids gets the total (untouched for n = 0).
+cudaError_t launch_candidates(const Key* keys, uint32_t n, unsigned long long* id_off, unsigned long long* scratch,
+                              sas_candidate* out, unsigned long long* n_ids, cudaStream_t s);
+size_t candidates_scratch_elems(uint64_t n);
 size_t scan_scratch_elems(uint64_t n);
 
 // sas_stack.cu (kernel: sas_stack_kernel.cuh)
@@ -217,8 +218,8 @@ cudaError_t launch_stack(const StackArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_stack_multi(int kx, int ky, int cb, bool peaks, const StackArgs* fargs,
                                const unsigned long long* unit_base, int n_fields,
                                unsigned long long* counter, size_t smem, int grid, cudaStream_t s);
-// Sets the shared-memory limit of both instantiations.
-cudaError_t stack_set_smem_attr(int kx, int ky, int cb, size_t smem);
+// Raises the shared-memory limit of the instantiation with or without peak selection.
+cudaError_t stack_set_smem_attr(int kx, int ky, int cb, size_t smem, bool peaks);
 // sas_stack_peaks.cu: the same with peak selection
 cudaError_t launch_stack_peaks(const StackArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_stack_multi_peaks(int kx, int ky, int cb, const StackArgs* fargs,
@@ -303,15 +304,17 @@ cudaError_t launch_sort_keys(Key* keys, uint32_t n, uint32_t n_pad, cudaStream_t
 // Sorts every aligned segment of `seg` keys (a power of two) of keys[0..n_total)
 // ascending; n_total is a multiple of seg.
 cudaError_t launch_sort_segments(Key* keys, uint32_t n_total, uint32_t seg, cudaStream_t s);
-cudaError_t launch_key_raw(const Key* keys, uint32_t n, uint32_t* raw, cudaStream_t s);
+// Sorts n keys into `sorted` (which may be `keys` only when sort_in_place(n)); equal
+// keys keep their order.  Without sort_in_place both need room for n keys, or for the
+// next power of two beyond kSortMerge keys.
+constexpr uint32_t kSortMerge = 1u << 16;
+bool sort_in_place(uint32_t n);
+cudaError_t launch_sort(Key* keys, uint32_t n, Key* sorted, cudaStream_t s);
 cudaError_t launch_gather_ids(const Key* keys, uint32_t n, const unsigned long long* id_off,
                               const SearchGeom& g, const CoarseGeom& cg, const Det* dets,
                               const uint32_t* boff, const uint32_t* ecount, const int32_t* sxt,
                               const int32_t* syt, uint32_t* ids_tmp, uint32_t* ids,
                               uint32_t* flags, cudaStream_t s);
-cudaError_t launch_write_candidates(const Key* keys, uint32_t n, const unsigned long long* id_off,
-                                    sas_candidate* out, cudaStream_t s);
-
 // A finished search's candidates together with what is needed to recount any
 // cell of its lattice: bucketed catalog, per-epoch counts, shift tables.
 struct CandView {

@@ -145,9 +145,75 @@ __global__ void k_bitonic_global(Key* keys, uint32_t n_pad, uint32_t k, uint32_t
   }
 }
 
-__global__ void k_key_raw(const Key* __restrict__ keys, uint32_t n, uint32_t* __restrict__ raw) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) raw[i] = ~(uint32_t)keys[i].a;
+// ---- sort by chunks and ranks --------------------------------------------------
+//
+// Up to kSortMerge keys: blocks sort chunks of kRankChunk keys in shared memory,
+// then every key finds its place by binary searches in the other chunks (an
+// earlier chunk's equal keys go first).  Two launches; the bitonic network over
+// 2048-key chunks took 57 us for its first stage alone (8 blocks of 1024 threads for
+// 16384 keys, 66 steps each), and a launch or two per doubling after that.
+
+constexpr int kRankChunk = 512;
+constexpr int kRankThreads = kRankChunk / 2;
+
+__global__ void __launch_bounds__(kRankThreads) k_sort_chunks(Key* keys, uint32_t n) {
+  __shared__ uint64_t sa[kRankChunk], sb[kRankChunk];
+  __shared__ uint32_t sc[kRankChunk];
+  const uint32_t base = blockIdx.x * kRankChunk, len = min((uint32_t)kRankChunk, n - base);
+  for (uint32_t i = threadIdx.x; i < kRankChunk; i += kRankThreads) {
+    const Key k = i < len ? keys[base + i] : max_key();
+    sa[i] = k.a;
+    sb[i] = k.b;
+    sc[i] = k.c;
+  }
+  __syncthreads();
+  uint32_t top = 2;  // the network over the next power of two of this chunk's keys
+  while (top < len) top <<= 1;
+  for (uint32_t k = 2; k <= top; k <<= 1) {
+    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+      const uint32_t t = threadIdx.x, i = ((t & ~(j - 1)) << 1) | (t & (j - 1)), x = i | j;
+      if (x < top) {
+        const uint64_t a0 = sa[i], a1 = sa[x], b0 = sb[i], b1 = sb[x];
+        const uint32_t c0 = sc[i], c1 = sc[x];
+        const bool less = a1 != a0 ? a1 < a0 : b1 != b0 ? b1 < b0 : c1 < c0;
+        if (less == ((i & k) == 0) && (a0 != a1 || b0 != b1 || c0 != c1)) {
+          sa[i] = a1; sa[x] = a0;
+          sb[i] = b1; sb[x] = b0;
+          sc[i] = c1; sc[x] = c0;
+        }
+      }
+      __syncthreads();
+    }
+  }
+  for (uint32_t i = threadIdx.x; i < len; i += kRankThreads) {
+    Key k;
+    k.a = sa[i];
+    k.b = sb[i];
+    k.c = sc[i];
+    k.pad = 0;
+    keys[base + i] = k;
+  }
+}
+
+__global__ void __launch_bounds__(128) k_rank_merge(const Key* __restrict__ keys, uint32_t n, Key* __restrict__ out) {
+  const uint32_t i = blockIdx.x * 128 + threadIdx.x;
+  if (i >= n) return;
+  const Key key = keys[i];
+  const uint32_t own = i / kRankChunk, chunks = (n + kRankChunk - 1) / kRankChunk;
+  uint32_t rank = i % kRankChunk;
+  for (uint32_t c = 0; c < chunks; ++c) {
+    if (c == own) continue;
+    uint32_t lo = c * kRankChunk, hi = min(lo + kRankChunk, n);
+    rank -= lo;
+    while (lo < hi) {
+      const uint32_t m = (lo + hi) >> 1;
+      const Key& k = keys[m];
+      const bool before = c < own ? !key_less(key, k) : key_less(k, key);
+      if (before) lo = m + 1; else hi = m;
+    }
+    rank += lo;
+  }
+  out[rank] = key;
 }
 
 // One warp per candidate: collect the ids of every detection in the cell
@@ -204,23 +270,6 @@ __global__ void k_gather_ids(const Key* __restrict__ keys, uint32_t n,
   }
 }
 
-__global__ void k_write_candidates(const Key* __restrict__ keys, uint32_t n,
-                                   const unsigned long long* __restrict__ id_off,
-                                   sas_candidate* __restrict__ out) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const Key k = keys[i];
-  sas_candidate c;
-  c.v_idx = (uint32_t)(k.b >> 32);
-  c.by = (uint32_t)k.b;
-  c.bx = k.c;
-  c.count = ~(uint32_t)(k.a >> 32);
-  c.raw = ~(uint32_t)k.a;
-  c.id_len = c.raw;
-  c.id_off = id_off[i];
-  out[i] = c;
-}
-
 unsigned blocks_for(uint64_t n, unsigned per) { return (unsigned)((n + per - 1) / per); }
 
 }  // namespace
@@ -270,10 +319,27 @@ cudaError_t launch_sort_segments(Key* keys, uint32_t n_total, uint32_t seg, cuda
   return cudaGetLastError();
 }
 
-cudaError_t launch_key_raw(const Key* keys, uint32_t n, uint32_t* raw, cudaStream_t s) {
-  if (n == 0) return cudaSuccess;
-  k_key_raw<<<blocks_for(n, 256), 256, 0, s>>>(keys, n, raw);
+bool sort_in_place(uint32_t n) { return n <= (uint32_t)kRankChunk; }
+
+cudaError_t launch_sort(Key* keys, uint32_t n, Key* sorted, cudaStream_t s) {
+  if (n > kSortMerge) {
+    uint32_t n_pad = 1;
+    while (n_pad < n) n_pad <<= 1;
+    if (keys != sorted) {
+      cudaError_t e = cudaMemcpyAsync(sorted, keys, (size_t)n * sizeof(Key), cudaMemcpyDeviceToDevice, s);
+      if (e != cudaSuccess) return e;
+    }
+    return launch_sort_keys(sorted, n, n_pad, s);
+  }
+  if (n <= 1) return n && keys != sorted ? cudaMemcpyAsync(sorted, keys, sizeof(Key), cudaMemcpyDeviceToDevice, s) : cudaSuccess;
+  k_sort_chunks<<<blocks_for(n, kRankChunk), kRankThreads, 0, s>>>(keys, n);
   note_launch();
+  if (!sort_in_place(n)) {
+    k_rank_merge<<<blocks_for(n, 128), 128, 0, s>>>(keys, n, sorted);
+    note_launch();
+  } else if (keys != sorted) {
+    return cudaMemcpyAsync(sorted, keys, (size_t)n * sizeof(Key), cudaMemcpyDeviceToDevice, s);
+  }
   return cudaGetLastError();
 }
 
@@ -285,14 +351,6 @@ cudaError_t launch_gather_ids(const Key* keys, uint32_t n, const unsigned long l
   if (n == 0) return cudaSuccess;
   k_gather_ids<<<blocks_for(n, kWarpsPerBlock), kWarpsPerBlock * 32, 0, s>>>(
       keys, n, id_off, g, cg, dets, boff, ecount, sxt, syt, ids_tmp, ids, flags);
-  note_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_write_candidates(const Key* keys, uint32_t n, const unsigned long long* id_off,
-                                    sas_candidate* out, cudaStream_t s) {
-  if (n == 0) return cudaSuccess;
-  k_write_candidates<<<blocks_for(n, 256), 256, 0, s>>>(keys, n, id_off, out);
   note_launch();
   return cudaGetLastError();
 }

@@ -43,13 +43,13 @@ cudaError_t launch_stack_multi(int kx, int ky, int cb, bool peaks, const StackAr
   return cudaErrorInvalidValue;
 }
 
-cudaError_t stack_set_smem_attr(int kx, int ky, int cb, size_t smem) {
+cudaError_t stack_set_smem_attr(int kx, int ky, int cb, size_t smem, bool peaks) {
+  if (peaks) return stack_set_smem_attr_peaks(kx, ky, cb, smem);
   cudaError_t e = cudaErrorInvalidValue;
 #define SAS_ATTR(KX, KY, CB) if (kx == KX && ky == KY && cb == CB) e = attr_t<KX, KY, CB, kModePlain>(smem);
   SAS_STACK_CONFIGS(SAS_ATTR)
 #undef SAS_ATTR
-  if (e != cudaSuccess) return e;
-  return stack_set_smem_attr_peaks(kx, ky, cb, smem);
+  return e;
 }
 
 }  // namespace sas

@@ -28,6 +28,7 @@ struct sas_batch {
   std::vector<uint32_t> n_min;
   std::vector<sas_opts> opts;
   std::vector<FieldPlan> plans;
+  std::vector<uint8_t> wide;   // field counts in 8-bit counters from zero (see sas_batch_create)
   std::vector<BatchField> hf;              // host copy of the field descriptors
   // Capacities of the arena: candidate-key slots per field (one power of two for
   // all fields: the segment of the segmented sort), emission slots and id slots
@@ -51,6 +52,7 @@ struct sas_batch {
   struct Group {
     int kx = 0, ky = 0, cb = 0;
     bool peaks = false;
+    bool wide = false;  // 8-bit counters from zero (kModePeaksWide)
     std::vector<uint32_t> fields;
     size_t smem = 0;
     int grid = 0;
@@ -76,6 +78,13 @@ int cuda_err(cudaError_t e, const char* where) {
 
 size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
+cudaError_t launch_group(const sas_batch::Group& g, cudaStream_t s) {
+  if (g.wide) return launch_stack_multi_wide(g.d_args, g.d_unit_base, (int)g.fields.size(), g.d_work, g.smem, g.grid, s);
+  return launch_stack_multi(g.kx, g.ky, g.cb, g.peaks, g.d_args, g.d_unit_base, (int)g.fields.size(), g.d_work, g.smem,
+                            g.grid, s);
+}
+
+
 // Records the device work of one batch pass on stream s (used under capture).
 cudaError_t record_pass(sas_batch* b, cudaStream_t s) {
   cudaError_t e;
@@ -87,9 +96,7 @@ cudaError_t record_pass(sas_batch* b, cudaStream_t s) {
   if ((e = cudaMemsetAsync(b->dev.bucket_count, 0, b->dev.total_buckets * 4, s)) != cudaSuccess) return e;
   if ((e = batch_launch_prep(b->dev, s)) != cudaSuccess) return e;
   for (const sas_batch::Group& g : b->groups)
-    if ((e = launch_stack_multi(g.kx, g.ky, g.cb, g.peaks, g.d_args, g.d_unit_base, (int)g.fields.size(),
-                                g.d_work, g.smem, g.grid, s)) != cudaSuccess)
-      return e;
+    if ((e = launch_group(g, s)) != cudaSuccess) return e;
   if ((e = batch_launch_post(b->dev, s)) != cudaSuccess) return e;
   if ((e = cudaMemcpyAsync(b->h_ctr, b->d_ctr, (size_t)b->n_fields * kCtrN * 4,
                            cudaMemcpyDeviceToHost, s)) != cudaSuccess)
@@ -125,6 +132,29 @@ void free_batch(sas_batch* b) {
 }  // namespace
 
 namespace {
+
+// The fields by stack kernel configuration.
+void group_fields(sas_batch* b) {
+  b->groups.clear();
+  for (uint32_t f = 0; f < b->n_fields; ++f) {
+    const TileCfg& tc = b->plans[f].tc;
+    sas_batch::Group* g = nullptr;
+    const bool peaks = b->opts[f].peaks_only || b->opts[f].n_low < b->n_min[f], wide = b->wide[f] != 0;
+    for (sas_batch::Group& h : b->groups)
+      if (h.kx == tc.kx && h.ky == tc.ky && h.cb == tc.cb && h.peaks == peaks && h.wide == wide) g = &h;
+    if (!g) {
+      b->groups.emplace_back();
+      g = &b->groups.back();
+      g->kx = tc.kx;
+      g->ky = tc.ky;
+      g->cb = tc.cb;
+      g->peaks = peaks;
+      g->wide = wide;
+    }
+    g->fields.push_back(f);
+    g->smem = std::max(g->smem, tc.smem);
+  }
+}
 
 // Lays out the device arena for the current capacities, writes the field
 // descriptors and records one pass of the whole pipeline as a graph.
@@ -284,7 +314,7 @@ int build_pass(sas_batch* b, const DevInfo& di, cudaStream_t s) {
   if (ce == cudaSuccess) ce = cudaMemcpyAsync(B.cand_off, cand_off.data(), (n_fields + 1) * 8, cudaMemcpyHostToDevice, s);
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
   for (const sas_batch::Group& g : b->groups)
-    if (ce == cudaSuccess) ce = stack_set_smem_attr(g.kx, g.ky, g.cb, g.smem, g.peaks);
+    if (ce == cudaSuccess) ce = g.wide ? stack_set_smem_attr_wide(g.smem) : stack_set_smem_attr(g.kx, g.ky, g.cb, g.smem, g.peaks);
   if (ce == cudaSuccess) ce = batch_set_attrs();
   // One launch of each group's stack kernel before the capture, with its work
   // counter far past the end (0x7F7F...: every CTA leaves at once, and the
@@ -294,8 +324,7 @@ int build_pass(sas_batch* b, const DevInfo& di, cudaStream_t s) {
   for (const sas_batch::Group& g : b->groups) {
     ce = cudaMemsetAsync(g.d_work, 0x7F, 8, s);
     if (ce == cudaSuccess)
-      ce = launch_stack_multi(g.kx, g.ky, g.cb, g.peaks, g.d_args, g.d_unit_base, (int)g.fields.size(), g.d_work,
-                              g.smem, g.grid, s);
+      ce = launch_group(g, s);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
     if (ce != cudaSuccess)
       return set_errorf(SAS_ERR_CUDA, "batch setup: stack kernel (kx %d, ky %d, %d-bit counters%s, %zu B shared, "
@@ -369,10 +398,12 @@ int sas_batch_create(const sas_grid* const* grids, const sas_catalog* cats, cons
     // one super-bin: a field whose brightest mover (one detection per epoch)
     // plus a generous noise allowance could get there counts in 16 bits.  A
     // wrap is still detected and recomputed exactly; this keeps it rare.
+    bool may_widen = false;
     if (o.counter_bits == 0) {
       const double lam = (double)c.n * 9.0 / ((double)desc.nbx * desc.nby);  // per 3 x 3-bin super-bin
       const double reach = (double)c.n_epochs + lam + 6.0 * std::sqrt(lam) + 2.0;
       o.counter_bits = reach >= 128.0 + o.n_low ? 16 : 8;
+      may_widen = o.counter_bits == 16 && reach < 250.0 && (o.peaks_only || o.n_low < n_min[f]);
     }
     o.v_begin = o.v_end = 0;
     b->opts.push_back(o);
@@ -387,27 +418,19 @@ int sas_batch_create(const sas_grid* const* grids, const sas_catalog* cats, cons
                       (uint64_t)desc.nvx * desc.nvy, o, di, &fp);
     }
     if (rc != SAS_OK) break;
+    // With peak selection 8-bit counters that start at zero hold 255 detections: the
+    // tiles stay those of the 16-bit plan (the peaks are defined within them), the
+    // reductions and the finish pass halve.  A wrap brings the 16 bits back (run).
+    const bool wide = may_widen && fp.tc.cb == 16 && fp.tc.kx == 8 && fp.tc.ky == 4;
+    if (wide) {
+      fp.tc.cb = 8;
+      fp.tc.smem = stack_smem_bytes(fp.tc);
+    }
+    b->wide.push_back(wide);
     b->plans.push_back(fp);
   }
   if (rc != SAS_OK) { free_batch(b); return rc; }
-  // group the fields by stack kernel configuration
-  for (uint32_t f = 0; f < n_fields; ++f) {
-    const TileCfg& tc = b->plans[f].tc;
-    sas_batch::Group* g = nullptr;
-    const bool peaks = b->opts[f].peaks_only || b->opts[f].n_low < b->n_min[f];
-    for (sas_batch::Group& h : b->groups)
-      if (h.kx == tc.kx && h.ky == tc.ky && h.cb == tc.cb && h.peaks == peaks) g = &h;
-    if (!g) {
-      b->groups.emplace_back();
-      g = &b->groups.back();
-      g->kx = tc.kx;
-      g->ky = tc.ky;
-      g->cb = tc.cb;
-      g->peaks = peaks;
-    }
-    g->fields.push_back(f);
-    g->smem = std::max(g->smem, tc.smem);
-  }
+  group_fields(b);
   b->emit_cap.resize(n_fields);
   b->ids_cap.resize(n_fields);
   for (uint32_t f = 0; f < n_fields; ++f) {
@@ -440,12 +463,19 @@ int sas_batch_run(sas_batch* b, void* stream) {
   // at most: a field cut short at one stage can need more at the next).
   for (int round = 0; round < 4; ++round) {
     bool grow = false;
+    std::vector<uint32_t> narrow;  // fields that need their 16-bit counters
     uint32_t key_seg = b->key_seg;
     std::vector<uint32_t> emit_cap = b->emit_cap;
     std::vector<uint64_t> ids_cap = b->ids_cap;
     for (uint32_t f = 0; f < b->n_fields; ++f) {
       const uint32_t* ctr = b->h_ctr + (size_t)f * kCtrN;
       const uint32_t fl = ctr[kCtrFlags];
+      if (b->wide[f] && !(fl & (kFlagEpoch | kFlagPos | kFlagShift)) &&
+          ((fl & kFlagCounter) || b->h_c64[(size_t)f * kC64N + kC64Balance] != 0)) {
+        narrow.push_back(f);  // a counter wrapped at 256
+        grow = true;
+        continue;
+      }
       if (fl & (kFlagEpoch | kFlagPos | kFlagShift | kFlagCounter | kFlagInternal)) continue;
       if (!(fl & kFlagEmitCap) && ctr[kCtrEmit] <= b->emit_cap[f]) continue;
       const uint64_t need_emit = ctr[kCtrEmit], need_keys = ctr[kCtrValid];
@@ -468,6 +498,13 @@ int sas_batch_run(sas_batch* b, void* stream) {
     b->emit_cap = emit_cap;
     b->ids_cap = ids_cap;
     free_pass(b);
+    for (uint32_t f : narrow) {
+      TileCfg& tc = b->plans[f].tc;
+      tc.cb = 16;
+      tc.smem = stack_smem_bytes(tc);
+      b->wide[f] = 0;
+    }
+    if (!narrow.empty()) group_fields(b);
     DevInfo di;
     int rc = device_info(b->device, &di);
     if (rc == SAS_OK) rc = build_pass(b, di, s);

@@ -42,33 +42,43 @@ __device__ __forceinline__ bool key_less_b(const Key& p, const Key& q) {
 __global__ void k_batch_ingest(const BatchField* __restrict__ F, int n_fields,
                                const unsigned long long* __restrict__ det_off,
                                uint32_t* __restrict__ bucket_count, uint32_t* __restrict__ bucket_of) {
+  // Detections come epoch by epoch, so a warp mostly adds to one epoch counter: one
+  // atomic per warp and counter (an atomic each took 1.85 ms for 7 million, all on
+  // a few hundred addresses).
   const unsigned long long total = det_off[n_fields];
-  for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < total;
-       i += (unsigned long long)gridDim.x * blockDim.x) {
-    const int f = find_field(det_off, n_fields, i);
-    const BatchField& bf = F[f];
-    const unsigned long long k = i - det_off[f];
-    const uint32_t e = bf.epoch[k];
-    const int32_t xi = bf.x[k], yi = bf.y[k];
-    uint32_t b = kInvalidBucket;
-    if (e >= bf.E) {
-      atomicOr(bf.counters + kCtrFlags, kFlagEpoch);
-    } else {
-      atomicAdd(&bf.ecount[e], 1u);
-      if (xi <= -kLimPos || xi >= kLimPos || yi <= -kLimPos || yi >= kLimPos) {
-        atomicOr(bf.counters + kCtrFlags, kFlagPos);
+  const int lane = threadIdx.x & 31;
+  for (unsigned long long i0 = blockIdx.x * (unsigned long long)blockDim.x + (threadIdx.x & ~31u); i0 < total;
+       i0 += (unsigned long long)gridDim.x * blockDim.x) {
+    const unsigned long long i = i0 + lane;
+    uint32_t* counter = nullptr;  // this detection's epoch counter
+    if (i < total) {
+      const int f = find_field(det_off, n_fields, i);
+      const BatchField& bf = F[f];
+      const unsigned long long k = i - det_off[f];
+      const uint32_t e = bf.epoch[k];
+      const int32_t xi = bf.x[k], yi = bf.y[k];
+      uint32_t b = kInvalidBucket;
+      if (e >= bf.E) {
+        atomicOr(bf.counters + kCtrFlags, kFlagEpoch);
       } else {
-        const CoarseGeom& cg = bf.args.cg;
-        const int64_t cx = floor_div64((int64_t)xi - cg.gx0, cg.cell);
-        const int64_t cy = floor_div64((int64_t)yi - cg.gy0, cg.cell);
-        if (cx >= 0 && cx < cg.ncx && cy >= 0 && cy < cg.ncy) {
-          b = (uint32_t)(bf.bucket_base +
-                         ((uint64_t)e * cg.ncy + (uint64_t)cy) * cg.ncx + (uint64_t)cx);
-          atomicAdd(&bucket_count[b], 1u);
+        counter = &bf.ecount[e];
+        if (xi <= -kLimPos || xi >= kLimPos || yi <= -kLimPos || yi >= kLimPos) {
+          atomicOr(bf.counters + kCtrFlags, kFlagPos);
+        } else {
+          const CoarseGeom& cg = bf.args.cg;
+          const int64_t cx = floor_div64((int64_t)xi - cg.gx0, cg.cell);
+          const int64_t cy = floor_div64((int64_t)yi - cg.gy0, cg.cell);
+          if (cx >= 0 && cx < cg.ncx && cy >= 0 && cy < cg.ncy) {
+            b = (uint32_t)(bf.bucket_base +
+                           ((uint64_t)e * cg.ncy + (uint64_t)cy) * cg.ncx + (uint64_t)cx);
+            atomicAdd(&bucket_count[b], 1u);
+          }
         }
       }
+      bucket_of[i] = b;
     }
-    bucket_of[i] = b;
+    const uint32_t same = __match_any_sync(0xffffffffu, (unsigned long long)(uintptr_t)counter);
+    if (counter && lane == __ffs(same) - 1) atomicAdd(counter, (uint32_t)__popc(same));
   }
 }
 

@@ -226,6 +226,10 @@ cudaError_t launch_stack_multi_peaks(int kx, int ky, int cb, const StackArgs* fa
                                      const unsigned long long* unit_base, int n_fields,
                                      unsigned long long* counter, size_t smem, int grid, cudaStream_t s);
 cudaError_t stack_set_smem_attr_peaks(int kx, int ky, int cb, size_t smem);
+// 8 x 4 lattice points with 8-bit counters that hold 255 detections
+cudaError_t launch_stack_multi_wide(const StackArgs* fargs, const unsigned long long* unit_base, int n_fields,
+                                    unsigned long long* counter, size_t smem, int grid, cudaStream_t s);
+cudaError_t stack_set_smem_attr_wide(size_t smem);
 
 // sas_stack_windows.cu: the kernel over blocks of cells
 bool windows_config_supported(int kx, int ky, int cb);

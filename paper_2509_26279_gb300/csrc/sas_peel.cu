@@ -579,7 +579,11 @@ int peel_clusters(const CandView& v, uint32_t n_min, uint32_t max_clusters, bool
       if (e == cudaSuccess) {
         k_tie_keys<<<blocks_of(nc, 256), 256, 0, s>>>(v.cands, (uint32_t)nc, keys);
         note_launch();
-        e = launch_sort_keys(keys, (uint32_t)nc, n_pad, s);
+        Key* sorted = keys;
+        e = cudaGetLastError();
+        if (e == cudaSuccess && nc <= kSortMerge && !sort_in_place((uint32_t)nc)) e = sc.get(&sorted, nc);
+        if (e == cudaSuccess) e = launch_sort(keys, (uint32_t)nc, sorted, s);
+        keys = sorted;
       }
       if (e == cudaSuccess) {
         k_tie_rank<<<blocks_of(nc, 256), 256, 0, s>>>(keys, (uint32_t)nc, rank, live[0]);
@@ -633,7 +637,11 @@ int peel_clusters(const CandView& v, uint32_t n_min, uint32_t max_clusters, bool
       if (e == cudaSuccess && n_pick) {
         k_pick_keys<<<blocks_of(n_pick, 256), 256, 0, s>>>(pick_key, n_pick, pkeys);
         note_launch();
-        e = launch_sort_keys(pkeys, n_pick, p_pad, s);
+        Key* sorted = pkeys;
+        e = cudaGetLastError();
+        if (e == cudaSuccess && n_pick <= kSortMerge && !sort_in_place(n_pick)) e = sc.get(&sorted, n_pick);
+        if (e == cudaSuccess) e = launch_sort(pkeys, n_pick, sorted, s);
+        pkeys = sorted;
       }
       if (e == cudaSuccess && n_out) {
         k_pick_len<<<blocks_of(n_out, 256), 256, 0, s>>>(pkeys, n_out, pk, pick_key, len);

@@ -158,13 +158,14 @@ constexpr int kRankThreads = kRankChunk / 2;
 
 __global__ void __launch_bounds__(kRankThreads) k_sort_chunks(Key* keys, uint32_t n) {
   __shared__ uint64_t sa[kRankChunk], sb[kRankChunk];
-  __shared__ uint32_t sc[kRankChunk];
+  __shared__ uint32_t sc[kRankChunk], sp[kRankChunk];  // pad: the caller's payload
   const uint32_t base = blockIdx.x * kRankChunk, len = min((uint32_t)kRankChunk, n - base);
   for (uint32_t i = threadIdx.x; i < kRankChunk; i += kRankThreads) {
     const Key k = i < len ? keys[base + i] : max_key();
     sa[i] = k.a;
     sb[i] = k.b;
     sc[i] = k.c;
+    sp[i] = k.pad;
   }
   __syncthreads();
   uint32_t top = 2;  // the network over the next power of two of this chunk's keys
@@ -180,6 +181,9 @@ __global__ void __launch_bounds__(kRankThreads) k_sort_chunks(Key* keys, uint32_
           sa[i] = a1; sa[x] = a0;
           sb[i] = b1; sb[x] = b0;
           sc[i] = c1; sc[x] = c0;
+          const uint32_t p0 = sp[i];
+          sp[i] = sp[x];
+          sp[x] = p0;
         }
       }
       __syncthreads();
@@ -190,30 +194,35 @@ __global__ void __launch_bounds__(kRankThreads) k_sort_chunks(Key* keys, uint32_
     k.a = sa[i];
     k.b = sb[i];
     k.c = sc[i];
-    k.pad = 0;
+    k.pad = sp[i];
     keys[base + i] = k;
   }
 }
 
-__global__ void __launch_bounds__(128) k_rank_merge(const Key* __restrict__ keys, uint32_t n, Key* __restrict__ out) {
-  const uint32_t i = blockIdx.x * 128 + threadIdx.x;
-  if (i >= n) return;
-  const Key key = keys[i];
+// Eight threads per key share the other chunks.
+__global__ void __launch_bounds__(256) k_rank_merge(const Key* __restrict__ keys, uint32_t n, Key* __restrict__ out) {
+  const uint32_t i = (blockIdx.x * 256 + threadIdx.x) >> 3, part = threadIdx.x & 7;
   const uint32_t own = i / kRankChunk, chunks = (n + kRankChunk - 1) / kRankChunk;
-  uint32_t rank = i % kRankChunk;
-  for (uint32_t c = 0; c < chunks; ++c) {
-    if (c == own) continue;
-    uint32_t lo = c * kRankChunk, hi = min(lo + kRankChunk, n);
-    rank -= lo;
-    while (lo < hi) {
-      const uint32_t m = (lo + hi) >> 1;
-      const Key& k = keys[m];
-      const bool before = c < own ? !key_less(key, k) : key_less(k, key);
-      if (before) lo = m + 1; else hi = m;
+  Key key{};
+  uint32_t rank = 0;
+  if (i < n) {
+    key = keys[i];
+    for (uint32_t c = part; c < chunks; c += 8) {
+      if (c == own) continue;
+      uint32_t lo = c * kRankChunk, hi = min(lo + kRankChunk, n);
+      rank -= lo;
+      while (lo < hi) {
+        const uint32_t m = (lo + hi) >> 1;
+        const Key& k = keys[m];
+        const bool before = c < own ? !key_less(key, k) : key_less(k, key);
+        if (before) lo = m + 1; else hi = m;
+      }
+      rank += lo;
     }
-    rank += lo;
   }
-  out[rank] = key;
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+  if (i < n && part == 0) out[rank + i % kRankChunk] = key;
 }
 
 // One warp per candidate: collect the ids of every detection in the cell
@@ -335,7 +344,7 @@ cudaError_t launch_sort(Key* keys, uint32_t n, Key* sorted, cudaStream_t s) {
   k_sort_chunks<<<blocks_for(n, kRankChunk), kRankThreads, 0, s>>>(keys, n);
   note_launch();
   if (!sort_in_place(n)) {
-    k_rank_merge<<<blocks_for(n, 128), 128, 0, s>>>(keys, n, sorted);
+    k_rank_merge<<<blocks_for((uint64_t)n * 8, 256), 256, 0, s>>>(keys, n, sorted);
     note_launch();
   } else if (keys != sorted) {
     return cudaMemcpyAsync(sorted, keys, (size_t)n * sizeof(Key), cudaMemcpyDeviceToDevice, s);

@@ -103,9 +103,11 @@ struct Pts {
   const int32_t* x;
   const int32_t* y;
   uint32_t n, nc;  // points, 32-point chunks
+  bool narrow;     // second moments of any subset fit int64
 };
 
-// Exact moments of the subset (bits: lane's membership word), then S, adj, det.
+// Exact moments of the subset (bits: lane's membership word), then S, adj, det:
+// every lane has all of it (the final fit; the starts use sfit below).
 __device__ __noinline__ WFit wfit(const Pts& p, uint32_t bits, int lane) {
   int64_t T = 0, X = 0, Y = 0;
   __int128 tt = 0, tx = 0, ty = 0, xx = 0, xy = 0, yy = 0;
@@ -160,16 +162,152 @@ __device__ __noinline__ WFit wfit(const Pts& p, uint32_t bits, int lane) {
   return f;
 }
 
+// What a C-step needs of a subset's fit, in every lane.
+struct SFit {
+  uint32_t m;
+  int64_t T, X, Y;
+  double a00, a01, a02, a11, a12, a22, det;
+};
+
+__device__ __forceinline__ int64_t shfl_xor_v(int64_t v, int o) {
+  return (int64_t)__shfl_xor_sync(0xffffffffu, (long long)v, o);
+}
+__device__ __forceinline__ __int128 shfl_xor_v(__int128 v, int o) { return shfl_xor_i128(v, o); }
+
+// Exact second moments of the subset, each in one lane: lane k < 6 returns the sum
+// of product k of (tt, tx, ty, xx, xy, yy) over the warp's members (other lanes:
+// anything).  Halves of the warp split the six sums between them as they add,
+// so the exchange takes 3 + 2 + 1 + 1 + 1 values instead of 5 x 6.
+template <typename V>
+__device__ __forceinline__ V moments(const Pts& p, uint32_t bits, int lane) {
+  V s[6] = {0, 0, 0, 0, 0, 0};
+  for (uint32_t c = 0; c < p.nc; ++c) {
+    if (!((bits >> c) & 1u)) continue;
+    const uint32_t i = c * 32 + lane;
+    const V t = p.t[i], x = p.x[i], y = p.y[i];
+    s[0] += t * t;
+    s[1] += t * x;
+    s[2] += t * y;
+    s[3] += x * x;
+    s[4] += x * y;
+    s[5] += y * y;
+  }
+  const bool up = lane & 16;  // lower half: sums 0-2, upper half: sums 3-5
+  V h[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) h[q] = (up ? s[3 + q] : s[q]) + shfl_xor_v(up ? s[q] : s[3 + q], 16);
+  const bool hi = lane & 8;   // sums 0, 1 / sum 2
+  const V e = shfl_xor_v(hi ? h[0] : h[2], 8), f = shfl_xor_v(h[1], 8);
+  V g0 = (hi ? h[2] : h[0]) + e, g1 = h[1] + f;  // hi: g0 = sum 2; else sums 0, 1
+  const bool one = lane & 4;  // of sums 0, 1: the second
+  V r = (!hi && one ? g1 : g0) + shfl_xor_v(hi || one ? g0 : g1, 4);
+  r += shfl_xor_v(r, 2);
+  r += shfl_xor_v(r, 1);
+  // sums 0, 1, 2, 3, 4, 5 are in lanes 0, 4, 8, 16, 20, 24
+  return r;
+}
+
+template <typename V>
+__device__ __forceinline__ V shfl_v(V v, int src);
+template <>
+__device__ __forceinline__ int64_t shfl_v(int64_t v, int src) {
+  return (int64_t)__shfl_sync(0xffffffffu, (long long)v, src);
+}
+template <>
+__device__ __forceinline__ __int128 shfl_v(__int128 v, int src) {
+  const uint64_t lo = __shfl_sync(0xffffffffu, (unsigned long long)(uint64_t)v, src);
+  const uint64_t hi = __shfl_sync(0xffffffffu, (unsigned long long)(uint64_t)(v >> 64), src);
+  return (__int128)(((unsigned __int128)hi << 64) | lo);
+}
+template <>
+__device__ __forceinline__ double shfl_v(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+
+// wfit's mean, adjugate and determinant by the same exact sums and the same double
+// operations, spread over lanes 0-5: each forms one scatter entry, one adjugate
+// entry, one product of the determinant.  FP64 (two operations a clock and SM) was
+// 73 % busy with all 32 lanes repeating the 23 operations and six conversions.
+__device__ __forceinline__ SFit sfit(const Pts& p, uint32_t bits, int lane) {
+  SFit f;
+  int64_t T = 0, X = 0, Y = 0;
+  for (uint32_t c = 0; c < p.nc; ++c) {
+    if (!((bits >> c) & 1u)) continue;
+    const uint32_t i = c * 32 + lane;
+    T += p.t[i];
+    X += p.x[i];
+    Y += p.y[i];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    T += shfl_xor_v(T, o);
+    X += shfl_xor_v(X, o);
+    Y += shfl_xor_v(Y, o);
+  }
+  f.m = __reduce_add_sync(0xffffffffu, __popc(bits));
+  f.T = T;
+  f.X = X;
+  f.Y = Y;
+  const int k = lane < 6 ? lane : 0, at = k < 3 ? 4 * k : 4 * k + 4;  // the lane that holds sum k
+  __int128 sum;
+  if (p.narrow) sum = (__int128)shfl_v(moments<int64_t>(p, bits, lane), at);
+  else sum = shfl_v(moments<__int128>(p, bits, lane), at);
+  const int64_t u = k < 3 ? T : k < 5 ? X : Y, v = k == 0 ? T : (k == 1 || k == 3) ? X : Y;
+  const double sk = i128_to_double((__int128)f.m * sum - (__int128)u * v);  // entry k of (00, 01, 02, 11, 12, 22)
+  // adjugate entry k = s[a] s[b] - s[c] s[d]
+  const int sh = 4 * k;
+  const double pa = shfl_v(sk, (0x010123 >> sh) & 7), pb = shfl_v(sk, (0x325445 >> sh) & 7);
+  const double pc = shfl_v(sk, (0x102214 >> sh) & 7), pd = shfl_v(sk, (0x142354 >> sh) & 7);
+  const double ak = sub(mul(pa, pb), mul(pc, pd));
+  const double dk = mul(sk, ak);
+  f.a00 = shfl_v(ak, 0);
+  f.a01 = shfl_v(ak, 1);
+  f.a02 = shfl_v(ak, 2);
+  f.a11 = shfl_v(ak, 3);
+  f.a12 = shfl_v(ak, 4);
+  f.a22 = shfl_v(ak, 5);
+  f.det = add(add(shfl_v(dk, 0), shfl_v(dk, 1)), shfl_v(dk, 2));
+  return f;
+}
+
 __device__ __forceinline__ uint64_t order_key(double q) {
   const uint64_t b = (uint64_t)__double_as_longlong(q);
   return (b >> 63) ? ~b : (b | (1ull << 63));
 }
 
-// Membership bits of the h smallest (key, index) among n <= 32 NC points:
-// each lane counts its NC points' ranks against every key (no dependent
-// reductions).
+// Membership bits of the h smallest (key, index) among n <= 32 NC points: each
+// lane counts its NC points' ranks against every key (no dependent reductions) --
+// first by the keys' upper words alone.  Points with fewer than h smaller upper
+// words are the h smallest when there are exactly h of them; else (equal upper
+// words at the boundary) the whole keys and indices decide.  (keys: 16-byte
+// aligned, entries n .. up to a multiple of 2 are never counted.)
 template <int NC>
 __device__ __forceinline__ uint32_t rank_select(const uint64_t* keys, uint32_t n, uint32_t h, int lane) {
+  uint32_t bits = 0;
+  {
+    uint32_t mine[NC], rank[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const uint32_t i = c * 32 + lane;
+      mine[c] = i < n ? (uint32_t)(keys[i] >> 32) : 0u;
+      rank[c] = i < n ? 0u : 0x80000000u;
+    }
+    const uint4* pairs = reinterpret_cast<const uint4*>(keys);
+    uint32_t j = 0;
+#pragma unroll 4
+    for (; j + 2 <= n; j += 2) {
+      const uint4 kk = pairs[j >> 1];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) rank[c] += (kk.y < mine[c] ? 1u : 0u) + (kk.w < mine[c] ? 1u : 0u);
+    }
+    if (j < n) {
+      const uint32_t k0 = (uint32_t)(keys[j] >> 32);
+#pragma unroll
+      for (int c = 0; c < NC; ++c) rank[c] += k0 < mine[c] ? 1u : 0u;
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) bits |= (rank[c] < h ? 1u : 0u) << c;
+    if (__reduce_add_sync(0xffffffffu, __popc(bits)) == h) return bits;
+    bits = 0;
+  }
   uint64_t mine[NC];
   uint32_t rank[NC];
 #pragma unroll
@@ -186,7 +324,6 @@ __device__ __forceinline__ uint32_t rank_select(const uint64_t* keys, uint32_t n
       rank[c] += (kj < mine[c] || (kj == mine[c] && j < i)) ? 1u : 0u;
     }
   }
-  uint32_t bits = 0;
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
     const uint32_t i = c * 32 + lane;
@@ -199,7 +336,7 @@ __device__ __forceinline__ uint32_t rank_select(const uint64_t* keys, uint32_t n
 // Up to 256 points: each point's rank is counted against every key (no
 // dependent reductions), for the cluster's number of 32-point chunks; more:
 // the h-th smallest key by binary descent.
-__device__ __noinline__ uint32_t wselect(const Pts& p, const WFit& f, uint32_t h, uint64_t* keys, int lane) {
+__device__ __noinline__ uint32_t wselect(const Pts& p, const SFit& f, uint32_t h, uint64_t* keys, int lane) {
   const int64_t m = f.m;
   for (uint32_t c = 0; c < p.nc; ++c) {
     const uint32_t i = c * 32 + lane;
@@ -282,24 +419,31 @@ __device__ __noinline__ StartOut run_start(const Pts& p, uint32_t h, uint64_t ke
     __syncwarp();
   };
   for (int q = 0; q < kDim + 1; ++q) draw();
-  WFit f = wfit(p, bits, lane);
-  while (f.det <= 0.0 && j < h) {
-    draw();
-    f = wfit(p, bits, lane);
+  // phase 0: the drawn points; 1: the h nearest; 2: C-steps (one copy of sfit and
+  // wselect in the loop keeps both inline)
+  uint32_t kept = 0, phase = 0, step = 0;
+  double det = 0.0;
+  for (;;) {
+    const SFit f = sfit(p, bits, lane);
+    if (phase == 0 && f.det <= 0.0) {
+      if (j < h) {
+        draw();
+        continue;
+      }
+      return StartOut{f.det, bits};
+    }
+    if (phase == 2 && !(f.det < det)) break;
+    det = f.det;
+    kept = bits;
+    if (phase > 0 && (step == max_steps || det <= 0.0)) break;
+    bits = wselect(p, f, h, keys, lane);
+    if (phase > 0) {
+      if (__all_sync(0xffffffffu, bits == kept)) break;  // same subset: same det, no decrease
+      ++step;
+    }
+    phase = phase == 0 ? 1 : 2;
   }
-  if (f.det <= 0.0) return StartOut{f.det, bits};
-  bits = wselect(p, f, h, keys, lane);
-  f = wfit(p, bits, lane);
-  for (uint32_t step = 0; step < max_steps; ++step) {
-    if (f.det <= 0.0) break;
-    const uint32_t b2 = wselect(p, f, h, keys, lane);
-    if (__all_sync(0xffffffffu, b2 == bits)) break;  // same subset: same det, no decrease
-    const WFit f2 = wfit(p, b2, lane);
-    if (!(f2.det < f.det)) break;
-    bits = b2;
-    f = f2;
-  }
-  return StartOut{f.det, bits};
+  return StartOut{det, kept};
 }
 
 __device__ __forceinline__ bool det_before(double da, uint32_t sa, double db, uint32_t sb) {
@@ -348,13 +492,17 @@ __device__ FitSmem carve(unsigned char* smem, uint32_t npad, uint32_t n_best) {
   return m;
 }
 
-__device__ uint32_t load_points(const FitArgs& a, uint32_t k, const FitSmem& m, int tid, int nthreads) {
+// *narrow: |t|, |x|, |y| < 2^26 for all (at most 2^10) points, as far as this thread saw.
+__device__ uint32_t load_points(const FitArgs& a, uint32_t k, const FitSmem& m, int tid, int nthreads, bool* narrow) {
   const uint32_t n = a.Pn[k];
+  *narrow = true;
   for (uint32_t i = tid; i < n; i += nthreads) {
     const Det d = a.pt[a.P[(size_t)k * a.cap + i]];
     m.t[i] = a.dt[d.e];
     m.x[i] = d.x;
     m.y[i] = d.y;
+    const int64_t lim = 1 << 26;
+    if (m.t[i] >= lim || m.t[i] <= -lim || d.x >= lim || d.x <= -lim || d.y >= lim || d.y <= -lim) *narrow = false;
   }
   return n;
 }
@@ -366,10 +514,11 @@ __global__ void __launch_bounds__(kFitThreads) k_fit_starts(FitArgs a) {
   if (a.status[k] != kRunning) return;
   if (a.Pn[k] < (uint32_t)kDim + 2) return;
   const FitSmem m = carve(smem, a.npad, a.n_best);
-  const uint32_t n = load_points(a, k, m, threadIdx.x, kFitThreads);
-  __syncthreads();
+  bool narrow;
+  const uint32_t n = load_points(a, k, m, threadIdx.x, kFitThreads, &narrow);
+  narrow = __syncthreads_and(narrow);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const Pts p{m.t, m.x, m.y, n, (n + 31) / 32};
+  const Pts p{m.t, m.x, m.y, n, (n + 31) / 32, narrow};
   const uint32_t h = (n + kDim + 1) / 2;
   const uint32_t stride = gridDim.x * kFitWarps;
   for (uint32_t s = blockIdx.x * kFitWarps + warp; s < a.n_starts; s += stride) {
@@ -386,36 +535,53 @@ __global__ void __launch_bounds__(kFitThreads) k_fit_best(FitArgs a) {
   if (a.status[k] != kRunning) return;
   if (a.Pn[k] < (uint32_t)kDim + 2) return;
   const FitSmem m = carve(smem, a.npad, a.n_best);
-  const uint32_t n = load_points(a, k, m, threadIdx.x, kFitThreads);
+  bool narrow;
+  const uint32_t n = load_points(a, k, m, threadIdx.x, kFitThreads, &narrow);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const double* det3 = a.det3 + (size_t)k * a.n_starts;
-  if (warp == 0) {  // the n_best lowest (det, start), in order
-    for (uint32_t b = 0; b < a.n_best; ++b) {
-      double bd = 0.0;
-      uint32_t bs = 0xFFFFFFFFu;
-      for (uint32_t s = lane; s < a.n_starts; s += 32) {
-        const double d = det3[s];
-        bool taken = false;
-        for (uint32_t q = 0; q < b; ++q) taken |= m.best[q] == s;
-        if (!taken && (bs == 0xFFFFFFFFu || det_before(d, s, bd, bs))) {
-          bd = d;
-          bs = s;
-        }
+  // the n_best lowest (det, start), in order: the block takes the first one after
+  // the one before it, n_best times
+  __shared__ double s_d[kFitWarps];
+  __shared__ uint32_t s_s[kFitWarps];
+  double pd = 0.0;
+  uint32_t ps = 0;
+  for (uint32_t b = 0; b < a.n_best; ++b) {
+    double bd = 0.0;
+    uint32_t bs = 0xFFFFFFFFu;
+    for (uint32_t s = threadIdx.x; s < a.n_starts; s += kFitThreads) {
+      const double d = det3[s];
+      if ((b == 0 || det_before(pd, ps, d, s)) && (bs == 0xFFFFFFFFu || det_before(d, s, bd, bs))) {
+        bd = d;
+        bs = s;
       }
-      for (int o = 16; o > 0; o >>= 1) {
-        const double od = __shfl_xor_sync(0xffffffffu, bd, o);
-        const uint32_t os = __shfl_xor_sync(0xffffffffu, bs, o);
-        if (os != 0xFFFFFFFFu && (bs == 0xFFFFFFFFu || det_before(od, os, bd, bs))) {
-          bd = od;
-          bs = os;
-        }
-      }
-      if (lane == 0) m.best[b] = bs;
-      __syncwarp();
     }
+    for (int o = 16; o > 0; o >>= 1) {
+      const double od = __shfl_xor_sync(0xffffffffu, bd, o);
+      const uint32_t os = __shfl_xor_sync(0xffffffffu, bs, o);
+      if (os != 0xFFFFFFFFu && (bs == 0xFFFFFFFFu || det_before(od, os, bd, bs))) {
+        bd = od;
+        bs = os;
+      }
+    }
+    if (lane == 0) {
+      s_d[warp] = bd;
+      s_s[warp] = bs;
+    }
+    __syncthreads();
+    bd = s_d[0];
+    bs = s_s[0];
+    for (int w = 1; w < kFitWarps; ++w)
+      if (s_s[w] != 0xFFFFFFFFu && (bs == 0xFFFFFFFFu || det_before(s_d[w], s_s[w], bd, bs))) {
+        bd = s_d[w];
+        bs = s_s[w];
+      }
+    pd = bd;
+    ps = bs;
+    if (threadIdx.x == 0) m.best[b] = bs;
+    __syncthreads();
   }
-  __syncthreads();
-  const Pts p{m.t, m.x, m.y, n, (n + 31) / 32};
+  narrow = __syncthreads_and(narrow);
+  const Pts p{m.t, m.x, m.y, n, (n + 31) / 32, narrow};
   const uint32_t h = (n + kDim + 1) / 2;
   const uint32_t b = blockIdx.x * kFitWarps + warp;
   if (b >= a.n_best) return;
@@ -436,10 +602,11 @@ __global__ void __launch_bounds__(32) k_fit_final(FitArgs a) {
   const uint32_t k = blockIdx.x;
   if (a.status[k] != kRunning) return;
   const FitSmem m = carve(smem, a.npad, 0);
-  const uint32_t n = load_points(a, k, m, threadIdx.x, 32);
+  bool narrow;
+  const uint32_t n = load_points(a, k, m, threadIdx.x, 32, &narrow);
   __syncwarp();
   const int lane = threadIdx.x;
-  const Pts p{m.t, m.x, m.y, n, (n + 31) / 32};
+  const Pts p{m.t, m.x, m.y, n, (n + 31) / 32, false};
   uint32_t bits;
   if (n < (uint32_t)kDim + 2) {
     bits = lane < (int)n ? 1u : 0u;  // n < 32: every point, one chunk

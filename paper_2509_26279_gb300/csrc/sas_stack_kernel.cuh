@@ -67,7 +67,12 @@ namespace {
 constexpr int kNT = 1024;
 // What the finish pass emits: super-bins at or over n_min (kModePlain), those and
 // the tile-local peaks (kModePeaks), blocks of cells (kModeWindows).
-enum { kModePlain = 0, kModePeaks = 1, kModeWindows = 2 };
+// kModePeaksWide: kModePeaks with counters that start at zero, so that they hold
+// 255 detections instead of 127 + n_low; n_low is found by adding 128 - n_low to
+// the low seven bits of every byte, two instructions more per word.  8-bit counters
+// then serve fields that needed 16-bit ones, at half the reductions and finish pass.
+enum { kModePlain = 0, kModePeaks = 1, kModeWindows = 2, kModePeaksWide = 3 };
+constexpr bool peak_mode(int mode) { return mode == kModePeaks || mode == kModePeaksWide; }
 constexpr int32_t kOutside = -(1 << 30);  // table entry of a lattice column that does not exist
 
 struct SmemLayout {
@@ -387,7 +392,9 @@ __device__ __forceinline__ void run_unit(const StackArgs& a, uint64_t unit, unsi
   const bool single_chunk = E <= (uint32_t)tc.ec;
   // counter start value: the top bit turns on when the count reaches n_low
   // (n_min with one threshold)
-  const uint32_t start = (1u << (CB - 1)) - a.n_low;
+  constexpr bool kWide = MODE == kModePeaksWide;
+  static_assert(!kWide || CB == 8, "wide counters are bytes");
+  const uint32_t start = kWide ? 0u : (1u << (CB - 1)) - a.n_low;
   uint32_t start_word = 0;
 #pragma unroll
   for (int q = 0; q < P; ++q) start_word |= start << (CB * q);
@@ -395,6 +402,11 @@ __device__ __forceinline__ void run_unit(const StackArgs& a, uint64_t unit, unsi
 #pragma unroll
   for (int q = 0; q < P; ++q) tmask |= (1u << (CB - 1)) << (CB * q);
   const uint4 start4 = make_uint4(start_word, start_word, start_word, start_word);
+  // the top bits of a word's counters that are at or over n_low
+  const uint32_t wide_bias = (128u - min(a.n_low, 128u)) * 0x01010101u;
+  auto tops = [&](uint32_t w) -> uint32_t {
+    return kWide ? ((((w & 0x7f7f7f7fu) + wide_bias) | w) & tmask) : w & tmask;
+  };
   if (init_cells) {  // first unit of this block, or of another field
     for (uint32_t i = tid; i < n_words / 4; i += kNT) reinterpret_cast<uint4*>(cells)[i] = start4;
     if (tid == 0) s_misc[43] = 0;
@@ -651,9 +663,9 @@ __device__ __forceinline__ void run_unit(const StackArgs& a, uint64_t unit, unsi
           const uint4 v = reinterpret_cast<const uint4*>(cells)[i];
           acc += (Acc)word_sum<CB>(v.x) + (Acc)word_sum<CB>(v.y) + (Acc)word_sum<CB>(v.z) + (Acc)word_sum<CB>(v.w);
           ++n_vec;
-          if ((v.x | v.y | v.z | v.w) & tmask) {
+          if (kWide ? tops(v.x) | tops(v.y) | tops(v.z) | tops(v.w) : (v.x | v.y | v.z | v.w) & tmask) {
             hit |= 1u << k;
-            ntop += __popc(v.x & tmask) + __popc(v.y & tmask) + __popc(v.z & tmask) + __popc(v.w & tmask);
+            ntop += __popc(tops(v.x)) + __popc(tops(v.y)) + __popc(tops(v.z)) + __popc(tops(v.w));
           } else {
             reinterpret_cast<uint4*>(cells)[i] = start4;
           }
@@ -678,7 +690,8 @@ __device__ __forceinline__ void run_unit(const StackArgs& a, uint64_t unit, unsi
           while (rr && idx < b0 + n_list) {
             const uint32_t k = (uint32_t)(__ffs(rr) - 1);
             rr &= rr - 1;
-            const uint4 v = reinterpret_cast<const uint4*>(cells)[k * kNT + tid];
+            uint4 v = reinterpret_cast<const uint4*>(cells)[k * kNT + tid];
+            if constexpr (kWide) v = make_uint4(tops(v.x), tops(v.y), tops(v.z), tops(v.w));
             uint32_t todo = 0;
 #pragma unroll
             for (int l = 0; l < P; ++l) {
@@ -805,7 +818,7 @@ __device__ __forceinline__ void run_unit(const StackArgs& a, uint64_t unit, unsi
     };
 
     auto finish = [&](int kx0, int ky0) {
-      if constexpr (MODE == kModePeaks) finish_peaks(kx0, ky0); else finish_plain(kx0, ky0);
+      if constexpr (peak_mode(MODE)) finish_peaks(kx0, ky0); else finish_plain(kx0, ky0);
     };
 
     const int nvt_bx = min(tc.bvx, (kxb - kxa) / KX + 1);
@@ -1195,7 +1208,7 @@ __global__ void __launch_bounds__(kNT, 1) k_stack(StackArgs a0, MultiArgs m) {
   // The next unit is drawn while the current one runs, so that nobody waits for
   // the counter's round trip (about 1500 cycles a unit) -- but for the peak tests,
   // whose registers are full.
-  constexpr bool kAhead = MODE != kModePeaks;
+  constexpr bool kAhead = !peak_mode(MODE);
   unsigned long long t_next = kAhead && tid == 0 ? atomicAdd(MULTI ? m.counter : a0.tile_counter, 1ull) : 0ull;
   while (true) {
     if (tid == 0) {
@@ -1223,7 +1236,7 @@ __global__ void __launch_bounds__(kNT, 1) k_stack(StackArgs a0, MultiArgs m) {
     const int field = s_field;
     if (local == ~0ull) break;
     if (MULTI && field != cur_field) {
-      if (MODE != kModePeaks && cur_field >= 0) {
+      if (!peak_mode(MODE) && cur_field >= 0) {
         report(s_args);
         __syncthreads();
       }
@@ -1239,10 +1252,10 @@ __global__ void __launch_bounds__(kNT, 1) k_stack(StackArgs a0, MultiArgs m) {
     else
       run_unit<KX, KY, CB, MODE>(a, local, smem, field != cur_field, balance, pairs64, my_flags);
     cur_field = field;
-    if constexpr (MODE == kModePeaks) report(a);  // its registers are short: no sums kept across units
+    if constexpr (peak_mode(MODE)) report(a);  // its registers are short: no sums kept across units
     __syncthreads();
   }
-  if (MODE != kModePeaks && cur_field >= 0) report(MULTI ? s_args : a0);
+  if (!peak_mode(MODE) && cur_field >= 0) report(MULTI ? s_args : a0);
 }
 
 template <int KX, int KY, int CB, int MODE>

@@ -25,6 +25,16 @@ cudaError_t launch_stack_multi_peaks(int kx, int ky, int cb, const StackArgs* fa
   return cudaErrorInvalidValue;
 }
 
+cudaError_t launch_stack_multi_wide(const StackArgs* fargs, const unsigned long long* unit_base, int n_fields,
+                                    unsigned long long* counter, size_t smem, int grid, cudaStream_t s) {
+  StackArgs proto{};
+  return launch_multi_t<8, 4, 8, kModePeaksWide>(proto, fargs, unit_base, n_fields, counter, smem, grid, s);
+}
+
+cudaError_t stack_set_smem_attr_wide(size_t smem) {
+  return raise_smem_limit((const void*)k_stack<8, 4, 8, true, kModePeaksWide>, smem);
+}
+
 cudaError_t stack_set_smem_attr_peaks(int kx, int ky, int cb, size_t smem) {
 #define SAS_ATTR(KX, KY, CB) if (kx == KX && ky == KY && cb == CB) return attr_t<KX, KY, CB, kModePeaks>(smem);
   SAS_STACK_CONFIGS(SAS_ATTR)

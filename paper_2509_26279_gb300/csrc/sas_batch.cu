@@ -28,6 +28,7 @@ struct sas_batch {
   std::vector<uint32_t> n_min;
   std::vector<sas_opts> opts;
   std::vector<FieldPlan> plans;
+  std::vector<FieldPlan> plans16;  // as planned, before a field's counters became wide
   std::vector<uint8_t> wide;   // field counts in 8-bit counters from zero (see sas_batch_create)
   std::vector<BatchField> hf;              // host copy of the field descriptors
   // Capacities of the arena: candidate-key slots per field (one power of two for
@@ -422,9 +423,11 @@ int sas_batch_create(const sas_grid* const* grids, const sas_catalog* cats, cons
     // tiles stay those of the 16-bit plan (the peaks are defined within them), the
     // reductions and the finish pass halve.  A wrap brings the 16 bits back (run).
     const bool wide = may_widen && fp.tc.cb == 16 && fp.tc.kx == 8 && fp.tc.ky == 4;
+    b->plans16.push_back(fp);
     if (wide) {
       fp.tc.cb = 8;
       fp.tc.smem = stack_smem_bytes(fp.tc);
+      one_epoch_chunk(desc, c.n, o, di, &fp);
     }
     b->wide.push_back(wide);
     b->plans.push_back(fp);
@@ -499,9 +502,7 @@ int sas_batch_run(sas_batch* b, void* stream) {
     b->ids_cap = ids_cap;
     free_pass(b);
     for (uint32_t f : narrow) {
-      TileCfg& tc = b->plans[f].tc;
-      tc.cb = 16;
-      tc.smem = stack_smem_bytes(tc);
+      b->plans[f] = b->plans16[f];
       b->wide[f] = 0;
     }
     if (!narrow.empty()) group_fields(b);

@@ -175,6 +175,8 @@ void bucket_grid(const sas_grid_desc& d, uint32_t E, int64_t dT, int64_t tph, Co
 bool magic_exact(int32_t bin, int64_t x_max);
 // log P(Poisson(lam) >= k)
 double log_poisson_tail(double lam, int k);
+// Fewer, taller bucket rows where that lets a unit take all its epochs at once.
+void one_epoch_chunk(const sas_grid_desc& d, uint64_t n, const sas_opts& o, const DevInfo& di, FieldPlan* fp);
 // Same plan with counters twice as wide (after a counter wrapped).
 int replan_wider(const sas_grid_desc& d, uint64_t n, uint32_t n_min, const sas_opts& o,
                  const DevInfo& di, FieldPlan* fp);

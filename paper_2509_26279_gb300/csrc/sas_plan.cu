@@ -241,6 +241,39 @@ void bucket_grid(const sas_grid_desc& d, uint32_t E, int64_t dT, int64_t tph, Co
   }
 }
 
+// A unit's epochs in one chunk.  With more epochs than its segments allow at the
+// plan's bucket rows, a unit was staged anew for every velocity tile of its block
+// and every chunk: 147 epochs against 128 cost 2.5 x per detection-shift.  Up to 256
+// epochs, fewer and taller bucket rows fit them all; the tiles stay as they are
+// (peak selection is defined within them), and the staging area gives up what
+// the longer shift tables take, if what the windows hold on average still fits.
+void one_epoch_chunk(const sas_grid_desc& d, uint64_t n, const sas_opts& o, const DevInfo& di, FieldPlan* fp) {
+  const uint32_t E = fp->g.E;
+  TileCfg tc = fp->tc;
+  if ((uint32_t)tc.ec >= E || E > (uint32_t)kMaxEpochChunk || o.coarse_bins) return;
+  const int64_t sbin = (int64_t)tc.s * d.bin, tw = tc.tx * sbin, th = tc.ty * sbin;
+  const int64_t spread_x = spread_bound((int64_t)(tc.bvx * tc.kx - 1) * std::llabs((int64_t)d.dvx), fp->dT, fp->g.tph);
+  const int64_t spread_y = spread_bound((int64_t)(tc.bvy * tc.ky - 1) * std::llabs((int64_t)d.dvy), fp->dT, fp->g.tph);
+  const int64_t rows = kSegCap / (int64_t)E;  // >= 4
+  CoarseGeom cg = fp->cg;
+  cg.cell = (int32_t)std::max<int64_t>(cg.cell, std::min<int64_t>((th + spread_y) / (rows - 2) + 1, kLimDomain));
+  bucket_grid(d, E, fp->dT, fp->g.tph, &cg);
+  tc.rows = (int)((th + spread_y) / cg.cell + 2);
+  if ((int64_t)tc.rows * E > kSegCap) return;
+  tc.ec = (int)E;
+  const double held = (double)n / ((double)d.nbx * d.bin * ((double)d.nby * d.bin)) * (double)(tw + spread_x) * (double)(th + spread_y);
+  const int64_t want = (int64_t)(1.15 * held) + kStackThreads, budget = (int64_t)di.smem_optin - 1024;
+  tc.scap = 0;
+  const int64_t room = (budget - (int64_t)stack_smem_bytes(tc)) / 8;
+  if (room < want) return;
+  tc.scap = (int)std::min<int64_t>(room, std::max<int64_t>(want, fp->tc.scap));
+  tc.smem = stack_smem_bytes(tc);
+  if ((int64_t)tc.smem > budget) return;
+  fp->tc = tc;
+  fp->cg = cg;
+  fp->nb = (uint64_t)E * cg.ncx * cg.ncy;
+}
+
 int plan_field(const sas_grid_desc& d, uint64_t n, uint32_t E, const int64_t* t, int64_t tph,
                uint32_t n_min, uint64_t v_begin, uint64_t v_end, const sas_opts& o,
                const DevInfo& di, FieldPlan* fp) {
@@ -297,6 +330,7 @@ int plan_field(const sas_grid_desc& d, uint64_t n, uint32_t E, const int64_t* t,
   g.nbx = (int32_t)d.nbx; g.nby = (int32_t)d.nby; g.bin = d.bin;
   g.E = E; g.tph = tph;
   g.v_begin = v_begin; g.v_end = v_end;
+  one_epoch_chunk(d, n, o, di, fp);
   return SAS_OK;
 }
 

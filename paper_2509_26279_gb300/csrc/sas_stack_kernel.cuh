@@ -494,8 +494,7 @@ __device__ __forceinline__ void run_unit(const StackArgs& a, uint64_t unit, unsi
     // --- stage detections [p0, p1) of the chunk that lie in the window, in
     //     bucket order (records of one epoch stay together, so the shift-table
     //     loads of a warp are broadcasts) ----------------------------------------
-    auto stage = [&](uint32_t e_base, uint32_t p0, uint32_t p1) -> uint32_t {
-      uint32_t n_kept = 0;
+    auto stage = [&](uint32_t e_base, uint32_t p0, uint32_t p1, uint32_t n_kept = 0) -> uint32_t {
       for (uint32_t j0 = p0; j0 < p1; j0 += kNT) {
         const uint32_t j = j0 + tid;
         uint32_t keep = 0;
@@ -825,8 +824,15 @@ __device__ __forceinline__ void run_unit(const StackArgs& a, uint64_t unit, unsi
     const int nvt_by = min(tc.bvy, (kyb - kya) / KY + 1);
     if (single_chunk) {
       const uint32_t D = prepare_chunk(0);
-      const bool once = D <= (uint32_t)tc.scap;
-      const uint32_t ns_once = once ? stage(0, 0, D) : 0u;  // staged once for the whole block
+      // staged once for the whole block when what the windows keep fits (the
+      // buckets hold some half more than the windows)
+      uint32_t ns_once = 0, staged_to = 0;
+      while (staged_to < D && ns_once + min(D - staged_to, (uint32_t)kNT) <= (uint32_t)tc.scap) {
+        const uint32_t to = min(D, staged_to + (uint32_t)kNT);
+        ns_once = stage(0, staged_to, to, ns_once);
+        staged_to = to;
+      }
+      const bool once = staged_to == D;
       for (int vty = 0; vty < nvt_by; ++vty)
         for (int vtx = 0; vtx < nvt_bx; ++vtx) {
           const int kx0 = kxa + vtx * KX, ky0 = kya + vty * KY;

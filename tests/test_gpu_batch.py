@@ -231,3 +231,34 @@ def test_batch_mixes_tile_shapes_and_counter_widths():
     assert widths == {(8, 16), (8, 8), (4, 16), (4, 8)}, widths
     assert b.stats()[1] == 0
     b.destroy()
+
+
+@pytest.mark.parametrize("epochs", [129, 170, 256])
+def test_many_epochs_in_one_chunk_and_wide_counters(epochs):
+    """Fields of more epochs than bucket rows of the usual height leave room for, with the peaks alone at a low threshold
+    (8-bit counters that start at zero) -- one of them with a cell that wraps such a counter, so that its 16-bit plan
+    comes back -- against the peak oracle with the tiles the batch reports."""
+    from oracle import lowpeaks as LP
+    fields, cats, specs = [], [], []
+    for i, extra in enumerate((0, 400)):
+        w = W.scaled(W.decam_tno(), frac_noise=0.03, width_px=500, height_px=400, n_epochs=epochs, n_movers=6,
+                     grid_half=9, seed=1900 + epochs + i)
+        cat = W.load(w)
+        if extra:  # 400 detections of one epoch in one super-bin
+            from tests import cases
+            cat = cases.catalog(np.r_[cat.x, np.full(extra, 100_500)], np.r_[cat.y, np.full(extra, 90_500)],
+                                np.r_[cat.epoch, np.zeros(extra, np.uint16)], cat.t, cat.ticks_per_hour)
+        x, y, e = _dev(cat)
+        fields.append((sas.Grid(w.grid), x, y, e, cat.t, cat.ticks_per_hour, 25))
+        cats.append(cat)
+        specs.append(w.grid)
+    b = sas.Batch(fields, opts=[sas.make_opts(n_low=10, peaks_only=1)] * 2)
+    b.run()
+    assert b.stats()[1] == 0 and b.rebuilds == (1 if epochs < 220 else 0)
+    for f, (cat, grid) in enumerate(zip(cats, specs)):
+        c, ids = b.candidates(f)
+        info = b.field_info(f)
+        ref = LP.search(cat, grid, 25, 10, LP.tiles_of(info), peaks_only=True)
+        assert len(ref.cands) > 0
+        _assert_oracle(c, ids, info["n_pairs"], ref)
+    b.destroy()

@@ -88,28 +88,51 @@ __device__ __forceinline__ float ld(const __nv_bfloat16* p) { return __bfloat162
 // bias + ReLU + BF16 rounding straight into the next layer's input layout.
 // Products are exact in FP32 and the sums accumulate in FP32.
 
-constexpr int kTcThreads = 512;   // 16 warps: 4 TMEM lane quadrants x 4 eight-channel slices
+//
+// Four stamps are in flight per SM: one CTA of four groups of 8 warps, each with its
+// own buffers, TMEM columns, mbarrier and named barrier, around one copy of the
+// weights (46 of 198 KB).  A group's chain -- build, MMAs, wait, TMEM loads, store, three
+// times a stamp -- is latency, which the other groups' work hides; with two CTAs of
+// 16 warps and a copy of the weights each, two stamps were in flight, the tensor
+// pipe 24 % and the issue slots 35 % busy.
+constexpr int kTcGroups = 4, kTcGrp = 256;  // 8 warps: 4 TMEM lane quadrants x 2 sixteen-channel halves
+constexpr int kTcThreads = kTcGroups * kTcGrp;
 constexpr int kTcRows0 = 288;     // x0: 15 x 15 pixels; tiles read up to row 2 * 128 - 1 + 2 * 15 + 2
 constexpr int kTcRows1 = 288;     // a1: 13 x 13 pixels; up to row 2 * 128 - 1 + 2 * 13 + 2
 constexpr int kTcRows2 = 160;     // a2: 11 x 11 pixels; up to row 127 + 2 * 11 + 2
 constexpr int kTcW1 = 9 * kCh * 16 * 2;   // per tap: 32 outputs x 16 input channels (9 real)
 constexpr int kTcW23 = 9 * kCh * kCh * 2; // per tap: 32 x 32
-constexpr int kSmX0 = 0;
-constexpr int kSmA1 = kSmX0 + 2 * kTcRows0 * 16;
-constexpr int kSmA2 = kSmA1 + 4 * kTcRows1 * 16;
-constexpr int kSmW1 = kSmA2 + 4 * kTcRows2 * 16;
+constexpr int kSmW1 = 0;
 constexpr int kSmW2 = kSmW1 + kTcW1;
 constexpr int kSmW3 = kSmW2 + kTcW23;
 constexpr int kSmBias = kSmW3 + kTcW23;
-constexpr int kSmBar = kSmBias + 3 * kCh * 4;
-constexpr int kTcSmem = kSmBar + 16;
-constexpr int kTcTmemCols = 256;  // conv1 tiles at columns 0, 32; conv2 at 64, 96; conv3 at 128
-static_assert(2 * kTcRows0 >= 2 * 128 + 2 * kS + 2 && kTcRows1 >= 2 * 128 + 2 * kH1 + 2 &&
+constexpr int kSmBar = kSmBias + 3 * kCh * 4;             // one mbarrier per group, then the TMEM base
+constexpr int kSmGrp = (kSmBar + 8 * kTcGroups + 16 + 127) / 128 * 128;
+constexpr int kGrX0 = 0;                                   // within a group's buffers
+constexpr int kGrA1 = kGrX0 + 2 * kTcRows0 * 16;
+constexpr int kGrA2 = kGrA1 + 4 * kTcRows1 * 16;
+constexpr int kGrBytes = kGrA2 + 4 * kTcRows2 * 16;
+constexpr int kTcSmem = kSmGrp + kTcGroups * kGrBytes;
+constexpr int kTcTmemCols = 512, kTcGrpCols = 128;  // per group: conv1 tiles at columns 0, 32; conv2 at 64, 96; conv3 at 0
+static_assert(kTcRows0 >= 2 * 128 + 2 * kS + 2 && kTcRows1 >= 2 * 128 + 2 * kH1 + 2 &&
                   kTcRows2 >= 128 + 2 * kH2 + 2, "shifted windows stay inside the buffers");
-static_assert(kTcRows0 >= 2 * 128 + 2 * kS + 2, "conv1 windows");
-static_assert(kSmW1 % 128 == 0 && kSmW2 % 128 == 0 && kSmW3 % 128 == 0 && kSmA1 % 16 == 0 &&
-                  kSmA2 % 16 == 0, "operand alignment");
-static_assert(2 * kTcSmem <= 227 * 1024, "two CTAs per SM");
+static_assert(kSmW1 % 128 == 0 && kSmW2 % 128 == 0 && kSmW3 % 128 == 0 && kGrA1 % 16 == 0 &&
+                  kGrA2 % 16 == 0 && kGrBytes % 128 == 0, "operand alignment");
+static_assert(kTcSmem <= 226 * 1024, "one CTA per SM");
+
+// Barrier of one group of kTcGrp threads; returns whether any of them passed `bad`.
+__device__ __forceinline__ bool group_sync_or(int group, bool bad) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\tbar.red.or.pred p, %2, %3, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r)
+      : "r"((uint32_t)bad), "r"(group + 1), "n"(kTcGrp)
+      : "memory");
+  return r != 0;
+}
+__device__ __forceinline__ void group_sync(int group) {
+  asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(kTcGrp) : "memory");
+}
 
 // Per-tap weights of a layer as the B operand: B_t[o][c] = w[o][c][t]; kc 16-byte
 // chunks per row (K = 8 kc; columns c >= cin stay as they are).  Read in memory order.
@@ -149,55 +172,57 @@ template <int NT, int W, int Rn>
 __device__ __forceinline__ void tc_conv_epi(uint32_t tmem_col, const float* bias, unsigned char* next,
                                             __nv_bfloat16* out_g) {
   constexpr int HO = W - 2;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp & 3, h = warp >> 2;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp & 3, h = (warp >> 2) & 1;
 #pragma unroll
   for (int t = 0; t < NT; ++t) {
-    float v[8];
-    tc::ld8(tmem_col + ((uint32_t)(q * 32) << 16) + (uint32_t)(t * 32 + h * 8), v);
+    float v[16];
+    tc::ld16(tmem_col + ((uint32_t)(q * 32) << 16) + (uint32_t)(t * 32 + h * 16), v);
     const int m = t * 128 + q * 32 + lane, y = m / W, x = m - y * W;
     if (y < HO && x < HO) {
       const int p = y * HO + x;
-      uint32_t pk[4];
+      uint32_t pk[8];
 #pragma unroll
-      for (int j = 0; j < 8; j += 2) {
-        const __nv_bfloat16 r0 = __float2bfloat16_rn(fmaxf(v[j] + bias[h * 8 + j], 0.f));
-        const __nv_bfloat16 r1 = __float2bfloat16_rn(fmaxf(v[j + 1] + bias[h * 8 + j + 1], 0.f));
+      for (int j = 0; j < 16; j += 2) {
+        const __nv_bfloat16 r0 = __float2bfloat16_rn(fmaxf(v[j] + bias[h * 16 + j], 0.f));
+        const __nv_bfloat16 r1 = __float2bfloat16_rn(fmaxf(v[j + 1] + bias[h * 16 + j + 1], 0.f));
         pk[j / 2] = (uint32_t)__bfloat16_as_ushort(r0) | ((uint32_t)__bfloat16_as_ushort(r1) << 16);
         if (out_g) {
-          out_g[(h * 8 + j) * HO * HO + p] = r0;
-          out_g[(h * 8 + j + 1) * HO * HO + p] = r1;
+          out_g[(h * 16 + j) * HO * HO + p] = r0;
+          out_g[(h * 16 + j + 1) * HO * HO + p] = r1;
         }
       }
-      if (next)
-        *reinterpret_cast<uint4*>(next + (h * Rn + p) * 16) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+      if (next) {
+        *reinterpret_cast<uint4*>(next + (2 * h * Rn + p) * 16) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        *reinterpret_cast<uint4*>(next + ((2 * h + 1) * Rn + p) * 16) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+      }
     }
   }
 }
 
-// One layer: operand visible to the tensor core, MMAs by thread 0, bounded
-// wait, epilogue.  Returns false (block-uniform) when the wait gave up.
+// One layer of a group: operand visible to the tensor core, MMAs by its first
+// thread, bounded wait, epilogue.  Returns false (group-uniform) when the wait gave up.
 template <int NT, int KS, int R, int W, int Rn>
-__device__ __forceinline__ bool tc_conv_layer(unsigned char* smc, int a_off, int w_off, uint32_t tmem_col,
-                                              uint64_t* bar, uint32_t& phase, const float* bias, int next_off,
-                                              __nv_bfloat16* out_g) {
+__device__ __forceinline__ bool tc_conv_layer(int group, const unsigned char* in, const unsigned char* w,
+                                              uint32_t tmem_col, uint64_t* bar, uint32_t& phase, const float* bias,
+                                              unsigned char* next, __nv_bfloat16* out_g) {
   tc::fence_smem_to_async();
   tc::fence_before_sync();
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  group_sync(group);
+  if ((threadIdx.x & (kTcGrp - 1)) == 0) {
     tc::fence_after_sync();
-    tc_conv_mma<NT, KS, R, W>(tc::smem_u32(smc + a_off), tc::smem_u32(smc + w_off), tmem_col);
+    tc_conv_mma<NT, KS, R, W>(tc::smem_u32(in), tc::smem_u32(w), tmem_col);
     tc::commit(bar);
   }
   const bool ok = tc::mbar_wait(bar, phase, 1u << 22);
   phase ^= 1u;
-  if (__syncthreads_or(!ok)) return false;
+  if (group_sync_or(group, !ok)) return false;
   tc::fence_after_sync();
-  tc_conv_epi<NT, W, Rn>(tmem_col, bias, next_off >= 0 ? smc + next_off : nullptr, out_g);
+  tc_conv_epi<NT, W, Rn>(tmem_col, bias, next, out_g);
   tc::fence_before_sync();
   return true;
 }
 
-__global__ void __launch_bounds__(kTcThreads, 2) k_conv_fwd_tc(const uint16_t* __restrict__ stamps,
+__global__ void __launch_bounds__(kTcThreads, 1) k_conv_fwd_tc(const uint16_t* __restrict__ stamps,
                                                                const uint32_t* __restrict__ idx, uint32_t n,
                                                                const __nv_bfloat16* __restrict__ wb,
                                                                __nv_bfloat16* a1g, __nv_bfloat16* a2g,
@@ -205,15 +230,17 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_conv_fwd_tc(const uint16_t* _
                                                                uint32_t* __restrict__ status) {
   extern __shared__ __align__(1024) unsigned char smc[];
   float* bias = reinterpret_cast<float*>(smc + kSmBias);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smc + kSmBar);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(smc + kSmBar + 8);
-  uint16_t* x0 = reinterpret_cast<uint16_t*>(smc + kSmX0);
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, group = tid / kTcGrp, gt = tid & (kTcGrp - 1);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smc + kSmBar) + group;
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(smc + kSmBar + 8 * kTcGroups);
+  unsigned char* buf = smc + kSmGrp + group * kGrBytes;
   if (tid < 32) tc::tmem_alloc(tslot, kTcTmemCols);
-  if (tid == 0) tc::mbar_init(bar, 1);
-  // activation buffers and conv1's weights: rows that are never written (input
-  // padding, channel padding) stay zero
+  if (gt == 0) tc::mbar_init(bar, 1);
+  // conv1's weights and the activation buffers: what is never written (channel and
+  // row padding) stays zero
   for (int i = tid; i < kSmW2 / 16; i += kTcThreads) reinterpret_cast<uint4*>(smc)[i] = make_uint4(0, 0, 0, 0);
+  for (int i = tid; i < kTcGroups * kGrBytes / 16; i += kTcThreads)
+    reinterpret_cast<uint4*>(smc + kSmGrp)[i] = make_uint4(0, 0, 0, 0);
   __syncthreads();
   tc_load_w_taps(wb + kW1, kQ, 2, smc + kSmW1);
   tc_load_w_taps(wb + kW2, kCh, 4, smc + kSmW2);
@@ -222,50 +249,62 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_conv_fwd_tc(const uint16_t* _
     const int l = tid / kCh, o = tid % kCh;
     bias[tid] = ld(wb + (l == 0 ? kB1 : l == 1 ? kB2 : kB3) + o);
   }
+  tc::fence_smem_to_async();
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  const uint32_t tmem = *tslot;
+  const uint32_t tmem = *tslot + (uint32_t)(group * kTcGrpCols);
   uint32_t phase = 0;
-  // each thread holds its share of the next stamp while the current one runs
-  constexpr int kPer = (kQ * kS * kS + kTcThreads - 1) / kTcThreads;
-  uint16_t nxt[kPer];
+  // A thread builds rows (8-channel chunk, pixel) gt and gt + 256 of x0, 16 bytes each,
+  // and holds the next stamp's counts while the current one runs.
+  constexpr int kPix = kS * kS;
+  uint32_t nxt[2][4];
   auto fetch = [&](uint32_t b) {
     if (b >= n) return;
-    const uint16_t* st = stamps + (size_t)(idx ? idx[b] : b) * kQ * kS * kS;
+    const uint16_t* st = stamps + (size_t)(idx ? idx[b] : b) * kQ * kPix;
 #pragma unroll
-    for (int r = 0; r < kPer; ++r) {
-      const int i = tid + r * kTcThreads;
-      nxt[r] = i < kQ * kS * kS ? st[i] : (uint16_t)0;
-    }
-  };
-  fetch(blockIdx.x);
-  for (uint32_t b = blockIdx.x; b < n; b += gridDim.x) {
-    // x0[chunk c / 8][row][c % 8] = count / 16 in BF16 (exact for counts <= 256 * 16)
+    for (int r = 0; r < 2; ++r) {
+      const int it = gt + r * kTcGrp, chunk = it / kPix, p = it - chunk * kPix;
 #pragma unroll
-    for (int r = 0; r < kPer; ++r) {
-      const int i = tid + r * kTcThreads;
-      if (i < kQ * kS * kS) {
-        const int c = i / (kS * kS), p = i - c * (kS * kS);
-        x0[((c >> 3) * kTcRows0 + p) * 8 + (c & 7)] =
-            __bfloat16_as_ushort(__float2bfloat16_rn((float)nxt[r] * 0.0625f));
+      for (int c = 0; c < 8; c += 2) {
+        const uint32_t v0 = chunk == 0 || (chunk == 1 && c == 0) ? st[(chunk * 8 + c) * kPix + p] : 0u;
+        const uint32_t v1 = chunk == 0 ? st[(c + 1) * kPix + p] : 0u;
+        nxt[r][c / 2] = v0 | (v1 << 16);
       }
     }
-    fetch(b + gridDim.x);
-    if (!tc_conv_layer<2, 1, kTcRows0, kS, kTcRows1>(smc, kSmX0, kSmW1, tmem, bar, phase, bias, kSmA1,
+  };
+  const uint32_t first = blockIdx.x + (uint32_t)group * gridDim.x, stride = kTcGroups * gridDim.x;
+  fetch(first);
+  for (uint32_t b = first; b < n; b += stride) {
+    // x0[chunk][row][channel] = count / 16 in BF16 (exact for counts <= 256 * 16)
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int it = gt + r * kTcGrp, chunk = it / kPix, p = it - chunk * kPix;
+      if (chunk < 2) {
+        uint32_t pk[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          pk[c] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn((float)(nxt[r][c] & 0xffffu) * 0.0625f)) |
+                  ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn((float)(nxt[r][c] >> 16) * 0.0625f)) << 16);
+        reinterpret_cast<uint4*>(buf + kGrX0)[chunk * kTcRows0 + p] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+      }
+    }
+    fetch(b + stride);
+    if (!tc_conv_layer<2, 1, kTcRows0, kS, kTcRows1>(group, buf + kGrX0, smc + kSmW1, tmem, bar, phase, bias, buf + kGrA1,
                                                      a1g ? a1g + (size_t)b * kCh * kH1 * kH1 : nullptr) ||
-        !tc_conv_layer<2, 2, kTcRows1, kH1, kTcRows2>(smc, kSmA1, kSmW2, tmem + 64, bar, phase, bias + kCh, kSmA2,
-                                                      a2g ? a2g + (size_t)b * kCh * kH2 * kH2 : nullptr) ||
-        !tc_conv_layer<1, 2, kTcRows2, kH2, 1>(smc, kSmA2, kSmW3, tmem + 128, bar, phase, bias + 2 * kCh, -1,
+        !tc_conv_layer<2, 2, kTcRows1, kH1, kTcRows2>(group, buf + kGrA1, smc + kSmW2, tmem + 64, bar, phase, bias + kCh,
+                                                      buf + kGrA2, a2g ? a2g + (size_t)b * kCh * kH2 * kH2 : nullptr) ||
+        !tc_conv_layer<1, 2, kTcRows2, kH2, 1>(group, buf + kGrA2, smc + kSmW3, tmem, bar, phase, bias + 2 * kCh, nullptr,
                                                a3g + (size_t)b * kF)) {
-      if (tid == 0) atomicOr(status, 1u);
+      if (gt == 0) atomicOr(status, 1u);
       break;
     }
-    __syncthreads();  // the next stamp's input overwrites x0, which the MMAs above read
+    // (the next stamp's x0 was read by MMAs that two waits have seen complete, and its
+    // first MMAs follow a group barrier behind this epilogue's TMEM loads)
   }
   tc::fence_before_sync();
   __syncthreads();
-  if (tid < 32) tc::tmem_free(tmem, kTcTmemCols);
+  if (tid < 32) tc::tmem_free(*tslot, kTcTmemCols);
 }
 
 // ---- forward: fc1 on the tensor cores, fc2 in the epilogue --------------------
@@ -1147,7 +1186,7 @@ int fwd_blocks() {
 cudaError_t forward(sas_vet* vt, const uint16_t* stamps, const uint32_t* idx, uint32_t n, bool keep,
                     float* logits, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  const int blocks = (int)std::min<uint32_t>(n, 2u * (uint32_t)fwd_blocks());  // two CTAs per SM
+  const int blocks = (int)std::min<uint32_t>(n, (uint32_t)fwd_blocks());
   k_conv_fwd_tc<<<blocks, kTcThreads, kTcSmem, s>>>(stamps, idx, n, vt->wb, keep ? vt->a1 : nullptr,
                                                    keep ? vt->a2 : nullptr, vt->a3, vt->status);
   const uint32_t tiles = (n + kFcTcRows - 1) / kFcTcRows, ldp = tiles * kFcTcRows;

@@ -73,6 +73,11 @@ static_assert((size_t)kFc1Slices * (kHid * kF + kHid) <= (size_t)kBackBlocks * k
 
 __device__ __forceinline__ float bf(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 __device__ __forceinline__ float ld(const __nv_bfloat16* p) { return __bfloat162float(*p); }
+// Two values rounded to BF16 in one word (one instruction).
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
 
 // ---- forward on the tensor cores: the three convolutions as implicit GEMMs ---
 //
@@ -183,12 +188,11 @@ __device__ __forceinline__ void tc_conv_epi(uint32_t tmem_col, const float* bias
       uint32_t pk[8];
 #pragma unroll
       for (int j = 0; j < 16; j += 2) {
-        const __nv_bfloat16 r0 = __float2bfloat16_rn(fmaxf(v[j] + bias[h * 16 + j], 0.f));
-        const __nv_bfloat16 r1 = __float2bfloat16_rn(fmaxf(v[j + 1] + bias[h * 16 + j + 1], 0.f));
-        pk[j / 2] = (uint32_t)__bfloat16_as_ushort(r0) | ((uint32_t)__bfloat16_as_ushort(r1) << 16);
+        pk[j / 2] = pack_bf16(fmaxf(v[j] + bias[h * 16 + j], 0.f), fmaxf(v[j + 1] + bias[h * 16 + j + 1], 0.f));
         if (out_g) {
-          out_g[(h * 16 + j) * HO * HO + p] = r0;
-          out_g[(h * 16 + j + 1) * HO * HO + p] = r1;
+          uint16_t* g = reinterpret_cast<uint16_t*>(out_g) + (h * 16 + j) * HO * HO + p;
+          g[0] = (uint16_t)pk[j / 2];
+          g[HO * HO] = (uint16_t)(pk[j / 2] >> 16);
         }
       }
       if (next) {
@@ -284,8 +288,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_fwd_tc(const uint16_t* _
         uint32_t pk[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c)
-          pk[c] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn((float)(nxt[r][c] & 0xffffu) * 0.0625f)) |
-                  ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn((float)(nxt[r][c] >> 16) * 0.0625f)) << 16);
+          // (2^23 + count) / 16 - 2^19 = count / 16, exactly: no integer conversion
+          pk[c] = pack_bf16(fmaf(__uint_as_float(0x4b000000u | (nxt[r][c] & 0xffffu)), 0.0625f, -524288.f),
+                            fmaf(__uint_as_float(0x4b000000u | (nxt[r][c] >> 16)), 0.0625f, -524288.f));
         reinterpret_cast<uint4*>(buf + kGrX0)[chunk * kTcRows0 + p] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
       }
     }
@@ -681,38 +686,63 @@ __global__ void k_fc1_sum(const float* __restrict__ part, uint32_t S, const floa
   }
 }
 
-// g3[b][k] = (sum_j g4[b][j] * fc1.w[j][k]) * (a3[b][k] > 0).
-// Block: 64 columns k x 32 stamps.
+// g3[b][k] = (sum_j g4[b][j] * fc1.w[j][k]) * (a3[b][k] > 0), in FP32 with j in order.
+// Block: 128 columns k x 64 stamps, 4 x 8 per thread: three 16-byte shared loads
+// feed 32 multiply-adds (one column x 8 stamps took nine loads for eight: 76 us for
+// 4096 stamps; the FP32 pipes need 17).
+constexpr int kDxCols = 128, kDxStamps = 64;
+constexpr int kDxSmem = kHid * (kDxCols + kDxStamps + 4) * 4;
+
 __global__ void __launch_bounds__(256) k_fc1_dx(const float* __restrict__ g4,
                                                 const __nv_bfloat16* __restrict__ wb,
                                                 const __nv_bfloat16* __restrict__ a3g, uint32_t n,
                                                 float* __restrict__ g3) {
-  __shared__ float Gs[32][kHid + 1];
-  __shared__ float Ws[kHid][64];
-  const int t = threadIdx.x, kk = t & 63, bg = t >> 6;
-  const int k0 = blockIdx.x * 64;
-  const uint32_t b0 = blockIdx.y * 32;
-  for (int i = t; i < 32 * kHid; i += 256) {
-    const uint32_t b = b0 + i / kHid;
-    Gs[i / kHid][i % kHid] = b < n ? g4[(size_t)b * kHid + i % kHid] : 0.f;
+  extern __shared__ __align__(16) float smx[];
+  float* Ws = smx;                      // [64 j][128 k]
+  float* Gs = smx + kHid * kDxCols;     // [64 j][64 stamps + 4]
+  constexpr int kG = kDxStamps + 4;
+  const int t = threadIdx.x, tx = t & 31, ty = t >> 5;
+  const int k0 = blockIdx.x * kDxCols;
+  const uint32_t b0 = blockIdx.y * kDxStamps;
+  for (int i = t; i < kHid * kDxCols / 4; i += 256) {  // four weights at a time (kF is a multiple of 4)
+    const int j = i / (kDxCols / 4), c = (i % (kDxCols / 4)) * 4;
+    uint2 w = make_uint2(0, 0);
+    if (k0 + c < kF) w = *reinterpret_cast<const uint2*>(wb + kWf1 + (size_t)j * kF + k0 + c);
+    *reinterpret_cast<float4*>(Ws + j * kDxCols + c) =
+        make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
+                    __uint_as_float(w.y & 0xffff0000u));
   }
-  for (int i = t; i < kHid * 64; i += 256) {
-    const int j = i / 64, k = k0 + i % 64;
-    Ws[j][i % 64] = k < kF ? ld(wb + kWf1 + (size_t)j * kF + k) : 0.f;
+  for (int i = t; i < kDxStamps * kHid; i += 256) {
+    const uint32_t r = i / kHid, j = i % kHid;
+    Gs[j * kG + r] = b0 + r < n ? g4[(size_t)(b0 + r) * kHid + j] : 0.f;
   }
   __syncthreads();
-  float acc[8] = {};
+  float acc[8][4] = {};
+#pragma unroll 4
   for (int j = 0; j < kHid; ++j) {
-    const float w = Ws[j][kk];
+    const float4 w = *reinterpret_cast<const float4*>(Ws + j * kDxCols + 4 * tx);
+    const float4 ga = *reinterpret_cast<const float4*>(Gs + j * kG + 8 * ty);
+    const float4 gb = *reinterpret_cast<const float4*>(Gs + j * kG + 8 * ty + 4);
+    const float g[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
 #pragma unroll
-    for (int s = 0; s < 8; ++s) acc[s] = fmaf(Gs[bg * 8 + s][j], w, acc[s]);
+    for (int s = 0; s < 8; ++s) {
+      acc[s][0] = fmaf(g[s], w.x, acc[s][0]);
+      acc[s][1] = fmaf(g[s], w.y, acc[s][1]);
+      acc[s][2] = fmaf(g[s], w.z, acc[s][2]);
+      acc[s][3] = fmaf(g[s], w.w, acc[s][3]);
+    }
   }
-  const int k = k0 + kk;
+  const int k = k0 + 4 * tx;
   if (k >= kF) return;
 #pragma unroll
   for (int s = 0; s < 8; ++s) {
-    const uint32_t b = b0 + bg * 8 + s;
-    if (b < n) g3[(size_t)b * kF + k] = ld(a3g + (size_t)b * kF + k) > 0.f ? acc[s] : 0.f;
+    const uint32_t b = b0 + 8 * ty + s;
+    if (b >= n) break;
+    const uint2 a = *reinterpret_cast<const uint2*>(a3g + (size_t)b * kF + k);
+    auto on = [](uint32_t bits) { return bits != 0u && bits < 0x8000u; };  // a > 0
+    *reinterpret_cast<float4*>(g3 + (size_t)b * kF + k) =
+        make_float4(on(a.x & 0xffffu) ? acc[s][0] : 0.f, on(a.x >> 16) ? acc[s][1] : 0.f,
+                    on(a.y & 0xffffu) ? acc[s][2] : 0.f, on(a.y >> 16) ? acc[s][3] : 0.f);
   }
 }
 
@@ -1164,6 +1194,8 @@ cudaError_t set_attrs() {
     e = cudaFuncSetAttribute(k_conv_back_tc<kH1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              ConvBack<kH1>::kSmem);
   if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_fc1_dx, cudaFuncAttributeMaxDynamicSharedMemorySize, kDxSmem);
+  if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_fc1_dw, cudaFuncAttributeMaxDynamicSharedMemorySize, kDwSmem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_conv1_dw_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kC1Smem);
@@ -1208,7 +1240,8 @@ cudaError_t gradients(sas_vet* vt, const uint16_t* stamps, const float* labels, 
   const uint32_t S = std::max<uint32_t>(1, std::min<uint32_t>(kFc1Slices, n / kDwChunk));
   k_fc1_dw<<<dim3(kDwTiles, S), kDwThreads, kDwSmem, s>>>(vt->g4, vt->a3, n, vt->partial, vt->status);
   k_fc1_sum<<<(kHid * kF + kHid + 255) / 256 + 1, 256, 0, s>>>(vt->partial, S, vt->lpart, n_loss, n, grad, vt->loss);
-  k_fc1_dx<<<dim3((kF + 63) / 64, (n + 31) / 32), 256, 0, s>>>(vt->g4, vt->wb, vt->a3, n, vt->g3);
+  k_fc1_dx<<<dim3((kF + kDxCols - 1) / kDxCols, (n + kDxStamps - 1) / kDxStamps), 256, kDxSmem, s>>>(
+      vt->g4, vt->wb, vt->a3, n, vt->g3);
   const int nb = (int)std::min<uint32_t>(n, kBackBlocks);
   const size_t per = (size_t)kBackBlocks * kPartialStride;
   k_conv_back_tc<kH2><<<nb, kBcThreads, ConvBack<kH2>::kSmem, s>>>(vt->g3, vt->a2, n, vt->wb + kW3, vt->g2,

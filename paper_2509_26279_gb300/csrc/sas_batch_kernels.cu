@@ -32,12 +32,6 @@ __device__ __forceinline__ Key max_key_b() {
   return k;
 }
 
-__device__ __forceinline__ bool key_less_b(const Key& p, const Key& q) {
-  if (p.a != q.a) return p.a < q.a;
-  if (p.b != q.b) return p.b < q.b;
-  return p.c < q.c;
-}
-
 // Validation, per-epoch counts and per-bucket counts of every detection.
 __global__ void k_batch_ingest(const BatchField* __restrict__ F, int n_fields,
                                const unsigned long long* __restrict__ det_off,

@@ -234,11 +234,7 @@ cudaError_t launch_stack_multi_wide(const StackArgs* fargs, const unsigned long 
 cudaError_t stack_set_smem_attr_wide(size_t smem);
 
 // sas_stack_windows.cu: the kernel over blocks of cells
-bool windows_config_supported(int kx, int ky, int cb);
 cudaError_t launch_stack_windows(const StackArgs& a, int grid, cudaStream_t s);
-cudaError_t launch_stack_multi_windows(int kx, int ky, int cb, const StackArgs* fargs,
-                                       const unsigned long long* unit_base, int n_fields,
-                                       unsigned long long* counter, size_t smem, int grid, cudaStream_t s);
 cudaError_t stack_set_smem_attr_windows(int kx, int ky, int cb, size_t smem);
 
 // ---- window search (sas_hier.cu) --------------------------------------------

@@ -19,8 +19,6 @@ size_t stack_smem_bytes(const TileCfg& tc) { return layout(tc).total; }
 
 size_t stack_counter_bytes(const TileCfg& tc) { return layout(tc).staged - layout(tc).cells; }
 
-int stack_threads() { return kNT; }
-
 cudaError_t launch_stack(const StackArgs& a, int grid, cudaStream_t s) {
   if (a.select != kSelectAll) return launch_stack_peaks(a, grid, s);
 #define SAS_LAUNCH(KX, KY, CB) \

@@ -9,13 +9,6 @@ namespace sas {
 
 #define SAS_WINDOW_CONFIGS(X) X(4, 4, 8) X(4, 4, 16)
 
-bool windows_config_supported(int kx, int ky, int cb) {
-#define SAS_CHECK(KX, KY, CB) if (kx == KX && ky == KY && cb == CB) return true;
-  SAS_WINDOW_CONFIGS(SAS_CHECK)
-#undef SAS_CHECK
-  return false;
-}
-
 cudaError_t launch_stack_windows(const StackArgs& a, int grid, cudaStream_t s) {
 #define SAS_LAUNCH(KX, KY, CB) \
   if (a.tc.kx == KX && a.tc.ky == KY && a.tc.cb == CB) return launch_t<KX, KY, CB, kModeWindows>(a, grid, s);
@@ -24,20 +17,10 @@ cudaError_t launch_stack_windows(const StackArgs& a, int grid, cudaStream_t s) {
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_stack_multi_windows(int kx, int ky, int cb, const StackArgs* fargs,
-                                       const unsigned long long* unit_base, int n_fields,
-                                       unsigned long long* counter, size_t smem, int grid, cudaStream_t s) {
-  StackArgs proto{};
-#define SAS_LAUNCH_M(KX, KY, CB)           \
-  if (kx == KX && ky == KY && cb == CB)    \
-    return launch_multi_t<KX, KY, CB, kModeWindows>(proto, fargs, unit_base, n_fields, counter, smem, grid, s);
-  SAS_WINDOW_CONFIGS(SAS_LAUNCH_M)
-#undef SAS_LAUNCH_M
-  return cudaErrorInvalidValue;
-}
-
 cudaError_t stack_set_smem_attr_windows(int kx, int ky, int cb, size_t smem) {
-#define SAS_ATTR(KX, KY, CB) if (kx == KX && ky == KY && cb == CB) return attr_t<KX, KY, CB, kModeWindows>(smem);
+#define SAS_ATTR(KX, KY, CB) \
+  if (kx == KX && ky == KY && cb == CB)    \
+    return raise_smem_limit((const void*)k_stack<KX, KY, CB, false, kModeWindows>, smem);
   SAS_WINDOW_CONFIGS(SAS_ATTR)
 #undef SAS_ATTR
   return cudaErrorInvalidValue;

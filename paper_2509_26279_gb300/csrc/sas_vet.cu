@@ -71,7 +71,6 @@ constexpr uint32_t kFc1Slices = 14;                  // stamp slices of the fc1 
 static_assert((size_t)kFc1Slices * (kHid * kF + kHid) <= (size_t)kBackBlocks * kPartialStride,
               "fc1 slices fit the partial buffer");
 
-__device__ __forceinline__ float bf(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 __device__ __forceinline__ float ld(const __nv_bfloat16* p) { return __bfloat162float(*p); }
 // Two values rounded to BF16 in one word (one instruction).
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {

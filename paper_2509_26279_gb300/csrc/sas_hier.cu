@@ -26,7 +26,11 @@
 //
 // plan_windows picks the group, the window side and the cell from the expected
 // instructions of both levels, and leaves the search to the one-level kernel
-// where the noise alone would fill the windows.  Everything stays exact whatever
+// where the noise alone would fill the windows.  At 2048 x 4096 px, 100 epochs and
+// 12,321 velocities level 1 takes 145 us and level 2 235 us, where the one-level
+// kernel and its exact counts took 1360 + 270 us; with a million velocities 8.9 ms
+// and 0.32 ms instead of 71.4 ms.  Level 1 is bound by shared memory and barriers
+// (58 % of the shared pipe, 48 % of the issue slots).  Everything stays exact whatever
 // the choice; a counter that wraps, a window list that overflows or a list
 // longer than a warp holds sets kFlagWindow and the host runs the one-level
 // search instead.
@@ -201,9 +205,47 @@ struct WarpList {
   int32_t first[16], off[16], len0[16], len1[16];
 };
 
+// The runs of bucketed detections under a window at an epoch: at most two bucket
+// rows (a bucket is no smaller than a window), and the window's corner there.
+struct Runs {
+  uint32_t k, k1, j, j1;
+  int32_t ox, oy;
+};
+__device__ __forceinline__ Runs window_runs(const WindowArgs& a, const int32_t* SX, const int32_t* SY, uint32_t e,
+                                            int32_t ux0, int32_t uy0, int span, uint64_t cell_m) {
+  Runs r{};
+  if (e >= a.g.E || a.ecount[e] == 0) return r;
+  const CoarseGeom& cg = a.cg;
+  r.ox = ux0 + SX[e];
+  r.oy = uy0 + SY[e];
+  int cxa, cxb, cya, cyb;
+  bucket_range(r.ox - cg.gx0, span, cell_m, cg.ncx, cxa, cxb);
+  bucket_range(r.oy - cg.gy0, span, cell_m, cg.ncy, cya, cyb);
+  if (cxa > cxb || cya > cyb) return r;
+  const uint32_t* row = a.boff + ((size_t)e * cg.ncy + cya) * cg.ncx;
+  r.k = row[cxa];
+  r.k1 = row[cxb + 1];
+  if (cyb > cya) {
+    row += cg.ncx;
+    r.j = row[cxa];
+    r.j1 = row[cxb + 1];
+  }
+  return r;
+}
+
+constexpr int32_t kOutside = INT32_MIN / 2;  // in no bin, whatever a group's edge adds
+
 // W: weighted stacking.  A bin's sum of weights takes the place of its raw count
 // (the masks are counted once per bit of the weights), and the sum of its
 // epochs' largest weights that of its distinct epochs.
+//
+// What bounds it: instruction issue (65 % of the slots at 2048 x 4096 px, 100 epochs,
+// 12,321 velocities) and the latency of each window's chain of loads.  Four blocks
+// of eight warps an SM; five left fewer registers and were no faster.  Windows
+// drawn one by one in a block, records and offsets asked for one turn ahead: 292 ->
+// 235 us there, 528 -> 400 us with weights, 380 -> 320 us for a million velocities.
+// (Two records a turn cost more instructions than it hid: 277 us, and 107 -> 128 us
+// where runs are short.)
 template <bool W>
 __global__ void __launch_bounds__(kWarps * 32, 4) k_window_cells(WindowArgs a, uint64_t cell_m) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -211,14 +253,25 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_window_cells(WindowArgs a, u
   WarpList<W>& L = reinterpret_cast<WarpList<W>*>(smem)[threadIdx.x >> 5];
   const uint32_t lt = (1u << lane) - 1u;
   const SearchGeom& g = a.g;
-  const CoarseGeom& cg = a.cg;
   const uint32_t E = g.E;
   const int P = a.cgm.bin, span = a.win * P, nvg = a.gx * a.gy;
   const uint32_t n_win = min(*a.n_windows, a.list_cap);
   unsigned long long raw_sum = 0;
   constexpr int kSeen = W ? 256 : 8;
   for (int i = lane; i < kSeen; i += 32) L.seen[i] = 0;
-  for (uint32_t w = blockIdx.x * kWarps + (threadIdx.x >> 5); w < n_win; w += gridDim.x * kWarps) {
+  // sides of a group are powers of two
+  const int lgx = __ffs(a.gx) - 1, jx = lane & (a.gx - 1);
+  const int jy0 = min(lane >> lgx, a.gy - 1), jy1 = min((lane + 32) >> lgx, a.gy - 1);
+  // A block takes every gridDim.x-th row of kWarps windows; its warps draw them one by
+  // one, as windows on a mover's track cost several times the others.
+  __shared__ uint32_t drawn;
+  if (threadIdx.x == 0) drawn = kWarps;
+  __syncthreads();
+  uint32_t i_win = threadIdx.x >> 5, ahead = 0;
+  for (;; i_win = __shfl_sync(0xffffffffu, ahead, 0)) {
+    const uint64_t w = ((uint64_t)(i_win / kWarps) * gridDim.x + blockIdx.x) * kWarps + i_win % kWarps;
+    if (w >= n_win) break;
+    if (lane == 0) ahead = atomicAdd(&drawn, 1u);
     const Emit em = a.windows[w];
     const int Kx = (int)(em.v_idx % (uint32_t)a.cgm.nvx), Ky = (int)(em.v_idx / (uint32_t)a.cgm.nvx);
     const int32_t ux0 = a.cgm.x_min + (int32_t)em.bx * P, uy0 = a.cgm.y_min + (int32_t)em.by * P;
@@ -242,56 +295,36 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_window_cells(WindowArgs a, u
       L.len0[lane] = own > 0 ? a.unit : 0;
       L.len1[lane] = own > 1 ? a.unit : 0;
     }
-    // the window's detections, 32 epochs at a time
+    // The window's detections, a lane per epoch.  The chain of loads (shift, bucket
+    // offsets, records) is what a window waits for, so the next 32 epochs' offsets
+    // are asked for before these ones' records are walked, and each record before the
+    // one ahead of it is looked at.
     const int32_t* SX = a.sXt + (size_t)Kx * E;
     const int32_t* SY = a.sYt + (size_t)Ky * E;
+    Runs next = window_runs(a, SX, SY, lane, ux0, uy0, span, cell_m);
     uint32_t n = 0;
     for (uint32_t eb = 0; eb < E; eb += 32) {
       const uint32_t e = eb + lane;
-      // the buckets under the window: at most two rows (a bucket is no smaller
-      // than a window), each a contiguous run of detections
-      uint32_t k = 0, k1 = 0, j = 0, j1 = 0;
-      int32_t ox = 0, oy = 0;
-      if (e < E && a.ecount[e] > 0) {
-        ox = ux0 + SX[e];
-        oy = uy0 + SY[e];
-        int cxa, cxb, cya, cyb;
-        bucket_range(ox - cg.gx0, span, cell_m, cg.ncx, cxa, cxb);
-        bucket_range(oy - cg.gy0, span, cell_m, cg.ncy, cya, cyb);
-        if (cxa <= cxb && cya <= cyb) {
-          const uint32_t* row = a.boff + ((size_t)e * cg.ncy + cya) * cg.ncx;
-          k = row[cxa];
-          k1 = row[cxb + 1];
-          if (cyb > cya) {
-            row += cg.ncx;
-            j = row[cxa];
-            j1 = row[cxb + 1];
-          }
-        }
-      }
-      while (__any_sync(0xffffffffu, k < k1 || j < j1)) {
-        if (k == k1) {
-          k = j;
-          k1 = j1;
-          j = j1;
-        }
-        bool hit = false;
-        int32_t X = 0, Y = 0;
-        uint32_t id = 0;
-        if (k < k1) {
-          const int4 d = *reinterpret_cast<const int4*>(a.dets + k++);
-          id = (uint32_t)d.w;
-          X = d.x - ox;
-          Y = d.y - oy;
-          hit = (uint32_t)X < (uint32_t)span && (uint32_t)Y < (uint32_t)span;
-        }
+      const Runs r = next;
+      if (eb + 32 < E) next = window_runs(a, SX, SY, e + 32, ux0, uy0, span, cell_m);
+      const uint32_t na = r.k1 - r.k, total = na + (r.j1 - r.j);
+      const int4* ra = reinterpret_cast<const int4*>(a.dets) + r.k;
+      const int4* rb = reinterpret_cast<const int4*>(a.dets) + r.j - na;
+      const uint32_t most = __reduce_max_sync(0xffffffffu, total);
+      int4 ahead_d{};
+      if (total > 0) ahead_d = *(na > 0 ? ra : rb);
+      for (uint32_t q = 0; q < most; ++q) {
+        const int4 d = ahead_d;
+        if (q + 1 < total) ahead_d = (q + 1 < na ? ra : rb)[q + 1];
+        const int32_t X = d.x - r.ox, Y = d.y - r.oy;
+        const bool hit = q < total && (uint32_t)X < (uint32_t)span && (uint32_t)Y < (uint32_t)span;
         const uint32_t m = __ballot_sync(0xffffffffu, hit);
         const uint32_t p = n + (uint32_t)__popc(m & lt);
         if (hit && p < kList) {
           L.x[p] = X;
           L.y[p] = Y;
           L.e[p] = (uint8_t)e;
-          if constexpr (W) L.w[p] = a.wts[id];
+          if constexpr (W) L.w[p] = a.wts[(uint32_t)d.w];
         }
         n += (uint32_t)__popc(m);
       }
@@ -310,27 +343,34 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_window_cells(WindowArgs a, u
     // and its row's mask share.  Some 250 instructions per 32 detections for up to 256
     // bins, where counting the detections one by one into packed counters took 1100.
     uint32_t raw[2][kMaxOwn][kMaxOwn] = {};
-    const int jx = lane % a.gx, jy0 = min(lane / a.gx, a.gy - 1), jy1 = min((lane + 32) / a.gx, a.gy - 1);
     for (uint32_t i0 = 0; i0 < n; i0 += 32) {
       const uint32_t i = i0 + lane;
       const uint32_t e = i < n ? L.e[i] : 0;
       const int32_t xs = i < n ? L.x[i] + SX[e] : 0, ys = i < n ? L.y[i] + SY[e] : 0;
       const int32_t* sx = a.sxt + (size_t)(Kx * a.gx) * E + e;
       const int32_t* sy = a.syt + (size_t)(Ky * a.gy) * E + e;
+      const int cols = i < n ? min(a.gx, g.nvx - Kx * a.gx) : 0, rows = i < n ? min(a.gy, g.nvy - Ky * a.gy) : 0;
+      int32_t tx[8], ty[8];  // all loads first, whatever the group's sides
+#pragma unroll
+      for (int j = 0; j < 8; ++j) tx[j] = j < cols ? xs - sx[(size_t)j * E] : kOutside;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) ty[j] = j < rows ? ys - sy[(size_t)j * E] : kOutside;
       uint32_t mine = 0;
-#pragma unroll 8
-      for (int j = 0; j < a.gx; ++j) {
-        const int32_t t = i < n && Kx * a.gx + j < g.nvx ? xs + L.off[j] - sx[(size_t)j * E] : -1;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        if (j >= a.gx) break;
+        const int32_t t = tx[j] + L.off[j];
         const uint32_t m0 = __ballot_sync(0xffffffffu, (uint32_t)t < (uint32_t)L.len0[j]);
         const uint32_t m1 = __ballot_sync(0xffffffffu, (uint32_t)(t - a.unit) < (uint32_t)L.len1[j]);
-        mine = lane == 2 * j ? m0 : lane == 2 * j + 1 ? m1 : mine;
+        if (lane >> 1 == j) mine = lane & 1 ? m1 : m0;
       }
-#pragma unroll 8
-      for (int j = 0; j < a.gy; ++j) {
-        const int32_t t = i < n && Ky * a.gy + j < g.nvy ? ys + L.off[8 + j] - sy[(size_t)j * E] : -1;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        if (j >= a.gy) break;
+        const int32_t t = ty[j] + L.off[8 + j];
         const uint32_t m0 = __ballot_sync(0xffffffffu, (uint32_t)t < (uint32_t)L.len0[8 + j]);
         const uint32_t m1 = __ballot_sync(0xffffffffu, (uint32_t)(t - a.unit) < (uint32_t)L.len1[8 + j]);
-        mine = lane == 16 + 2 * j ? m0 : lane == 17 + 2 * j ? m1 : mine;
+        if (lane >> 1 == 8 + j) mine = lane & 1 ? m1 : m0;
       }
       uint32_t both[2][kMaxOwn][kMaxOwn];
 #pragma unroll
@@ -370,7 +410,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_window_cells(WindowArgs a, u
       const int b = __ffs(__shfl_sync(0xffffffffu, todo, src)) - 1;
       if (lane == src) todo &= todo - 1;
       const int v = src + (b & 4 ? 32 : 0), c = b & 1, r = (b >> 1) & 1;
-      const int kx = v % a.gx, ky = v / a.gx;
+      const int kx = v & (a.gx - 1), ky = v >> lgx;
       const int32_t* sx = a.sxt + (size_t)(Kx * a.gx + kx) * E;
       const int32_t* sy = a.syt + (size_t)(Ky * a.gy + ky) * E;
       const int32_t ax = L.off[kx] - c * a.unit, ay = L.off[8 + ky] - r * a.unit;

@@ -101,7 +101,11 @@ typedef struct sas_catalog {
 } sas_catalog;
 
 /* Optional knobs of sas_stack (pass NULL for defaults).  Tile fields of 0 let
- * the library choose (built-in table or the autotuner cache). */
+ * the library choose (built-in table or the autotuner cache).  A search with all
+ * tile fields 0 and one threshold may run in two levels (groups of velocities
+ * over coarse cells first, then the velocities and bins of the cells that can
+ * reach N_min); a tile field that is set, n_low or peaks_only keep the search to
+ * one level over the tiles that the result's info names. */
 typedef struct sas_opts {
   uint64_t v_begin, v_end;   /* search only lattice indices [v_begin, v_end); 0,0 = all */
   uint64_t max_candidates;   /* keep the first K candidates in output order; 0 = all    */
@@ -137,15 +141,17 @@ typedef struct sas_result_info {
   uint64_t n_candidates;     /* after the optional top-K cut                      */
   uint64_t n_ids;            /* total contributing ids of those candidates        */
   uint64_t n_pairs;          /* in-domain (detection, velocity) pairs = detection-shifts */
-  uint64_t n_emitted;        /* cells that crossed the counter threshold (superset) */
+  uint64_t n_emitted;        /* counters that crossed the threshold (a superset: super-bins,
+                                or the windows of a two-level search)               */
   int64_t t0;                /* reference epoch (ticks)                           */
   uint32_t counter_bits;     /* counter width the stack kernel ran with           */
-  uint32_t tile_kx, tile_ky, tile_bx, tile_by;  /* the plan it ran with             */
+  uint32_t tile_kx, tile_ky, tile_bx, tile_by;  /* the one-level plan               */
   uint32_t superbin;         /* bins per counter side                             */
   uint32_t vblock_x, vblock_y;  /* velocity tiles per staged detection set          */
   uint32_t staged_cap;       /* staged detection records per CTA                  */
   uint32_t n_low;            /* lower threshold of the peak selection (n_min when off) */
-  float ms_stack;            /* device time of the stack kernel (CUDA events)     */
+  float ms_stack;            /* device time of the stack kernels (CUDA events; both
+                                levels, exact counts included, of a two-level search) */
   float ms_total;            /* device time of the whole call                     */
   float ms_prep;             /* ingest, buckets, reference epoch, shift tables    */
   float ms_count;            /* exact counts of emitted cells + ordering          */
@@ -253,7 +259,9 @@ void sas_result_free(sas_result* result);
  * sas_batch_run replays the pass on `stream` and synchronizes; a field that
  * exceeded the batch's fixed capacities (emissions, 32768 candidates, ids) or
  * whose counters wrapped is recomputed by sas_stack, so every field's result
- * equals sas_stack's.  Results stay valid until the next run.
+ * equals sas_stack's.  (Peak-selected fields of 129 to 255 epochs count in 8 bits
+ * from zero on the tiles of their 16-bit plan; if such a counter wraps, the batch
+ * is rebuilt once with 16-bit counters for them and replayed.)  Results stay valid until the next run.
  * Errors: as sas_stack; SAS_ERR_ARG for fields that cannot share a launch. */
 typedef struct sas_batch sas_batch;
 int sas_batch_create(const sas_grid* const* grids, const sas_catalog* cats, const uint32_t* n_min,
@@ -306,7 +314,10 @@ int sas_batch_vet(const sas_batch* batch, sas_vet* vetter, uint32_t* field_out, 
  * rejects for this field are skipped.  `reps` timed runs each after one
  * warm-up; *best gets the options with the lowest median device time of the
  * whole search (*best_ms).  Every combination gives the same candidates
- * (Sec. 2.1 steps 1-3 are independent of the tiling); only the speed differs. */
+ * (Sec. 2.1 steps 1-3 are independent of the tiling); only the speed differs.
+ * Every combination searches in one level (sas_opts): it tunes fields of a batch
+ * and searches with a lowered threshold, while a single search with one threshold
+ * is usually fastest with no tile option set. */
 int sas_autotune(const sas_grid* grid, const sas_catalog* cat, uint32_t n_min,
                  const sas_opts* base, uint32_t reps, void* stream, sas_opts* best,
                  float* best_ms);
@@ -551,9 +562,10 @@ int sas_param_dx_scan(double nu, double nu_th, const double* a, uint32_t n_epoch
  * Arithmetic: the kernels use BF16 copies of the weights (round to nearest
  * even), round the input and every stored activation to BF16 and accumulate
  * in FP32.  The forward convolutions and fc1 run on the tensor cores (tcgen05,
- * BF16 operands); deltas and gradients are FP32, and the backward of conv2 and
- * conv3 runs on the tensor cores with TF32 operands (the deltas round to TF32
- * there).  Adam updates the FP32 masters and refreshes the BF16 copies.
+ * BF16 operands); deltas and gradients are FP32.  The backward of conv2 and conv3
+ * cuts the deltas to TF32 and multiplies them, as two BF16 parts that add up to
+ * the cut value, on the tensor cores; the weight gradients of conv1 and fc1 take
+ * the FP32 deltas as three BF16 parts that add up to them exactly.  Adam updates the FP32 masters and refreshes the BF16 copies.
  * Gradients are bit-reproducible for a batch.
  * A vetter lives on the device that was current at sas_vet_create; every call
  * makes that device current for its duration. */

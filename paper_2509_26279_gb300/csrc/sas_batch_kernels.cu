@@ -153,7 +153,7 @@ constexpr int kWarps = 8;
 // Exact counts of every bin of every emitted super-bin of every field; one warp
 // per emission slot (slots beyond a field's emission count exit).
 // Grid: x blocks per field, y = field; each warp walks the field's emissions.
-__global__ void k_batch_cell_count(const BatchField* __restrict__ F, const Det* __restrict__ dets,
+__global__ void __launch_bounds__(kWarps * 32, 4) k_batch_cell_count(const BatchField* __restrict__ F, const Det* __restrict__ dets,
                                    const uint32_t* __restrict__ boff) {
   const int lane = threadIdx.x & 31;
   const BatchField& bf = F[blockIdx.y];
@@ -163,7 +163,7 @@ __global__ void k_batch_cell_count(const BatchField* __restrict__ F, const Det* 
   const uint64_t cell_m = div_magic((uint32_t)cg.cell), bin_m = div_magic((uint32_t)g.bin);
   for (uint32_t j = blockIdx.x * kWarps + (threadIdx.x >> 5); j < n_emit; j += gridDim.x * kWarps) {
     const Emit em = bf.args.emits[j];
-    count_superbin(em, bf.args.tc.s, g, cg, cell_m, bin_m, dets, boff + bf.bucket_base, bf.ecount, bf.sxt,
+    count_superbin<false, true>(em, bf.args.tc.s, g, cg, cell_m, bin_m, dets, boff + bf.bucket_base, bf.ecount, bf.sxt,
                    bf.syt, (em.flags & kEmitLowPeak) ? bf.args.n_low : bf.args.n_min, lane,
                    [&](int, uint32_t bx, uint32_t by, uint32_t distinct, uint32_t raw) {
                      Key k;

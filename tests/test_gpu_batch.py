@@ -262,3 +262,25 @@ def test_many_epochs_in_one_chunk_and_wide_counters(epochs):
         assert len(ref.cands) > 0
         _assert_oracle(c, ids, info["n_pairs"], ref)
     b.destroy()
+
+
+@pytest.mark.parametrize("superbin,coarse", [(4, 1), (4, 2), (3, 1), (1, 1)])
+def test_counts_over_buckets_smaller_than_a_super_bin(superbin, coarse):
+    """A batch's exact counts walk two bucket rows per epoch ahead of use and any further rows (up to five under a
+    4 x 4 super-bin over one-bin buckets) after them; 1, 31, 33 and 65 epochs end inside and past a block of 32."""
+    fields, refs = [], []
+    for E in (1, 31, 33, 65):
+        w = W.scaled(W.decam_tno(), frac_noise=0.05, width_px=260, height_px=190, n_epochs=E, n_movers=4,
+                     grid_half=4, seed=3100 + E)
+        cat, n_min = W.load(w), max(1, min(5, E // 6))
+        x, y, e = _dev(cat)
+        fields.append((sas.Grid(w.grid), x, y, e, cat.t, cat.ticks_per_hour, n_min))
+        refs.append(oracle.stack(cat, w.grid, n_min))
+    b = sas.Batch(fields, opts=[sas.make_opts(superbin=superbin, coarse_bins=coarse, tile_bx=8, tile_by=8)] * len(fields))
+    b.run()
+    assert b.stats()[1] == 0
+    for f, ref in enumerate(refs):
+        assert len(ref.cands) > 0
+        c, ids = b.candidates(f)
+        _assert_oracle(c, ids, b.field_info(f)["n_pairs"], ref)
+    b.destroy()

@@ -557,6 +557,7 @@ double window_tiles(const sas_grid_desc& d, uint64_t n, uint64_t Ky_lo, uint64_t
     if ((double)tw + sx >= (double)(1 << 24) || (double)th + sy >= (double)(1 << 24)) continue;
     const double cell = std::max(std::ceil(((double)th + sy) / (rows - 2)), (double)(wp->win * g.bin));
     const double units = vtiles * ntx * nty;
+    if (units > (double)UINT32_MAX) continue;  // the kernel numbers its units in 32 bits
     const double records = per_px2 * ((double)tw + sx + cell) * ((double)th + sy + cell);
     const double cost = std::ceil(units / di.sms) * (9000.0 + (double)tc.tx * tc.ty * 0.85 * (cb / 8) + records * 2.5);
     if (best != 0 && cost >= best) continue;

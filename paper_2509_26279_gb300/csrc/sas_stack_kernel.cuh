@@ -1253,7 +1253,7 @@ __global__ void __launch_bounds__(kNT, 1) k_stack(StackArgs a0, MultiArgs m) {
     }
     const StackArgs& a = MULTI ? s_args : a0;
     if (kAhead && tid == 0) t_next = atomicAdd(MULTI ? m.counter : a0.tile_counter, 1ull);
-    if constexpr (MODE == kModeWindows)
+    if constexpr (MODE == kModeWindows)  // plan_windows takes no search of 2^32 units
       run_unit_windows<KX, KY, CB>(a, (uint32_t)local, smem, field != cur_field, balance, pairs64, my_flags);
     else
       run_unit<KX, KY, CB, MODE>(a, local, smem, field != cur_field, balance, pairs64, my_flags);

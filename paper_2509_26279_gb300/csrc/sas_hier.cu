@@ -35,6 +35,7 @@
 // longer than a warp holds sets kFlagWindow and the host runs the one-level
 // search instead.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdlib>
 
@@ -572,6 +573,13 @@ double window_tiles(const sas_grid_desc& d, uint64_t n, uint64_t Ky_lo, uint64_t
   return wp->tc.rows * (int)E > wp->tc.seg_cap ? 0 : best;
 }
 
+// Twice the centre velocity of every group of grp lattice steps, times any dt in
+// [0, dT], fits 64 bits.
+bool centre_fits(int32_t v0, int32_t dv, uint32_t nv, int grp, int64_t dT) {
+  const double most = 2.0 * std::fabs((double)v0) + 2.0 * ((double)nv + grp) * std::fabs((double)dv);
+  return most * (double)dT < 9.0e18;
+}
+
 }  // namespace
 
 bool plan_windows(const sas_grid_desc& d, uint64_t n, uint32_t n_min, double mean_weight, uint64_t v_begin,
@@ -604,6 +612,10 @@ bool plan_windows(const sas_grid_desc& d, uint64_t n, uint32_t n_min, double mea
       for (int win = 2; win <= 3; ++win) {
         const int gx = 1 << lx, gy = 1 << ly;
         if (gx * gy == 1 || (square && gx != gy)) continue;
+        // steps of a group are 32-bit; twice its centre velocity times dt (k_window_tables) is 64-bit
+        if (gx * std::llabs((int64_t)d.dvx) > INT32_MAX || gy * std::llabs((int64_t)d.dvy) > INT32_MAX ||
+            !centre_fits(d.vx0, d.dvx, d.nvx, gx, fp.dT) || !centre_fits(d.vy0, d.dvy, d.nvy, gy, fp.dT))
+          continue;
         const double hx = 0.5 * (gx - 1) * std::fabs((double)d.dvx) * hour, hy = 0.5 * (gy - 1) * std::fabs((double)d.dvy) * hour;
         const double side = std::ceil(((double)unit + std::max(hx, hy) + 2.0) / (win - 1));
         if (side > (double)(kMaxOwn * unit) || side * win >= (double)(1 << 20)) continue;

@@ -936,7 +936,7 @@ __device__ __forceinline__ void run_unit_windows(const StackArgs& a, uint32_t un
       const int32_t t0 = a.syt[(size_t)ky0 * E + e], t1 = a.syt[(size_t)kyb * E + e];
       bucket_range(X0 + min(s0, s1) - cg.gx0, abs(s1 - s0) + (int32_t)tw_x, a.cell_m, cg.ncx, r.x, r.y);
       bucket_range(Y0 + min(t0, t1) - cg.gy0, abs(t1 - t0) + (int32_t)tw_y, a.cell_m, cg.ncy, r.z, r.w);
-      if (r.w - r.z >= tc.rows) my_flags |= kFlagInternal;
+      if (r.w - r.z >= tc.rows) my_flags |= kFlagWindow;  // more bucket rows than planned for
     }
     s_win[e] = r;
   }

@@ -50,3 +50,19 @@ def test_more_than_32_bits_of_units(plan, n):
     size do not fit the 32 bits that its kernel numbers them with."""
     p = plan(n, 100, 14_400, 25, **_grid(4001, 4001, 364, 134_000, 134_000))
     assert p is None or p["units"] < 1 << 32
+
+
+@pytest.mark.parametrize("dv,nv,span", [(3 * 10**8, 14, 6), (3 * 10**8, 14, 20), (5 * 10**8, 8, 20)])
+def test_group_steps_beyond_32_bits(plan, dv, nv, span):
+    """Steps of some 10^8 mpx/h are legal over a few milliseconds; a group's step of eight of them is not an int32."""
+    p = plan(5_000_000, 100, span, 60, tph=3_600_000,
+             **_grid(nv, nv, dv, 4096, 4096, vx0=-(nv // 2) * dv + 1000, vy0=-(nv // 2) * dv + 1000))
+    assert p is None or p["step_x"] == p["gx"] * dv
+
+
+def test_centre_velocity_times_time_beyond_64_bits(plan):
+    """Twice a centre velocity of 2^31 mpx/h over 2^32 ticks is 2^64; the same lattice over fewer ticks is planned."""
+    grid = _grid(75, 83, 3, 1024, 2048, 4000, vx0=2_100_000_000, vy0=2_100_000_000)
+    assert plan(2_000_000, 60, 1 << 30, 20, tph=1 << 38, **grid)
+    p = plan(2_000_000, 60, (1 << 32) - 1, 20, tph=1 << 40, **grid)
+    assert p is None

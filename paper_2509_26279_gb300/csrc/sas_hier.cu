@@ -627,7 +627,7 @@ bool plan_windows(const sas_grid_desc& d, uint64_t n, uint32_t n_min, double mea
         // windows that noise alone fills: about 2000 instructions of level 2 each
         const double windows = (n_v / (gx * gy) + 1) * (double)nbx * nby;
         const double lam = density * (double)(win * P) * (double)(win * P);
-        const double chance = windows * std::exp(std::min(0.0, log_poisson_tail(lam, n_eq)));
+        const double chance = windows * ((double)n_eq <= lam ? 1.0 : std::exp(std::min(0.0, log_poisson_tail(lam, n_eq))));
         const double level2 = chance * ((cb == 16 ? 3000.0 : 2000.0) / 2.2 / di.sms);
         if (level2 >= best || chance > 4e6) continue;
         WindowPlan w{};

@@ -173,7 +173,7 @@ int choose_tiles(const sas_grid_desc& d, uint32_t E, uint64_t n, int64_t dT, int
 void bucket_grid(const sas_grid_desc& d, uint32_t E, int64_t dT, int64_t tph, CoarseGeom* cg);
 // umulhi(X, magic_for(bin)) == X / bin for 0 <= X <= x_max
 bool magic_exact(int32_t bin, int64_t x_max);
-// log P(Poisson(lam) >= k)
+// log P(Poisson(lam) >= k), for k > lam: 200 terms from k on, which fall only there
 double log_poisson_tail(double lam, int k);
 // Fewer, taller bucket rows where that lets a unit take all its epochs at once.
 void one_epoch_chunk(const sas_grid_desc& d, uint64_t n, const sas_opts& o, const DevInfo& di, FieldPlan* fp);

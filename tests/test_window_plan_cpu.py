@@ -66,3 +66,10 @@ def test_centre_velocity_times_time_beyond_64_bits(plan):
     assert plan(2_000_000, 60, 1 << 30, 20, tph=1 << 38, **grid)
     p = plan(2_000_000, 60, (1 << 32) - 1, 20, tph=1 << 40, **grid)
     assert p is None
+
+
+@pytest.mark.parametrize("lam,n_min", [(400, 25), (540, 64), (812, 90), (812, 128)])
+def test_noise_that_fills_every_window(plan, lam, n_min):
+    """lam detections per window of 10.6 px on average, far above the threshold: every window would be kept."""
+    n = int(lam / 10.6**2 * 2048 * 4096)
+    assert plan(n, 255, 14_400, n_min, **_grid()) is None

@@ -117,7 +117,7 @@ struct Arena {
 
 // What the kernels of a search report, in one block so that one copy reads it.
 struct Counters {
-  uint32_t flags, n_emit, n_valid, pad;
+  uint32_t flags, n_emit, n_valid, n_long;  // n_long: windows that the long pass counts
   unsigned long long pairs, tile, raw, balance, pairs1, n_ids;  // pairs1: of the window search's first level
   long long t0;
 };
@@ -488,10 +488,12 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
       CK(launch_window_pairs(wa, dx, dy, dep, n, s), "pair count");
       CK(launch_stack_windows(sa, (int)std::min<uint64_t>((uint64_t)di.sms, std::max<uint64_t>(sa.n_tiles, 1)), s),
          "window kernel");
+      wa.n_long = &d_cnt->n_long;
       for (;;) {
         wa.keys = d_keys;
         wa.key_cap = key_cap;
         CK(launch_window_cells(wa, di.sms, s), "window cells");
+        if (wa.n_queue) CK(launch_window_long(wa, di.sms, s), "long windows");
         cudaEventRecord(evs1, s);
         CK(read_counters(), "stack sync");
         tr.mark("windows done");
@@ -501,11 +503,26 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
           rc = SAS_ERR_INTERNAL;
           goto done;
         }
+        if (h.n_long != wa.n_queue) {  // long windows, known now
+          wa.n_queue = h.n_long;
+          CK(sc.alloc(&wa.queue, wa.n_queue), "alloc long windows");
+          CK(cudaMemsetAsync(wa.n_long, 0, 4, s), "memset");
+          CK(launch_window_queue(wa, di.sms, s), "long window queue");
+          CK(launch_window_long(wa, di.sms, s), "long windows");
+          cudaEventRecord(evs1, s);
+          CK(read_counters(), "long windows sync");
+          if (h.flags & kFlagWindow) {
+            without = true;
+            rc = SAS_ERR_INTERNAL;
+            goto done;
+          }
+        }
         if (h.n_valid <= key_cap) break;
         key_cap = h.n_valid;
         if (key_cap >= (1u << 30)) { rc = fail(SAS_ERR_OOM, "too many candidate bins; raise n_min"); goto done; }
         CK(sc.alloc(&d_keys, key_cap), "alloc keys");
         CK(cudaMemsetAsync(&d_cnt->n_valid, 0, 4, s), "memset");
+        CK(cudaMemsetAsync(wa.n_long, 0, 4, s), "memset");
         CK(cudaMemsetAsync(&d_cnt->raw, 0, 8, s), "memset");
       }
       cudaEventRecord(evc0, s);

@@ -31,9 +31,9 @@
 // kernel and its exact counts took 1360 + 270 us; with a million velocities 8.9 ms
 // and 0.32 ms instead of 71.4 ms.  Level 1 is bound by shared memory and barriers
 // (58 % of the shared pipe, 48 % of the issue slots).  Everything stays exact whatever
-// the choice; a counter that wraps, a window list that overflows or a list
-// longer than a warp holds sets kFlagWindow and the host runs the one-level
-// search instead.
+// the choice.  A window of more detections than a warp lists at first is counted by a
+// second pass with longer lists; a counter that wraps, a window list that overflows or a
+// window of more than those hold makes the host run the one-level search instead.
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -46,7 +46,7 @@ namespace sas {
 namespace {
 
 constexpr int kWarps = 8;         // warps of a level-2 block
-constexpr uint32_t kList = 256;   // detections a warp's list holds
+constexpr uint32_t kList = 256, kLongList = 2048;  // detections a warp's list holds: at first, and of a long window
 constexpr int kMaxOwn = 2;        // bins per axis that a window owns at one velocity (P <= 2 bins)
 constexpr int kMaxWindowEpochs = 255;
 
@@ -195,11 +195,11 @@ __global__ void __launch_bounds__(256) k_window_pairs(WindowArgs a, const int32_
 // ---- level 2 ------------------------------------------------------------------
 
 // A warp's window: its detections relative to the window's corner.
-template <bool W>
+template <bool W, uint32_t N>
 struct WarpList {
-  int32_t x[kList], y[kList];
-  uint8_t e[kList];
-  uint8_t w[W ? kList : 4];       // weights
+  int32_t x[N], y[N];
+  uint8_t e[N];
+  uint8_t w[W ? N : 4];           // weights
   uint32_t seen[W ? 256 : 8];     // of the bin being counted: its epochs' bits, or their largest weights
   // per lattice column (8) and row (8) of the group: first owned bin, offset of its
   // edge, and the lengths of the first and second owned bin (0: not owned)
@@ -247,16 +247,23 @@ constexpr int32_t kOutside = INT32_MIN / 2;  // in no bin, whatever a group's ed
 // 235 us there, 528 -> 400 us with weights, 380 -> 320 us for a million velocities.
 // (Two records a turn cost more instructions than it hid: 277 us, and 107 -> 128 us
 // where runs are short.)
-template <bool W>
-__global__ void __launch_bounds__(kWarps * 32, 4) k_window_cells(WindowArgs a, uint64_t cell_m) {
+//
+// LONG: the windows in the queue, with room for kLongList detections each.  A window
+// of more than kList (two steady sources in it over 130 epochs, say) is marked by the
+// first pass and counted here, by one block an SM; fields without such windows do
+// not launch it.
+template <bool W, bool LONG>
+__global__ void __launch_bounds__(kWarps * 32, LONG ? 1 : 4) k_window_cells(WindowArgs a, uint64_t cell_m) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31;
-  WarpList<W>& L = reinterpret_cast<WarpList<W>*>(smem)[threadIdx.x >> 5];
+  constexpr uint32_t kCap = LONG ? kLongList : kList;
+  using List = WarpList<W, kCap>;
+  List& L = reinterpret_cast<List*>(smem)[threadIdx.x >> 5];
   const uint32_t lt = (1u << lane) - 1u;
   const SearchGeom& g = a.g;
   const uint32_t E = g.E;
   const int P = a.cgm.bin, span = a.win * P, nvg = a.gx * a.gy;
-  const uint32_t n_win = min(*a.n_windows, a.list_cap);
+  const uint32_t n_win = LONG ? a.n_queue : min(*a.n_windows, a.list_cap);
   unsigned long long raw_sum = 0;
   constexpr int kSeen = W ? 256 : 8;
   for (int i = lane; i < kSeen; i += 32) L.seen[i] = 0;
@@ -273,7 +280,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_window_cells(WindowArgs a, u
     const uint64_t w = ((uint64_t)(i_win / kWarps) * gridDim.x + blockIdx.x) * kWarps + i_win % kWarps;
     if (w >= n_win) break;
     if (lane == 0) ahead = atomicAdd(&drawn, 1u);
-    const Emit em = a.windows[w];
+    const Emit em = a.windows[LONG ? a.queue[w] : (uint32_t)w];
     const int Kx = (int)(em.v_idx % (uint32_t)a.cgm.nvx), Ky = (int)(em.v_idx / (uint32_t)a.cgm.nvx);
     const int32_t ux0 = a.cgm.x_min + (int32_t)em.bx * P, uy0 = a.cgm.y_min + (int32_t)em.by * P;
     __syncwarp();
@@ -321,7 +328,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_window_cells(WindowArgs a, u
         const bool hit = q < total && (uint32_t)X < (uint32_t)span && (uint32_t)Y < (uint32_t)span;
         const uint32_t m = __ballot_sync(0xffffffffu, hit);
         const uint32_t p = n + (uint32_t)__popc(m & lt);
-        if (hit && p < kList) {
+        if (hit && p < kCap) {
           L.x[p] = X;
           L.y[p] = Y;
           L.e[p] = (uint8_t)e;
@@ -331,8 +338,15 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_window_cells(WindowArgs a, u
       }
     }
     if (!W && n < a.n_min) continue;  // warp-uniform (the window's counters also hold the halo's rounding)
-    if (n > kList) {
-      if (lane == 0) atomicOr(a.flags, kFlagWindow);
+    if (n > kCap) {
+      if (lane == 0) {
+        if constexpr (LONG) {
+          atomicOr(a.flags, kFlagWindow);
+        } else {
+          a.windows[w].flags = kEmitLong;
+          atomicAdd(a.n_long, 1u);
+        }
+      }
       continue;
     }
     __syncwarp();
@@ -458,6 +472,16 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_window_cells(WindowArgs a, u
   if (lane == 0 && raw_sum) atomicAdd(a.raw_total, raw_sum);
 }
 
+// Places of the marked windows.
+__global__ void __launch_bounds__(1024) k_window_queue(WindowArgs a) {
+  const uint32_t n_win = min(*a.n_windows, a.list_cap);
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_win; i += gridDim.x * blockDim.x) {
+    if (a.windows[i].flags != kEmitLong) continue;
+    const uint32_t p = atomicAdd(a.n_long, 1u);
+    if (p < a.n_queue) a.queue[p] = i;
+  }
+}
+
 }  // namespace
 
 cudaError_t launch_window_tables(const WindowArgs& a, cudaStream_t s) {
@@ -479,19 +503,30 @@ cudaError_t launch_window_pairs(const WindowArgs& a, const int32_t* x, const int
   return cudaGetLastError();
 }
 
-template <bool W>
-static cudaError_t launch_cells(const WindowArgs& a, int sms, cudaStream_t s) {
-  constexpr size_t smem = kWarps * sizeof(WarpList<W>);
-  static_assert(smem <= 56 * 1024, "four blocks an SM");
-  cudaError_t e = cudaFuncSetAttribute(k_window_cells<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <bool W, bool LONG>
+static cudaError_t launch_cells(const WindowArgs& a, int blocks, cudaStream_t s) {
+  constexpr size_t smem = kWarps * sizeof(WarpList<W, LONG ? kLongList : kList>);
+  static_assert(smem <= (LONG ? 225 : 56) * 1024, "one block an SM, or four");
+  cudaError_t e = cudaFuncSetAttribute(k_window_cells<W, LONG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_window_cells<W><<<sms * 4, kWarps * 32, smem, s>>>(a, div_magic((uint32_t)a.cg.cell));
+  k_window_cells<W, LONG><<<blocks, kWarps * 32, smem, s>>>(a, div_magic((uint32_t)a.cg.cell));
   note_launch();
   return cudaGetLastError();
 }
 
 cudaError_t launch_window_cells(const WindowArgs& a, int sms, cudaStream_t s) {
-  return a.wts ? launch_cells<true>(a, sms, s) : launch_cells<false>(a, sms, s);
+  return a.wts ? launch_cells<true, false>(a, 4 * sms, s) : launch_cells<false, false>(a, 4 * sms, s);
+}
+
+cudaError_t launch_window_queue(const WindowArgs& a, int sms, cudaStream_t s) {
+  k_window_queue<<<2 * sms, 1024, 0, s>>>(a);
+  note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_window_long(const WindowArgs& a, int sms, cudaStream_t s) {
+  const int blocks = (int)std::min<uint32_t>((a.n_queue + kWarps - 1) / kWarps, (uint32_t)sms);
+  return a.wts ? launch_cells<true, true>(a, blocks, s) : launch_cells<false, true>(a, blocks, s);
 }
 
 // ---- planning -----------------------------------------------------------------

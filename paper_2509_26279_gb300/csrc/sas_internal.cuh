@@ -68,6 +68,7 @@ enum : uint32_t { kSelectAll = 0u, kSelectPlainAndPeaks = 1u, kSelectPeaks = 2u 
 enum : uint32_t {
   kEmitPlain = 1u,    // the super-bin's count reached n_min: its bins are counted against n_min
   kEmitLowPeak = 2u,  // count >= n_low and no neighbour of the tile larger: counted against n_low
+  kEmitLong = 4u,     // window search: a window of more detections than a warp lists at first
 };
 
 // Candidate sort key, compared lexicographically (a, b, c):
@@ -277,9 +278,12 @@ struct WindowArgs {
   uint8_t* vact;         // coarse lattice points with a searched fine one, or null
   uint32_t* vsum;        // [(nvy + 1)][(nvx + 1)] searched points below and left, or null: all are searched
   const uint8_t* wts;    // weight per detection id (weighted stacking), or null
-  const Emit* windows;
+  Emit* windows;
   const uint32_t* n_windows;
   uint32_t list_cap;
+  uint32_t* n_long;      // windows marked kEmitLong
+  uint32_t* queue;       // [n_queue] their places in the list, once they are known
+  uint32_t n_queue;
   uint32_t n_min;
   Key* keys;
   uint32_t key_cap;
@@ -291,7 +295,12 @@ struct WindowArgs {
 cudaError_t launch_window_tables(const WindowArgs& a, cudaStream_t s);
 cudaError_t launch_window_pairs(const WindowArgs& a, const int32_t* x, const int32_t* y, const uint16_t* epoch,
                                 uint64_t n, cudaStream_t s);
+// Counts all windows but the long ones, which it marks (n_long).
 cudaError_t launch_window_cells(const WindowArgs& a, int sms, cudaStream_t s);
+// Lists the marked windows in queue (n_long, zero before, counts them again).
+cudaError_t launch_window_queue(const WindowArgs& a, int sms, cudaStream_t s);
+// Counts the windows in queue.
+cudaError_t launch_window_long(const WindowArgs& a, int sms, cudaStream_t s);
 
 // sas_post.cu
 // Appends one key per bin of an emitted super-bin that lies in the domain and

@@ -153,3 +153,44 @@ def test_oracle():
     ref = oracle.stack(cat, grid, 13, threads=0)
     assert len(ref.cands) > 0
     assert_same(res, ref)
+
+
+def _spot(cat, count, epochs):
+    """cat without detections near (400, 700) px and with `count` there: 3 x 3 positions (5 x 5 for more) 3.6 px apart, each
+    in every epoch until `count` is reached.  Cells of at most 3.6 px see no more than one of them an epoch."""
+    keep = (np.abs(cat.x - 400_000) > 60_000) | (np.abs(cat.y - 700_000) > 60_000)
+    k = np.arange(count)
+    p, e, side = k // epochs, (k % epochs).astype(np.uint16), 3 if count <= 9 * epochs else 5
+    x, y = (400_000 + 3600 * (p % side)).astype(np.int32), (700_000 + 3600 * (p // side)).astype(np.int32)
+    return cases.catalog(np.r_[cat.x[keep], x], np.r_[cat.y[keep], y], np.r_[cat.epoch[keep], e], cat.t, cat.ticks_per_hour)
+
+
+@pytest.mark.parametrize("epochs,count,two_levels", [(130, 256, True), (130, 257, True), (130, 1170, True), (250, 2000, True),
+                                                     (250, 6250, False)])
+def test_detections_in_one_window(epochs, count, two_levels):
+    """Up to 256 detections of a window are listed by the first pass, up to 2048 by the second, and more send the field to
+    the one-level search."""
+    cat = _spot(_field(11, epochs=epochs, noise=40_000 // epochs, movers=20), count, epochs)
+    two, one = _check(cat, _grid(), epochs // 3)
+    assert two[2] > 0
+    assert (two[3]["n_emitted"] != one[3]["n_emitted"]) == two_levels
+
+
+def test_long_windows_with_weights():
+    cat, grid = _spot(_field(12, epochs=130, noise=300, movers=20), 1170, 130), _grid()
+    w = (20 + np.random.default_rng(4).integers(0, 60, len(cat.x))).astype(np.uint8)
+    got = []
+    for tiles in (dict(), dict(tile_kx=8, tile_ky=4)):
+        res = sas.sas_stack_weighted(sas.Grid(grid), cat.x, cat.y, cat.epoch, w, cat.t, cat.ticks_per_hour, 2000,
+                                     opts=sas.make_opts(**tiles))
+        c, ids = res.candidates()
+        got.append((c.tobytes(), ids.tobytes(), res.info()["n_pairs"], res.info()["n_emitted"]))
+    assert got[0][:3] == got[1][:3] and len(got[0][0]) > 0
+    assert got[0][3] != got[1][3]
+
+
+def test_bright_movers_over_many_epochs():
+    """Movers seen in nearly all of 255 epochs: with the noise around them their windows hold more than 256 detections."""
+    r = W.FieldRecipe(1021, 1777, 255, 4.0, 500, 25, (0.5, 15.0), (1.0, 0.97))
+    two, one = _check(W.make_catalog(r, 13), _grid(), 90)
+    assert two[2] > 0 and two[3]["n_emitted"] != one[3]["n_emitted"]

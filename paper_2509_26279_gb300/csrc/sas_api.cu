@@ -19,9 +19,10 @@ using namespace sas;
 
 struct sas_grid {
   sas_grid_desc d;
-  // emission count of the previous search on this grid: sizes the next
-  // emission list so that repeated searches do not need an exact rerun
-  std::atomic<uint32_t> emit_hint{0};
+  // emissions of the previous search on this grid -- super-bins of a one-level search,
+  // windows of a two-level one: they size the next emission list of the same
+  // kind so that repeated searches do not need an exact rerun
+  std::atomic<uint32_t> emit_hint{0}, window_hint{0};
 };
 
 struct sas_result {
@@ -115,6 +116,9 @@ struct Arena {
   }
 };
 
+// Windows that a two-level search lists (1 GB); more leave the field to the one-level search.
+constexpr uint32_t kMaxWindows = 1u << 26;
+
 // What the kernels of a search report, in one block so that one copy reads it.
 struct Counters {
   uint32_t flags, n_emit, n_valid, n_long;  // n_long: windows that the long pass counts
@@ -184,6 +188,7 @@ int sas_create_grid(const sas_grid_desc* desc, sas_grid** out) {
   if (!g) return fail(SAS_ERR_OOM, "host allocation");
   g->d = d;
   g->emit_hint.store(0);
+  g->window_hint.store(0);
   *out = g;
   return SAS_OK;
 }
@@ -334,10 +339,11 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
     const uint16_t* dep = cat->epoch;
     const uint8_t* d_w = weights;
     const bool host = !cat->on_device;
-    const uint32_t hint = grid->emit_hint.load(std::memory_order_relaxed);
+    std::atomic<uint32_t>& last_emit = const_cast<sas_grid*>(grid)->*(use_win ? &sas_grid::window_hint : &sas_grid::emit_hint);
+    const uint32_t hint = last_emit.load(std::memory_order_relaxed);
     uint32_t emit_cap = (uint32_t)std::min<uint64_t>(
-        std::max<uint64_t>({(uint64_t)1 << 16, 2 * n, (uint64_t)hint + hint / 4 + 1024}), (uint64_t)1 << 26);
-    if (use_win) emit_cap = std::max(wplan.list_cap, hint + hint / 4);
+        std::max<uint64_t>({use_win ? (uint64_t)wplan.list_cap : std::max<uint64_t>((uint64_t)1 << 16, 2 * n),
+                            (uint64_t)hint + hint / 4 + 1024}), (uint64_t)1 << 26);
     uint32_t key_cap = use_win ? 1u << 17 : 0;
     const size_t npts = use_win && wplan.masked ? ((size_t)d.nvx + 1) * ((size_t)d.nvy + 1) : 0;
     const size_t nK = use_win ? (size_t)wplan.g.nvx * wplan.g.nvy : 0;
@@ -467,9 +473,7 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
       wa.sxt = d_sxt;
       wa.syt = d_syt;
       wa.wts = d_w;
-      wa.windows = d_emits;
       wa.n_windows = &d_cnt->n_emit;
-      wa.list_cap = emit_cap;
       wa.n_min = n_min;
       wa.n_valid = &d_cnt->n_valid;
       wa.raw_total = &d_cnt->raw;
@@ -480,16 +484,19 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
       sa.vact = wa.vact;
       sa.sxt = wa.sXt;
       sa.syt = wa.sYt;
-      sa.emits = d_emits;
-      sa.emit_cap = emit_cap;
       sa.n_pairs = &d_cnt->pairs1;
       cudaEventRecord(evs0, s);
       CK(launch_window_tables(wa, s), "group tables");
       CK(launch_window_pairs(wa, dx, dy, dep, n, s), "pair count");
-      CK(launch_stack_windows(sa, (int)std::min<uint64_t>((uint64_t)di.sms, std::max<uint64_t>(sa.n_tiles, 1)), s),
-         "window kernel");
       wa.n_long = &d_cnt->n_long;
-      for (;;) {
+      for (bool level1 = true;;) {
+        if (level1) {
+          wa.windows = sa.emits = d_emits;
+          wa.list_cap = sa.emit_cap = emit_cap;
+          CK(launch_stack_windows(sa, (int)std::min<uint64_t>((uint64_t)di.sms, std::max<uint64_t>(sa.n_tiles, 1)), s),
+             "window kernel");
+          level1 = false;
+        }
         wa.keys = d_keys;
         wa.key_cap = key_cap;
         CK(launch_window_cells(wa, di.sms, s), "window cells");
@@ -498,10 +505,19 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
         CK(read_counters(), "stack sync");
         tr.mark("windows done");
         if ((rc = input_error())) goto done;
-        if ((h.flags & (kFlagWindow | kFlagEmitCap)) || h.balance != 0 || h.n_emit > emit_cap) {
+        const bool full = (h.flags & kFlagEmitCap) || h.n_emit > emit_cap;
+        if ((h.flags & kFlagWindow) || h.balance != 0 || (full && (h.n_emit <= emit_cap || h.n_emit > kMaxWindows))) {
           without = true;
           rc = SAS_ERR_INTERNAL;
           goto done;
+        }
+        if (full) {  // level 1 again with room for what it found
+          emit_cap = h.n_emit;
+          CK(sc.alloc(&d_emits, emit_cap), "alloc windows");
+          CK(cudaMemsetAsync(d_cnt, 0, offsetof(Counters, pairs), s), "memset");
+          CK(cudaMemsetAsync(&d_cnt->tile, 0, offsetof(Counters, n_ids) - offsetof(Counters, tile), s), "memset");
+          level1 = true;
+          continue;
         }
         if (h.n_long != wa.n_queue) {  // long windows, known now
           wa.n_queue = h.n_long;
@@ -577,7 +593,7 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
       break;
     }
     {
-      const_cast<sas_grid*>(grid)->emit_hint.store(h.n_emit, std::memory_order_relaxed);
+      last_emit.store(h.n_emit, std::memory_order_relaxed);
       // a8: total order of the valid keys; a7: candidates, contributing ids
       const uint32_t n_emit = h.n_emit, n_valid = h.n_valid;
       n_out = n_valid;

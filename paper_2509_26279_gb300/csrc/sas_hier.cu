@@ -32,8 +32,9 @@
 // and 0.32 ms instead of 71.4 ms.  Level 1 is bound by shared memory and barriers
 // (58 % of the shared pipe, 48 % of the issue slots).  Everything stays exact whatever
 // the choice.  A window of more detections than a warp lists at first is counted by a
-// second pass with longer lists; a counter that wraps, a window list that overflows or a
-// window of more than those hold makes the host run the one-level search instead.
+// second pass with longer lists, and a window list that overflows is made longer; a counter
+// that wraps or a window of more than those lists hold makes the host run the one-level
+// search instead.
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -263,7 +264,8 @@ __global__ void __launch_bounds__(kWarps * 32, LONG ? 1 : 4) k_window_cells(Wind
   const SearchGeom& g = a.g;
   const uint32_t E = g.E;
   const int P = a.cgm.bin, span = a.win * P, nvg = a.gx * a.gy;
-  const uint32_t n_win = LONG ? a.n_queue : min(*a.n_windows, a.list_cap);
+  const uint32_t n_win = LONG ? a.n_queue : *a.n_windows;
+  if (!LONG && n_win > a.list_cap) return;  // level 1 runs again with a longer list
   unsigned long long raw_sum = 0;
   constexpr int kSeen = W ? 256 : 8;
   for (int i = lane; i < kSeen; i += 32) L.seen[i] = 0;
@@ -474,7 +476,7 @@ __global__ void __launch_bounds__(kWarps * 32, LONG ? 1 : 4) k_window_cells(Wind
 
 // Places of the marked windows.
 __global__ void __launch_bounds__(1024) k_window_queue(WindowArgs a) {
-  const uint32_t n_win = min(*a.n_windows, a.list_cap);
+  const uint32_t n_win = *a.n_windows;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_win; i += gridDim.x * blockDim.x) {
     if (a.windows[i].flags != kEmitLong) continue;
     const uint32_t p = atomicAdd(a.n_long, 1u);

@@ -194,3 +194,41 @@ def test_bright_movers_over_many_epochs():
     r = W.FieldRecipe(1021, 1777, 255, 4.0, 500, 25, (0.5, 15.0), (1.0, 0.97))
     two, one = _check(W.make_catalog(r, 13), _grid(), 90)
     assert two[2] > 0 and two[3]["n_emitted"] != one[3]["n_emitted"]
+
+
+def _pool(attribute):
+    """An attribute of the device's stream-ordered pool."""
+    import ctypes
+    cu, pool, v = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(), ctypes.c_uint64(0)
+    assert cu.cuDeviceGetDefaultMemPool(ctypes.byref(pool), torch.cuda.current_device()) == 0
+    if attribute == "reset":
+        assert cu.cuMemPoolSetAttribute(pool, 8, ctypes.byref(v)) == 0   # CU_MEMPOOL_ATTR_USED_MEM_HIGH
+    else:
+        assert cu.cuMemPoolGetAttribute(pool, {"used": 7, "high": 8}[attribute], ctypes.byref(v)) == 0
+    return v.value
+
+
+def test_a_low_threshold_search_does_not_size_the_window_list():
+    """Super-bins emitted by a one-level search on a grid say nothing about the windows of the next search on it."""
+    cat, grid = _field(10), sas.Grid(_grid())
+
+    def peak():
+        torch.cuda.synchronize()
+        _pool("reset")
+        before = _pool("used")
+        sas.stack_catalog(grid, cat, 14).free()
+        return _pool("high") - before
+    alone = [peak(), peak()]
+    low = sas.stack_catalog(grid, cat, 4, opts=sas.make_opts(superbin=3))  # one level
+    assert low.info()["n_emitted"] > 1 << 20
+    low.free()
+    assert peak() <= max(alone) + (1 << 20)
+
+
+def test_more_windows_and_candidates_than_their_lists_hold_at_first():
+    """Many movers: more windows than noise would leave and more candidates than the key list's first 131072; both lists
+    grow to what was counted."""
+    cat = _field(14, movers=2500)
+    two, one = _check(cat, _grid(), 14)
+    assert two[2] > 1 << 17
+    assert two[3]["n_emitted"] > (1 << 18) + cat.n and two[3]["n_emitted"] != one[3]["n_emitted"]

@@ -206,10 +206,10 @@ namespace {
 // The search (Sec. 2.1 steps 1-3); with weights (one uint8 per detection, in
 // host or device memory like the catalog) cells are scored by the sum over
 // epochs of their largest weight and n_min is the score threshold.
-// windows: the window search (sas_hier.cu) may be used; it is run again without
-// when a field turns out not to fit it.
+// window_bits: the least counter width of a window search (sas_hier.cu), 0 for none; a
+// field that turns out not to fit it is searched again with wider counters or without.
 int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weights, uint32_t n_min,
-               const sas_opts* opts, void* stream, sas_result** out, bool windows = true) {
+               const sas_opts* opts, void* stream, sas_result** out, int window_bits = 8) {
   if (!grid || !cat || !out) return fail(SAS_ERR_ARG, "null argument");
   const Tracer tr;
   const sas_grid_desc& d = grid->d;
@@ -305,10 +305,10 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
   }
   // A caller that sets tile sizes gets the one-level kernel with those tiles.
   WindowPlan wplan;
-  const bool use_win = windows && n_low == n_min && !o.peaks_only && !o.tile_kx && !o.tile_ky && !o.tile_bx &&
+  const bool use_win = window_bits && n_low == n_min && !o.peaks_only && !o.tile_kx && !o.tile_ky && !o.tile_bx &&
                        !o.tile_by && !o.counter_bits && !o.coarse_bins && !o.superbin && !o.velocity_block &&
-                       plan_windows(d, n, n_min, mean_weight, v_begin, v_end, di, plan, &wplan);
-  bool without = false;  // the window search gave up: run again without it
+                       plan_windows(d, n, n_min, mean_weight, v_begin, v_end, di, plan, &wplan, window_bits);
+  int again = -1;  // the window search gave up: run again with these window_bits
   const CoarseGeom& cg = use_win ? wplan.cg : plan.cg;
   const uint64_t nb = use_win ? wplan.nb : plan.nb;
   const SearchGeom& g = plan.g;
@@ -474,6 +474,7 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
       wa.syt = d_syt;
       wa.wts = d_w;
       wa.n_windows = &d_cnt->n_emit;
+      wa.balance = &d_cnt->balance;
       wa.n_min = n_min;
       wa.n_valid = &d_cnt->n_valid;
       wa.raw_total = &d_cnt->raw;
@@ -505,9 +506,9 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
         CK(read_counters(), "stack sync");
         tr.mark("windows done");
         if ((rc = input_error())) goto done;
-        const bool full = (h.flags & kFlagEmitCap) || h.n_emit > emit_cap;
-        if ((h.flags & kFlagWindow) || h.balance != 0 || (full && (h.n_emit <= emit_cap || h.n_emit > kMaxWindows))) {
-          without = true;
+        const bool full = (h.flags & kFlagEmitCap) || h.n_emit > emit_cap, wrapped = h.balance != 0;
+        if (wrapped || (h.flags & kFlagWindow) || (full && (h.n_emit <= emit_cap || h.n_emit > kMaxWindows))) {
+          again = wrapped && wplan.tc.cb == 8 ? 16 : 0;
           rc = SAS_ERR_INTERNAL;
           goto done;
         }
@@ -528,7 +529,7 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
           cudaEventRecord(evs1, s);
           CK(read_counters(), "long windows sync");
           if (h.flags & kFlagWindow) {
-            without = true;
+            again = 0;
             rc = SAS_ERR_INTERNAL;
             goto done;
           }
@@ -655,7 +656,7 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
       if (p) cudaFreeAsync(p, s);
     cudaStreamSynchronize(s);
     delete res;
-    return without ? stack_impl(grid, cat, weights, n_min, opts, stream, out, false) : rc;
+    return again >= 0 ? stack_impl(grid, cat, weights, n_min, opts, stream, out, again) : rc;
   }
   *out = res;
   return SAS_OK;

@@ -32,9 +32,9 @@
 // and 0.32 ms instead of 71.4 ms.  Level 1 is bound by shared memory and barriers
 // (58 % of the shared pipe, 48 % of the issue slots).  Everything stays exact whatever
 // the choice.  A window of more detections than a warp lists at first is counted by a
-// second pass with longer lists, and a window list that overflows is made longer; a counter
-// that wraps or a window of more than those lists hold makes the host run the one-level
-// search instead.
+// second pass with longer lists, a window list that overflows is made longer, and 8-bit
+// counters that wrap are replaced by 16-bit ones; a 16-bit counter that wraps or a window of
+// more than the longer lists hold makes the host run the one-level search instead.
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(kWarps * 32, LONG ? 1 : 4) k_window_cells(Wind
   const uint32_t E = g.E;
   const int P = a.cgm.bin, span = a.win * P, nvg = a.gx * a.gy;
   const uint32_t n_win = LONG ? a.n_queue : *a.n_windows;
-  if (!LONG && n_win > a.list_cap) return;  // level 1 runs again with a longer list
+  if (!LONG && (n_win > a.list_cap || *a.balance != 0)) return;  // level 1 runs again: longer list, wider counters
   unsigned long long raw_sum = 0;
   constexpr int kSeen = W ? 256 : 8;
   for (int i = lane; i < kSeen; i += 32) L.seen[i] = 0;
@@ -620,7 +620,7 @@ bool centre_fits(int32_t v0, int32_t dv, uint32_t nv, int grp, int64_t dT) {
 }  // namespace
 
 bool plan_windows(const sas_grid_desc& d, uint64_t n, uint32_t n_min, double mean_weight, uint64_t v_begin,
-                  uint64_t v_end, const DevInfo& di, const FieldPlan& fp, WindowPlan* wp) {
+                  uint64_t v_end, const DevInfo& di, const FieldPlan& fp, WindowPlan* wp, int min_bits) {
   const uint32_t E = fp.g.E;
   const uint64_t nv = (uint64_t)d.nvx * d.nvy;
   if (E > (uint32_t)kMaxWindowEpochs || n_min < 2 || n_min > (mean_weight > 0 ? 32768u : 128u)) return false;
@@ -639,7 +639,7 @@ bool plan_windows(const sas_grid_desc& d, uint64_t n, uint32_t n_min, double mea
   const int64_t unit = d.bin;
   const double density = (double)n / ((double)d.nbx * d.nby * (double)d.bin * d.bin);
   // weighted: 16-bit counters of weights; noise windows by the number of mean weights that reach n_min
-  const int cb = mean_weight > 0 ? 16 : 8;
+  const int cb = mean_weight > 0 ? 16 : min_bits;
   const int n_eq = mean_weight > 0 ? std::max(2, (int)((double)n_min / mean_weight)) : (int)n_min;
   const bool square = std::llabs((int64_t)d.dvx) == std::llabs((int64_t)d.dvy);
   double best = one_level - 40000;
@@ -665,7 +665,7 @@ bool plan_windows(const sas_grid_desc& d, uint64_t n, uint32_t n_min, double mea
         const double windows = (n_v / (gx * gy) + 1) * (double)nbx * nby;
         const double lam = density * (double)(win * P) * (double)(win * P);
         const double chance = windows * ((double)n_eq <= lam ? 1.0 : std::exp(std::min(0.0, log_poisson_tail(lam, n_eq))));
-        const double level2 = chance * ((cb == 16 ? 3000.0 : 2000.0) / 2.2 / di.sms);
+        const double level2 = chance * ((mean_weight > 0 ? 3000.0 : 2000.0) / 2.2 / di.sms);
         if (level2 >= best || chance > 4e6) continue;
         WindowPlan w{};
         w.gx = gx;

@@ -255,8 +255,9 @@ struct WindowPlan {
 // Whether the window search is expected to take fewer instructions than the
 // stack kernel over the fine lattice as planned in fp; fills wp if so.
 // mean_weight: of the detections in weighted stacking (n_min is the score threshold), else 0.
+// min_bits: 16 after an 8-bit counter wrapped.
 bool plan_windows(const sas_grid_desc& d, uint64_t n, uint32_t n_min, double mean_weight, uint64_t v_begin,
-                  uint64_t v_end, const DevInfo& di, const FieldPlan& fp, WindowPlan* wp);
+                  uint64_t v_end, const DevInfo& di, const FieldPlan& fp, WindowPlan* wp, int min_bits = 8);
 // Level 1's arguments (lattice rows ky_lo..ky_hi of the fine lattice).
 void fill_window_args(const WindowPlan& wp, uint32_t n_min, uint32_t ky_lo, uint32_t ky_hi, StackArgs* sa);
 // Device arrays of a window search, besides those of every search.
@@ -280,6 +281,7 @@ struct WindowArgs {
   const uint8_t* wts;    // weight per detection id (weighted stacking), or null
   Emit* windows;
   const uint32_t* n_windows;
+  const unsigned long long* balance;  // of level 1: nonzero when a counter wrapped
   uint32_t list_cap;
   uint32_t* n_long;      // windows marked kEmitLong
   uint32_t* queue;       // [n_queue] their places in the list, once they are known

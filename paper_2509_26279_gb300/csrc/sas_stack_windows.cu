@@ -1,6 +1,6 @@
 // The stack kernel's instantiations of the window search (sas_hier.cu): tiles of
 // 4 x 4 groups of lattice points, 8-bit counters for detections and 16-bit ones
-// for weights.  Four columns of groups share the row's address, and 16 points a
+// for weights and for detections whose 8-bit counters wrapped.  Four columns of groups share the row's address, and 16 points a
 // tile leave room for tiles of some 100 x 100 cells, whose overlap (2 cells) and
 // shift spread (about a third of a tile) stay small.
 #include "sas_stack_kernel.cuh"

@@ -232,3 +232,16 @@ def test_more_windows_and_candidates_than_their_lists_hold_at_first():
     two, one = _check(cat, _grid(), 14)
     assert two[2] > 1 << 17
     assert two[3]["n_emitted"] > (1 << 18) + cat.n and two[3]["n_emitted"] != one[3]["n_emitted"]
+
+
+@pytest.mark.parametrize("used,per_epoch,two_levels", [(130, 1, True), (130, 4, True), (1, 70_000, False)])
+def test_counters_that_wrap(used, per_epoch, two_levels):
+    """Detections of one position in the first `used` epochs: within and above what a cell's 8-bit counter holds, and above
+    what 16 bits and a window's list hold."""
+    cat = _field(15, epochs=130, noise=300, movers=20)
+    x, y = np.full(per_epoch * used, 400_100, np.int32), np.full(per_epoch * used, 700_100, np.int32)
+    e = np.tile(np.arange(used, dtype=np.uint16), per_epoch)
+    cat = cases.catalog(np.r_[cat.x, x], np.r_[cat.y, y], np.r_[cat.epoch, e], cat.t, cat.ticks_per_hour)
+    two, one = _check(cat, _grid(), 40)
+    assert two[2] > 0
+    assert (two[3]["n_emitted"] != one[3]["n_emitted"]) == two_levels

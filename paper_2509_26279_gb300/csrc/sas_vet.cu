@@ -27,6 +27,7 @@
 
 struct sas_vet {
   int device;
+  int sms;               // the device's SMs
   uint32_t max_batch;
   uint64_t step;
   float beta1, beta2, eps;
@@ -1180,9 +1181,9 @@ __global__ void k_adam(float* __restrict__ master, float* __restrict__ m, float*
 
 // ---- host side -----------------------------------------------------------------
 
+// Shared-memory limits of the kernels on the current device (they are the device's own,
+// so every vetter sets them on its device).
 cudaError_t set_attrs() {
-  static bool done = false;
-  if (done) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(k_conv_fwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_fc_fwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kFcTcSmem);
@@ -1198,26 +1199,14 @@ cudaError_t set_attrs() {
     e = cudaFuncSetAttribute(k_fc1_dw, cudaFuncAttributeMaxDynamicSharedMemorySize, kDwSmem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_conv1_dw_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kC1Smem);
-  if (e == cudaSuccess) done = true;
   return e;
-}
-
-int fwd_blocks() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    n = sms > 0 ? sms : 152;
-  }
-  return n;
 }
 
 // Forward of n <= max_batch stamps; with keep, stores the activations training needs.
 cudaError_t forward(sas_vet* vt, const uint16_t* stamps, const uint32_t* idx, uint32_t n, bool keep,
                     float* logits, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  const int blocks = (int)std::min<uint32_t>(n, (uint32_t)fwd_blocks());
+  const int blocks = (int)std::min<uint32_t>(n, (uint32_t)vt->sms);
   k_conv_fwd_tc<<<blocks, kTcThreads, kTcSmem, s>>>(stamps, idx, n, vt->wb, keep ? vt->a1 : nullptr,
                                                    keep ? vt->a2 : nullptr, vt->a3, vt->status);
   const uint32_t tiles = (n + kFcTcRows - 1) / kFcTcRows, ldp = tiles * kFcTcRows;
@@ -1320,10 +1309,14 @@ int sas_vet_create(int device, uint32_t max_batch, sas_vet** out) {
   if (max_batch == 0 || max_batch > SAS_VET_MAX_BATCH)
     return set_errorf(SAS_ERR_ARG, "sas_vet_create: max_batch must be 1..%u", (unsigned)SAS_VET_MAX_BATCH);
   DeviceGuard guard(device);
-  if (cudaError_t e = vet::set_attrs(); e != cudaSuccess) return cuda_fail(e, "sas_vet_create");
+  int sms = 0;
+  cudaError_t ae = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+  if (ae == cudaSuccess) ae = vet::set_attrs();
+  if (ae != cudaSuccess) return cuda_fail(ae, "sas_vet_create");
   sas_vet* vt = new sas_vet();
   std::memset(vt, 0, sizeof(*vt));
   vt->device = device;
+  vt->sms = sms;
   vt->max_batch = max_batch;
   vt->beta1 = 0.9f;
   vt->beta2 = 0.999f;

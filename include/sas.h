@@ -315,9 +315,10 @@ int sas_batch_vet(const sas_batch* batch, sas_vet* vetter, uint32_t* field_out, 
  * warm-up; *best gets the options with the lowest median device time of the
  * whole search (*best_ms).  Every combination gives the same candidates
  * (Sec. 2.1 steps 1-3 are independent of the tiling); only the speed differs.
- * Every combination searches in one level (sas_opts): it tunes fields of a batch
- * and searches with a lowered threshold, while a single search with one threshold
- * is usually fastest with no tile option set. */
+ * Every combination searches in one level (sas_opts); where the options as given
+ * search in two levels they are timed too, and returned with their tile options
+ * still 0 if they win.  To tune a field of a batch, whose searches run in one level,
+ * give base a counter_bits of its own. */
 int sas_autotune(const sas_grid* grid, const sas_catalog* cat, uint32_t n_min,
                  const sas_opts* base, uint32_t reps, void* stream, sas_opts* best,
                  float* best_ms);

@@ -46,6 +46,7 @@ struct sas_result {
   uint32_t n_min;     // the search's threshold (the score threshold when weighted)
   int complete;       // every cell >= n_min is in the list (no top-K cut)
   int weighted;       // counts are weighted scores
+  int two_levels;     // found by the window search
 };
 
 namespace {
@@ -144,6 +145,8 @@ struct Tracer {
 }  // namespace
 
 namespace sas {
+bool result_two_levels(const sas_result* r) { return r->two_levels != 0; }
+
 CandView result_view(const sas_result* r) {
   CandView v;
   v.cands = r->d_cands;
@@ -629,6 +632,7 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
       const unsigned long long n_ids = h.n_ids;
       res->info.n_candidates = n_out;
       res->complete = n_out == n_valid;
+      res->two_levels = use_win;
       res->info.n_ids = n_ids;
       res->info.n_pairs = h.pairs;
       res->info.n_emitted = n_emit;

@@ -781,6 +781,30 @@ int sas_autotune(const sas_grid* grid, const sas_catalog* cat, uint32_t n_min, c
   if (o0.superbin) sbs = {o0.superbin};
   if (o0.velocity_block) vbs = {o0.velocity_block};
   if (o0.tile_bx || o0.tile_by) bxs = {o0.tile_bx};
+  // Median device time of a search with options o: its status.
+  auto time_search = [&](const sas_opts& o, float* med, bool* two_levels) -> int {
+    std::vector<float> ts;
+    for (uint32_t r = 0; r <= reps; ++r) {
+      sas_result* res = nullptr;
+      if (int rc = sas_stack(grid, cat, n_min, &o, stream, &res)) return rc;
+      sas_result_info inf;
+      sas_result_get_info(res, &inf);
+      if (r > 0) ts.push_back(inf.ms_total);
+      *two_levels = result_two_levels(res);
+      sas_result_free(res);
+    }
+    std::sort(ts.begin(), ts.end());
+    *med = ts[ts.size() / 2];
+    return SAS_OK;
+  };
+  // The options as given, if the search then runs in two levels (with tiles set it
+  // does not).
+  float med = 0;
+  bool two_levels = false;
+  if (time_search(o0, &med, &two_levels) == SAS_OK && two_levels) {
+    best_t = med;
+    any = true;
+  }
   for (const auto& vt : vtiles)
   for (uint32_t sb : sbs)
   for (uint32_t bx : bxs)
@@ -791,20 +815,7 @@ int sas_autotune(const sas_grid* grid, const sas_catalog* cat, uint32_t n_min, c
       o.superbin = sb;
       o.tile_bx = bx;
       o.velocity_block = vb;
-      std::vector<float> ts;
-      int rc = SAS_OK;
-      for (uint32_t r = 0; r <= reps && rc == SAS_OK; ++r) {
-        sas_result* res = nullptr;
-        rc = sas_stack(grid, cat, n_min, &o, stream, &res);
-        if (rc != SAS_OK) break;
-        sas_result_info inf;
-        sas_result_get_info(res, &inf);
-        if (r > 0) ts.push_back(inf.ms_total);
-        sas_result_free(res);
-      }
-      if (rc != SAS_OK) continue;  // a configuration the planner rejects for this field
-      std::sort(ts.begin(), ts.end());
-      const float med = ts[ts.size() / 2];
+      if (time_search(o, &med, &two_levels) != SAS_OK) continue;  // a configuration the planner rejects for this field
       if (med < best_t) {
         best_t = med;
         best_o = o;

@@ -403,6 +403,7 @@ int refine_tracks(const RefineIn& in, const sas_refine_opts& o, cudaStream_t s, 
 
 // sas_api.cu: the candidate view of a finished search.
 CandView result_view(const sas_result* r);
+bool result_two_levels(const sas_result* r);  // found by the window search
 
 // sas_probe.cu
 cudaError_t run_atomic_probe(uint32_t iters, cudaStream_t s, double* ops_per_s, double* sm_mhz);

@@ -10,7 +10,9 @@ each field takes its class's options.  The cache is a JSON object
 "tile_by": by, "velocity_block": b, "ms": t, "planner_ms": t0, "device": name}}
 (0: the planner's choice for that field; planner_ms: the planner's own options
 timed the same way on the same field)
-that can be written to disk and reused across runs on the same GPU model.
+that can be written to disk and reused across runs on the same GPU model.  The
+choices are for the one-level search that a batch runs; a single search with
+one threshold is usually fastest with no tile option set.
 
 Host logic only: the timing runs in the library (sas_autotune).
 """
@@ -76,6 +78,9 @@ class TuneCache:
         from . import sas
         key = tag + size_class(field.E, field.cat.n, field.w.grid, field.w.n_min)
         if key not in self.entries:
+            # the planner's own counter width for this threshold, set so that the search keeps to one level
+            base = sas.make_opts(**{k: getattr(base, k) for k, _ in sas.sas_opts._fields_} if base is not None else {})
+            base.counter_bits = base.counter_bits or (8 if field.w.n_min <= 128 else 16 if field.w.n_min <= 32768 else 32)
             best, ms = sas.sas_autotune(field.grid, field.dx, field.dy, field.de, field.cat.t,
                                         field.cat.ticks_per_hour, field.w.n_min, base=base, reps=reps)
             # the planner's own choice on the same field, timed the same way (device

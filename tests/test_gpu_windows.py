@@ -245,3 +245,32 @@ def test_counters_that_wrap(used, per_epoch, two_levels):
     two, one = _check(cat, _grid(), 40)
     assert two[2] > 0
     assert (two[3]["n_emitted"] != one[3]["n_emitted"]) == two_levels
+
+
+def test_autotune_returns_the_two_level_search_where_it_is_faster():
+    """sas_autotune's own combinations set tiles, which keep a search to one level."""
+    cat, grid = _field(16, noise=2000), sas.Grid(_grid())
+    d = [torch.from_numpy(a).cuda() for a in (cat.x, cat.y, cat.epoch.view(np.int16))]
+    best, ms = sas.sas_autotune(grid, *d, cat.t, cat.ticks_per_hour, 22, reps=2)
+    n = [sas.sas_stack(grid, *d, cat.t, cat.ticks_per_hour, 22, on_device=True, opts=o).info()["n_emitted"]
+         for o in (best, sas.make_opts(), sas.make_opts(tile_kx=8, tile_ky=8))]
+    assert n[0] == n[1] != n[2] and ms > 0
+    one, _ = sas.sas_autotune(grid, *d, cat.t, cat.ticks_per_hour, 22, base=sas.make_opts(counter_bits=8), reps=1)
+    assert one.superbin in (1, 2, 3, 4)
+
+
+def test_tuning_cache_keeps_tiles_for_batches():
+    """The cache's choices go to batches, which search in one level: they name tiles."""
+    from paper_2509_26279_gb300 import tuning
+
+    class F:
+        pass
+
+    f = F()
+    f.cat, spec = _field(16, noise=2000), _grid()
+    f.grid, f.E = sas.Grid(spec), f.cat.n_epochs
+    f.dx, f.dy, f.de = (torch.from_numpy(a).cuda() for a in (f.cat.x, f.cat.y, f.cat.epoch.view(np.int16)))
+    f.w = F()
+    f.w.grid, f.w.n_min = spec, 22
+    e = tuning.TuneCache().tune(f, reps=1)
+    assert e["superbin"] in (1, 2, 3, 4) and e["tile_kx"] == 8

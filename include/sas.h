@@ -144,8 +144,10 @@ typedef struct sas_result_info {
   uint64_t n_emitted;        /* counters that crossed the threshold (a superset: super-bins,
                                 or the windows of a two-level search)               */
   int64_t t0;                /* reference epoch (ticks)                           */
-  uint32_t counter_bits;     /* counter width the stack kernel ran with           */
-  uint32_t tile_kx, tile_ky, tile_bx, tile_by;  /* the one-level plan               */
+  uint32_t counter_bits;     /* counter width the stack kernel ran with (level 1's of a
+                                two-level search)                                   */
+  /* The one-level plan of the field, also where the search ran in two levels: */
+  uint32_t tile_kx, tile_ky, tile_bx, tile_by;  /* lattice points and super-bins per tile */
   uint32_t superbin;         /* bins per counter side                             */
   uint32_t vblock_x, vblock_y;  /* velocity tiles per staged detection set          */
   uint32_t staged_cap;       /* staged detection records per CTA                  */

@@ -637,7 +637,7 @@ int stack_impl(const sas_grid* grid, const sas_catalog* cat, const uint8_t* weig
       res->info.n_pairs = h.pairs;
       res->info.n_emitted = n_emit;
       res->info.t0 = h.t0;
-      res->info.counter_bits = (uint32_t)plan.tc.cb;
+      res->info.counter_bits = (uint32_t)(use_win ? wplan.tc.cb : plan.tc.cb);
       res->info.tile_kx = (uint32_t)plan.tc.kx;
       res->info.tile_ky = (uint32_t)plan.tc.ky;
       res->info.tile_bx = (uint32_t)plan.tc.tx;

@@ -274,3 +274,12 @@ def test_tuning_cache_keeps_tiles_for_batches():
     f.w.grid, f.w.n_min = spec, 22
     e = tuning.TuneCache().tune(f, reps=1)
     assert e["superbin"] in (1, 2, 3, 4) and e["tile_kx"] == 8
+
+
+def test_the_info_names_the_counters_that_ran():
+    """Weights are counted in 16 bits by a two-level search and, at this threshold, in 8 by the one-level plan."""
+    cat, grid = _field(9, movers=60), sas.Grid(_grid())
+    w = np.ones(len(cat.x), np.uint8)
+    bits = [sas.sas_stack_weighted(grid, cat.x, cat.y, cat.epoch, w, cat.t, cat.ticks_per_hour, 16, opts=o).info()["counter_bits"]
+            for o in (None, sas.make_opts(tile_kx=8, tile_ky=4))]
+    assert bits == [16, 8]

@@ -283,3 +283,16 @@ def test_the_info_names_the_counters_that_ran():
     bits = [sas.sas_stack_weighted(grid, cat.x, cat.y, cat.epoch, w, cat.t, cat.ticks_per_hour, 16, opts=o).info()["counter_bits"]
             for o in (None, sas.make_opts(tile_kx=8, tile_ky=4))]
     assert bits == [16, 8]
+
+
+@pytest.mark.parametrize("a,b", [(5, 3000), (333, 5999), (75 * 40 - 7, 75 * 40 + 1400), (2100, 75 * 83), (3, 1203)])
+def test_lattice_ranges_of_a_denser_field(a, b):
+    """Ranges that begin and end inside rows and inside groups, of a field dense enough that each is searched in two levels."""
+    two, one = _check(_field(17, noise=2000), _grid(), 22, v_begin=a, v_end=b)
+    assert two[2] > 0 and two[3]["n_emitted"] != one[3]["n_emitted"]
+
+
+@pytest.mark.parametrize("epochs,n_min", [(11, 8), (128, 30), (150, 128), (255, 60)])
+def test_epoch_counts_are_searched_in_two_levels(epochs, n_min):
+    two, one = _check(_field(4, epochs=epochs, noise=60000 // epochs, movers=30), _grid(), n_min)
+    assert two[3]["n_emitted"] != one[3]["n_emitted"]

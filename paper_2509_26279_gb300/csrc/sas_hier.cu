@@ -632,7 +632,8 @@ bool plan_windows(const sas_grid_desc& d, uint64_t n, uint32_t n_min, double mea
   StackArgs sa{};
   fill_stack_args(fp, n_min, n_min, 0, &sa);
   const double counters = n_v * (double)d.nbx * d.nby / ((double)fp.sb * fp.sb);
-  const double one_level = (double)n * n_v * (fp.cb == 8 ? (sa.merge ? 5e-4 : 8e-4) : 1.4e-3) + counters * (fp.cb / 32.0) * (6.0 / 32.0 / 2.2 / di.sms);
+  const double one_level = (double)n * n_v * (fp.cb == 8 ? (sa.merge ? 5e-4 : 8e-4) : 1.4e-3) +
+                           counters * (fp.cb / 32.0) * (6.0 / 32.0 / 2.2 / di.sms);
   // the window search launches five more kernels: about 40000 cycles
   if (one_level < 60000) return false;
   const double hour = (double)fp.dT / (double)fp.g.tph;

@@ -317,9 +317,9 @@ cudaError_t launch_sort_keys(Key* keys, uint32_t n, uint32_t n_pad, cudaStream_t
 // Sorts every aligned segment of `seg` keys (a power of two) of keys[0..n_total)
 // ascending; n_total is a multiple of seg.
 cudaError_t launch_sort_segments(Key* keys, uint32_t n_total, uint32_t seg, cudaStream_t s);
-// Sorts n keys into `sorted` (which may be `keys` only when sort_in_place(n)); equal
-// keys keep their order.  Without sort_in_place both need room for n keys, or for the
-// next power of two beyond kSortMerge keys.
+// Sorts n keys, no two of them equal, into `sorted` (which may be `keys` only when
+// sort_in_place(n)).  Without sort_in_place both need room for n keys, or for the next
+// power of two beyond kSortMerge keys.
 constexpr uint32_t kSortMerge = 1u << 16;
 bool sort_in_place(uint32_t n);
 cudaError_t launch_sort(Key* keys, uint32_t n, Key* sorted, cudaStream_t s);

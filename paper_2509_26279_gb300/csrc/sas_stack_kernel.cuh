@@ -1001,35 +1001,34 @@ __device__ __forceinline__ void run_unit_windows(const StackArgs& a, uint32_t un
   {
     uint32_t pairs = 0, added = 0;  // pairs, and the weight they added
     auto records = [&](auto weighted) {
-                constexpr bool WT = decltype(weighted)::value;
-                                const uint32_t share = ((total + kNT - 1) / kNT) * 32u;
-                const uint32_t j_lo = (uint32_t)warp * share, j_hi = min(j_lo + share, total);
-                uint32_t lo = 0;
-                for (uint32_t hi = n_seg; hi - lo > 1 && j_lo < j_hi;) {  // segment of the share's first record
-                  const uint32_t mid = (lo + hi) >> 1;
-                  if (s_seg_pos[mid] <= j_lo) lo = mid; else hi = mid;
-                }
-                for (uint32_t j0 = j_lo; j0 < j_hi; j0 += 32) {
-                  const uint32_t j = min(j0 + lane, j_hi - 1);
-                  const uint32_t at = lo + (uint32_t)lane;
-                  const uint32_t start_at = at < n_seg ? s_seg_pos[at] : 0xffffffffu;
-                  const uint32_t src_at = at < n_seg ? s_seg_src[at] : 0u;
-                  uint32_t k = 0;  // the last of the 32 segments that starts at or before j
-      #pragma unroll
-                  for (int step = 16; step > 0; step >>= 1)
-                    if (__shfl_sync(0xffffffffu, start_at, k + step) <= j) k += step;
-                  const uint32_t d_at = __shfl_sync(0xffffffffu, src_at, k) + (j - __shfl_sync(0xffffffffu, start_at, k));
-                  lo += __shfl_sync(0xffffffffu, k, 31);
-                  if (j0 + lane < j_hi) {
-                    const Det d = a.dets[d_at];
-                    const uint32_t w = WT ? a.w[d.id] : 1u;
-                    const uint32_t p = process_rec_windows<KX, KY, CB, WT>(d.x, d.y, s_ox + d.e * oxs ,
-                                                                           s_oy + d.e * oys , cells_s, tw_x, tw_y,
-                                                                           a.magic, tc.tx, txty, w);
-                    pairs += p;
-                    added += WT ? p * w : p;
-                  }
-                }
+      constexpr bool WT = decltype(weighted)::value;
+      const uint32_t share = ((total + kNT - 1) / kNT) * 32u;
+      const uint32_t j_lo = (uint32_t)warp * share, j_hi = min(j_lo + share, total);
+      uint32_t lo = 0;
+      for (uint32_t hi = n_seg; hi - lo > 1 && j_lo < j_hi;) {  // segment of the share's first record
+        const uint32_t mid = (lo + hi) >> 1;
+        if (s_seg_pos[mid] <= j_lo) lo = mid; else hi = mid;
+      }
+      for (uint32_t j0 = j_lo; j0 < j_hi; j0 += 32) {
+        const uint32_t j = min(j0 + lane, j_hi - 1);
+        const uint32_t at = lo + (uint32_t)lane;
+        const uint32_t start_at = at < n_seg ? s_seg_pos[at] : 0xffffffffu;
+        const uint32_t src_at = at < n_seg ? s_seg_src[at] : 0u;
+        uint32_t k = 0;  // the last of the 32 segments that starts at or before j
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1)
+          if (__shfl_sync(0xffffffffu, start_at, k + step) <= j) k += step;
+        const uint32_t d_at = __shfl_sync(0xffffffffu, src_at, k) + (j - __shfl_sync(0xffffffffu, start_at, k));
+        lo += __shfl_sync(0xffffffffu, k, 31);
+        if (j0 + lane < j_hi) {
+          const Det d = a.dets[d_at];
+          const uint32_t w = WT ? a.w[d.id] : 1u;
+          const uint32_t p = process_rec_windows<KX, KY, CB, WT>(d.x, d.y, s_ox + d.e * oxs, s_oy + d.e * oys, cells_s, tw_x,
+                                                                 tw_y, a.magic, tc.tx, txty, w);
+          pairs += p;
+          added += WT ? p * w : p;
+        }
+      }
     };
     if (a.w) records(std::true_type{}); else records(std::false_type{});
     pairs64 += pairs;

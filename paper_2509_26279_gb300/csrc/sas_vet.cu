@@ -1330,7 +1330,8 @@ int sas_vet_create(int device, uint32_t max_batch, sas_vet** out) {
       {(void**)&vt->grad, N * 4}, {(void**)&vt->wb, N * 2},
       {(void**)&vt->a1, B * vet::kCh * vet::kH1 * vet::kH1 * 2}, {(void**)&vt->a2, B * vet::kCh * vet::kH2 * vet::kH2 * 2},
       {(void**)&vt->a3, B * vet::kF * 2}, {(void**)&vt->a4, B * vet::kHid * 2}, {(void**)&vt->logits, B * 4},
-      {(void**)&vt->lpart, (B + vet::kLossStamps - 1) / vet::kLossStamps * vet::kLossOut * 4}, {(void**)&vt->g4, B * vet::kHid * 4}, {(void**)&vt->g3, B * vet::kF * 4},
+      {(void**)&vt->lpart, (B + vet::kLossStamps - 1) / vet::kLossStamps * vet::kLossOut * 4},
+      {(void**)&vt->g4, B * vet::kHid * 4}, {(void**)&vt->g3, B * vet::kF * 4},
       {(void**)&vt->g2, B * vet::kCh * vet::kH2 * vet::kH2 * 4}, {(void**)&vt->g1, B * vet::kCh * vet::kH1 * vet::kH1 * 4},
       {(void**)&vt->partial, (size_t)3 * vet::kBackBlocks * vet::kPartialStride * 4}, {(void**)&vt->loss, 4},
       {(void**)&vt->status, 4},

@@ -14,12 +14,14 @@ N_min = 25.  The metric is detection-shifts per second: in-domain
             host->device copy of the catalog and the device->host copy of the
             candidates and ids (into page-locked arrays allocated once and
             reused) are inside the timed region (wall clock)
-  roofline  detection-shifts per second of the stack kernels against the
-            shared-memory reduction peak measured in this run by the library's
-            probe.  A kernel that counts every detection-shift with a reduction
-            of its own stays below 1; a window search counts once per group of
-            velocities and looks again only at the windows it keeps, so its
-            ratio says how many such kernels' work it replaces and may exceed 1
+  roofline  frac: shared-memory reductions that the stack kernels execute per
+            second (their number from the committed ncu summary, where it was
+            taken on the current source; else null) against the reduction peak
+            measured in this run by the library's probe.  pairs_vs_peak:
+            detection-shifts searched per second over the same peak.  A
+            two-level search counts once per group of velocities, so this says
+            how much one-reduction-per-detection-shift work it replaces, not
+            how busy the resource is, and may exceed 1
 
   fields    fields/s of the plain form (one search per field) against the
             batched + vetted form on 60 uneven fields, with recall per
@@ -145,21 +147,22 @@ def stack_source_sha256() -> str:
     return h.hexdigest()
 
 
-def stack_traffic(workload: str):
-    """DRAM bytes of a search's stack kernels from the committed ncu summary of this
-    workload, if it was taken on the current stack kernel source; else None."""
+def stack_profile(workload: str):
+    """(DRAM bytes, shared-memory reductions) of a search's stack kernels from the committed
+    ncu summary of this workload, if it was taken on the current stack kernel source; else Nones."""
     p = os.path.join(ROOT, "profiles", f"k_stack_{workload}.md")
     if not os.path.exists(p):
-        return None
+        return None, None
     fields = {}
     for line in open(p):
         k, sep, v = line.strip().partition(":")
-        if sep and k in ("stack_source_sha256", "traffic_bytes_per_launch"):
+        if sep and k in ("stack_source_sha256", "traffic_bytes_per_launch", "shared_atomic_instructions_per_search"):
             fields[k] = v.strip()
     h = stack_source_sha256()
-    if fields.get("stack_source_sha256") != h or "traffic_bytes_per_launch" not in fields:
-        return None
-    return int(fields["traffic_bytes_per_launch"])
+    if fields.get("stack_source_sha256") != h:
+        return None, None
+    traffic, atomics = fields.get("traffic_bytes_per_launch"), fields.get("shared_atomic_instructions_per_search")
+    return None if traffic is None else int(traffic), None if atomics is None else 32 * int(atomics)
 
 
 def host_info() -> dict:
@@ -568,8 +571,9 @@ def config_entry(name: str, steps: int, warmup: int, dev, stream, flush, peak_op
                  cpu_budget_s: float) -> dict:
     """One more search workload measured like the main line (device-resident
     inputs, L2 flushed between steps, CUDA events on the library's stream):
-    det-shifts/s of the whole search, the stack kernel's mean time and its
-    fraction of the in-run reduction peak, and the oracle beside it."""
+    det-shifts/s of the whole search, the stack kernels' mean time and the
+    detection-shifts they search against the in-run reduction peak, and the
+    oracle beside it."""
     import torch
     from paper_2509_26279_gb300 import sas
     w = getattr(W, name)()
@@ -605,9 +609,9 @@ def config_entry(name: str, steps: int, warmup: int, dev, stream, flush, peak_op
            "n_pairs_per_step": n_pairs, "candidates": int(info0["n_candidates"]),
            "tile": [info0["tile_kx"], info0["tile_ky"], info0["tile_bx"], info0["tile_by"]],
            "superbin": int(info0["superbin"]), "velocity_block": [info0["vblock_x"], info0["vblock_y"]],
-           "roofline": {"bound": "smem_atomic", "kernel": "k_stack", "stack_ms": statistics.mean(stack_ms),
-                        "achieved": achieved / 1e9, "peak": peak_ops / 1e9, "unit": "Gop/s",
-                        "frac": achieved / peak_ops}}
+           "roofline": {"bound": "smem_atomic", "kernel": "k_stack, k_window_*", "stack_ms": statistics.mean(stack_ms),
+                        "peak": peak_ops / 1e9, "unit": "Gop/s", "pairs": achieved / 1e9,
+                        "pairs_vs_peak": achieved / peak_ops}}
     if cpu_budget_s > 0:
         out["cpu_baseline"] = cpu_baseline(w, cat, cpu_budget_s)
     return out
@@ -898,16 +902,21 @@ def main():
         if dist is not None:
             dist.destroy_process_group()
         return 0
-    achieved = n_pairs / (statistics.mean(stack_ms) * 1e-3)
-    roof = {"bound": "smem_atomic", "achieved": achieved / 1e9, "peak": peak_ops / 1e9,
-            "unit": "Gop/s", "frac": achieved / peak_ops, "traffic": stack_traffic(args.workload),
+    pairs = n_pairs / (statistics.mean(stack_ms) * 1e-3)
+    traffic, reductions = stack_profile(args.workload)
+    achieved = reductions / (statistics.mean(stack_ms) * 1e-3) if reductions else None
+    roof = {"bound": "smem_atomic", "achieved": achieved / 1e9 if achieved else None, "peak": peak_ops / 1e9,
+            "unit": "Gop/s", "frac": achieved / peak_ops if achieved else None, "traffic": traffic,
             "kernel": "k_stack, k_window_*", "stack_ms": statistics.mean(stack_ms),
-            "achieved_is": "detection-shifts searched per second of the stack kernels (one reduction "
-                           "counts a group of velocities in a window search, so frac may exceed 1)",
+            "achieved_is": "shared-memory reductions executed by the stack kernels (32 lanes per warp "
+                           "instruction counted by ncu) per second",
+            "pairs": pairs / 1e9, "pairs_vs_peak": pairs / peak_ops,
+            "pairs_is": "detection-shifts searched per second of the stack kernels; a two-level search counts "
+                        "a group of velocities with one reduction, so pairs_vs_peak may exceed 1",
             "peak_source": f"sas_probe_shared_reduction_peak (conflict-free red.shared.add.u32), this run "
                            f"({probe_mhz:.0f} MHz)",
             "peak_atomic_returning": atom_ops / 1e9,
-            "frac_vs_atomic_returning": achieved / atom_ops,
+            "pairs_vs_atomic_returning": pairs / atom_ops,
             "peak_atomic_returning_source": f"sas_probe_shared_atomic_peak (conflict-free atomicAdd, old value "
                                             f"used), this run ({atom_mhz:.0f} MHz)",
             "atomic_or_b64": or64_ops / 1e9,

@@ -28,7 +28,7 @@ N_min = 25.  The metric is detection-shifts per second: in-domain
             magnitude bin and purity (after training the vetter, untimed)
 
   configs   the other search workloads (tiny, fast_movers) measured the same
-            way, each with its stack kernel's roofline fraction and the oracle
+            way, each with its detection-shifts against the peak and the oracle
 
 --impl reference times the CPU oracle (the plain definition; its OpenMP form
 over velocity chunks on all host cores) on a bounded lattice sample of the same

@@ -251,8 +251,11 @@ constexpr int32_t kOutside = INT32_MIN / 2;  // in no bin, whatever a group's ed
 //
 // LONG: the windows in the queue, with room for kLongList detections each.  A window
 // of more than kList (two steady sources in it over 130 epochs, say) is marked by the
-// first pass and counted here, by one block an SM; fields without such windows do
-// not launch it.
+// first pass and counted here; fields without such windows do not launch it.  Longer
+// lists for all would cost the first pass its occupancy; these leave one block of
+// eight warps an SM (163 KB, weighted 174), and a few windows are bound by one warp's
+// exact counts, bin after bin: 0.3 ms for one pair of sources at 2048 x 4096 px, 130
+// epochs and 12,321 velocities, where the one-level search instead took 5.4 ms more.
 template <bool W, bool LONG>
 __global__ void __launch_bounds__(kWarps * 32, LONG ? 1 : 4) k_window_cells(WindowArgs a, uint64_t cell_m) {
   extern __shared__ __align__(16) unsigned char smem[];

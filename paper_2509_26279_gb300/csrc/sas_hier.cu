@@ -268,7 +268,8 @@ __global__ void __launch_bounds__(kWarps * 32, LONG ? 1 : 4) k_window_cells(Wind
   const uint32_t E = g.E;
   const int P = a.cgm.bin, span = a.win * P, nvg = a.gx * a.gy;
   const uint32_t n_win = LONG ? a.n_queue : *a.n_windows;
-  if (!LONG && (n_win > a.list_cap || *a.balance != 0)) return;  // level 1 runs again: longer list, wider counters
+  const unsigned long long wrapped = LONG ? 0 : *a.balance;  // both loads at once
+  if (!LONG && (n_win > a.list_cap || wrapped)) return;  // level 1 runs again: longer list, wider counters
   unsigned long long raw_sum = 0;
   constexpr int kSeen = W ? 256 : 8;
   for (int i = lane; i < kSeen; i += 32) L.seen[i] = 0;
